@@ -208,16 +208,24 @@ cudaError_t launch_passes(fcas_ctx* c, int64_t n, double* d_fit, int64_t* d_tc, 
     return launch_passes_with(c, c->d_params, c->d_inter, c->d_partials, c->chunk, n, d_fit, d_tc, st);
 }
 
-// Per-particle buffers of the adjoint: band sums and a staging array for host outputs.
+// Buffers of the adjoint: partial band sums of one launch's particles and a staging array for host outputs.
 int ensure_grad(fcas_ctx* c, int64_t n) {
+    const FitnessPlan plan = make_plan(c);
+    const size_t need = sizeof(double) * 12 * (size_t)c->setup.n_det * grad_segments(plan) *
+                        (size_t)std::min(n, grad_chunk(plan));
+    if (need > c->gsums_bytes) {
+        if (c->d_gsums) cudaFree(c->d_gsums);
+        c->d_gsums = nullptr;
+        c->gsums_bytes = 0;
+        const int rc = dev_alloc(&c->d_gsums, need, "gradient sums");
+        if (rc) return rc;
+        c->gsums_bytes = need;
+    }
     if (n <= c->grad_cap) return FCAS_OK;
-    if (c->d_gsums) cudaFree(c->d_gsums);
     if (c->d_gstage) cudaFree(c->d_gstage);
-    c->d_gsums = nullptr;
     c->d_gstage = nullptr;
     c->grad_cap = 0;
-    int rc = dev_alloc(&c->d_gsums, sizeof(double) * 12 * (size_t)c->setup.n_det * n, "gradient sums");
-    if (!rc) rc = dev_alloc(&c->d_gstage, sizeof(double) * 4 * (size_t)n, "gradient staging");
+    const int rc = dev_alloc(&c->d_gstage, sizeof(double) * 4 * (size_t)n, "gradient staging");
     if (rc) return rc;
     c->grad_cap = n;
     return FCAS_OK;
@@ -228,18 +236,11 @@ int ensure_grad(fcas_ctx* c, int64_t n) {
 // ensure_grad for n).
 cudaError_t gradient_device(fcas_ctx* c, int64_t n, const double* d_theta, const int64_t* d_tc, double* d_grad,
                             cudaStream_t st) {
-    cudaError_t e = launch_geometry(d_theta, n, c->d_params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low,
-                                    c->df, pass_a_kstep(c), st);
+    const cudaError_t e = launch_geometry(d_theta, n, c->d_params, c->d_det, c->d_sigma2s, c->setup.n_det,
+                                          c->setup.f_low, c->df, pass_a_kstep(c), st);
     if (e != cudaSuccess) return e;
-    const FitnessPlan plan = make_plan(c);
-    if (c->setup.precision == FCAS_PREC_FP32)
-        e = launch_grad_sums<float>(plan, c->k1b, c->k_lo, c->k_hi, c->d_params, d_tc, n, c->d_gsums, st);
-    else
-        e = launch_grad_sums<double>(plan, c->k1b, c->k_lo, c->k_hi, c->d_params, d_tc, n, c->d_gsums, st,
-                                     c->setup.precision == FCAS_PREC_FF);
-    if (e != cudaSuccess) return e;
-    return launch_grad_final(d_theta, d_tc, n, c->d_gsums, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low,
-                             c->df, d_grad, st);
+    return launch_gradient(make_plan(c), c->setup.precision, c->k_lo, c->k_hi, c->d_params, d_theta, d_tc, n,
+                           c->d_gsums, c->d_det, c->d_sigma2s, c->setup.f_low, c->df, d_grad, st);
 }
 
 // Scratch of the fitness path (allocated at create unless FCAS_SETUP_LAZY_SCRATCH, else on first use).

@@ -71,7 +71,8 @@ struct fcas_ctx {
     int64_t chunk = 0;
     int64_t nb_partials = 0;
     // adjoint
-    double* d_gsums = nullptr;       // [n][D][12] per-detector sums at t*
+    double* d_gsums = nullptr;       // [n][D][segments][12] partial per-detector sums at t*
+    size_t gsums_bytes = 0;
     double* d_gstage = nullptr;      // [n][4] gradient staging for host outputs
     int64_t grad_cap = 0;
     unsigned char* d_polish = nullptr;  // working arrays of fcas_polish

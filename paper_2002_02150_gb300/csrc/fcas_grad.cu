@@ -8,108 +8,214 @@
 //   dZ_i/d(alpha, delta) = 2 pi i (d(Delta^i df)/d(alpha, delta)) sum_k k Q_i e^{...},
 //   dZ_i/d(tau0, tau1.5) = 2 pi i sum_j (dc_j/dtau) sum_k B_j(k) Q_i e^{...}
 // with B_j = phi^-5/3, phi^-1, phi^-2/3, phi^-1/3. A reduction kernel forms the six sums per
-// (particle, detector) in one sweep of the band; a per-particle kernel combines them in binary64.
+// (particle, detector) over segments of the band; a per-particle kernel adds the segments and combines
+// the sums in binary64.
 #include <cmath>
 
+#include "fcas_ff.cuh"
 #include "fcas_kernels.cuh"
 
 namespace fcas {
 
 constexpr int kGradSums = 12;   // Z, F (= sum k Q), S_53, S_1, S_23, S_13: complex, as (re, im) doubles
 
-template <typename Real>
-__global__ void __launch_bounds__(256)
-grad_sums_kernel(const cplx<Real>* __restrict__ y, bool y_ff, const Basis<Real>* __restrict__ basis,
-                 const ParticleParams* __restrict__ params, const int64_t* __restrict__ tc, int n_det, int log_n,
-                 int log_n1, int log_n2, int k1b, int64_t k_lo, int64_t k_hi, double* __restrict__ sums) {
-    __shared__ double red[kGradSums][8];
-    const int64_t p = blockIdx.x;
-    const int i = blockIdx.y;
-    const ParticleParams& pp = params[p];
-    const int64_t t = tc[p];
-    const int64_t n = (int64_t)1 << log_n, n1 = (int64_t)1 << log_n1, half2 = ((int64_t)1 << log_n2) / 2;
-    const int64_t per_blk = half2 * k1b;
-    double acc[kGradSums];
+// One running sum of the adjoint. The FP32 form's terms are FP32 values times float-float weights; their
+// sum is kept as a compensated pair on the FP32 units (Ogita, Rump & Oishi 2005: the rounding error of
+// every product and every addition is formed exactly and added to the second word), as accurate as the
+// binary64 sum of the same terms for the at most 2^10 terms a thread adds, at ~11 FP32 instructions per
+// term where a binary64 one holds the SM's binary64 unit for as long as 64 FP32 instructions would take.
+struct SumF {
+    float h, l;
+};
+__device__ __forceinline__ void sum_zero(SumF& a) { a.h = a.l = 0.0f; }
+__device__ __forceinline__ void sum_zero(double& a) { a = 0.0; }
+__device__ __forceinline__ void sum_add(SumF& a, float q) {
+    float e;
+    a.h = ff_two_sum(a.h, q, e);
+    a.l = __fadd_rn(a.l, e);
+}
+// a += w q for an exact float w
+__device__ __forceinline__ void sum_add_w(SumF& a, float w, float q) {
+    const float p = __fmul_rn(w, q);
+    float e;
+    a.h = ff_two_sum(a.h, p, e);
+    a.l = __fadd_rn(a.l, __fadd_rn(e, __fmaf_rn(w, q, -p)));
+}
+// a += (w.x + w.y) q
+__device__ __forceinline__ void sum_add_w(SumF& a, float2 w, float q) {
+    const float p = __fmul_rn(w.x, q);
+    float e;
+    a.h = ff_two_sum(a.h, p, e);
+    a.l = __fadd_rn(a.l, __fadd_rn(e, __fmaf_rn(w.y, q, __fmaf_rn(w.x, q, -p))));
+}
+__device__ __forceinline__ void sum_add(double& a, double q) { a += q; }
+__device__ __forceinline__ void sum_add_w(double& a, double w, double q) { a += w * q; }
+__device__ __forceinline__ SumF sum_of(SumF a, SumF b) {
+    const ffloat r = ff_add(ffloat(a.h, a.l), ffloat(b.h, b.l));
+    return SumF{r.h, r.l};
+}
+__device__ __forceinline__ double sum_of(double a, double b) { return a + b; }
+// the pair as a float-float number (the second word may have outgrown half an ulp of the first)
+__device__ __forceinline__ void sum_normalise(SumF& a) {
+    float e;
+    a.h = ff_two_sum(a.h, a.l, e);
+    a.l = e;
+}
+__device__ __forceinline__ void sum_normalise(double&) {}
+__device__ __forceinline__ SumF sum_xor(SumF a, int off) {
+    return SumF{__shfl_xor_sync(0xffffffffu, a.h, off), __shfl_xor_sync(0xffffffffu, a.l, off)};
+}
+__device__ __forceinline__ double sum_xor(double a, int off) { return __shfl_xor_sync(0xffffffffu, a, off); }
+__device__ __forceinline__ double sum_value(SumF a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double sum_value(double a) { return a; }
+template <typename Real> struct grad_sum { using type = double; };
+template <> struct grad_sum<float> { using type = SumF; };
+
+constexpr int kGradThreads = 256;
+constexpr int kGradDet = 2;                        // detectors per CTA: they share a bin's chirp phase
+constexpr int kGradVals = kGradDet * kGradSums;    // 24 sums per thread
+
+// Sums of one warp's 24 values: the first three butterfly steps halve the values each lane carries (24 ->
+// 12 -> 6 -> 3), the last two add whole lanes: 27 additions where a reduction value by value takes 120.
+// Afterwards lane l holds in v[0..2] the totals of values 3 (l >> 2) .. + 2 in the order (l & 16) 12 +
+// (l & 8) 6 + (l & 4) 3.
+template <typename Acc>
+__device__ __forceinline__ void warp_sums(Acc (&v)[kGradVals], int lane) {
 #pragma unroll
-    for (int q = 0; q < kGradSums; ++q) acc[q] = 0.0;
-    if (pp.valid && t >= 0) {
-        for (int64_t g = threadIdx.x; g < n / 2; g += blockDim.x) {
-            const int64_t blk = g / per_blk, rem = g % per_blk;
-            const int64_t k = blk * k1b + rem % k1b + n1 * (rem / k1b);
-            if (k < k_lo || k > k_hi) continue;
-            cplx<Real> yv;
-            if constexpr (sizeof(Real) == 8) {
-                if (y_ff) {   // float-float layout (FCAS_PREC_FF contexts): 16-byte entries hi/lo re, hi/lo im
-                    const float4 q = reinterpret_cast<const float4*>(y)[(blk * n_det + i) * per_blk + rem];
-                    yv = make_double2((double)q.x + (double)q.y, (double)q.z + (double)q.w);
-                } else {
-                    yv = y[(blk * n_det + i) * per_blk + rem];
-                }
-            } else {
-                yv = y[(blk * n_det + i) * per_blk + rem];
+    for (int step = 0; step < 3; ++step) {
+        const int off = 16 >> step, half = kGradVals >> (step + 1);
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < kGradVals / 2; ++i) {
+            if (i < half) {
+                const Acc mine = up ? v[i + half] : v[i], send = up ? v[i] : v[i + half];
+                v[i] = sum_of(mine, sum_xor(send, off));
             }
-            const Basis<Real> b = basis[g];
-            const double shift = (double)((k * t) & (n - 1)) / (double)n;   // k t / N mod 1, exact
-            double qr, qi, b53, b1, b23, b13;
-            if constexpr (sizeof(Real) == 4) {
-                const ChirpPowers cpw = chirp_powers(b);
-                float s = frac_mul_ff(pp.ch[0], pp.cl[0], cpw.b53.x, cpw.b53.y);
-                s += frac_mul_ff(pp.ch[1], pp.cl[1], cpw.b1.x, cpw.b1.y);
-                s += frac_mul_ff(pp.ch[2], pp.cl[2], cpw.b23.x, cpw.b23.y);
-                s += frac_mul_ff(pp.ch[3], pp.cl[3], cpw.b13.x, cpw.b13.y);
-                float th = s + frac_mul_ff((float)k, 0.0f, pp.dh[i], pp.dl[i]) + (float)shift;
-                th -= rintf(th);
-                float sn, cs;
-                sincospif(2.0f * th, &sn, &cs);
-                qr = (double)(yv.x * cs - yv.y * sn);
-                qi = (double)(yv.x * sn + yv.y * cs);
-                b53 = (double)cpw.b53.x + (double)cpw.b53.y;
-                b1 = (double)cpw.b1.x + (double)cpw.b1.y;
-                b23 = (double)cpw.b23.x + (double)cpw.b23.y;
-                b13 = (double)cpw.b13.x + (double)cpw.b13.y;
-            } else {
-                double th = pp.c[0] * b.a.x + pp.c[1] * b.a.y + pp.c[2] * b.b.x + pp.c[3] * b.b.y;
-                th -= rint(th);
-                double kd = (double)k * pp.dturn[i];
-                th += kd - rint(kd) + shift;
-                th -= rint(th);
-                double sn, cs;
-                sincospi(2.0 * th, &sn, &cs);
-                qr = yv.x * cs - yv.y * sn;
-                qi = yv.x * sn + yv.y * cs;
-                b53 = b.a.x;
-                b1 = b.a.y;
-                b23 = b.b.x;
-                b13 = b.b.y;
-            }
-            const double kk = (double)k;
-            acc[0] += qr;
-            acc[1] += qi;
-            acc[2] += kk * qr;
-            acc[3] += kk * qi;
-            acc[4] += b53 * qr;
-            acc[5] += b53 * qi;
-            acc[6] += b1 * qr;
-            acc[7] += b1 * qi;
-            acc[8] += b23 * qr;
-            acc[9] += b23 * qi;
-            acc[10] += b13 * qr;
-            acc[11] += b13 * qi;
         }
     }
-    // fixed-order reduction: warp shuffles, then the 8 warp partials in order
 #pragma unroll
-    for (int q = 0; q < kGradSums; ++q) {
-        double v = acc[q];
+    for (int off = 2; off > 0; off >>= 1)
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if ((threadIdx.x & 31) == 0) red[q][threadIdx.x >> 5] = v;
+        for (int i = 0; i < kGradVals / 8; ++i) v[i] = sum_of(v[i], sum_xor(v[i], off));
+}
+
+// Partial band sums of a particle: CTA (particle, detector pair, segment) adds the terms of its segment's
+// column blocks (blks of them) at the rows k2 that hold band bins. The segments do not depend on the
+// number of particles, so neither do the sums' bits. One CTA per (particle, detector) over the whole band
+// left most SMs idle for a few particles and its twelve binary64 sums per bin held the binary64 unit: 8
+// particles of the 60-min workload 42.9 -> 1.36 ms a call, forward and backward of 40 particles on 64 s
+// 799 -> 398 us. Bound now by FP32 issue (about 200 instructions per bin and detector).
+template <typename Real>
+__global__ void __launch_bounds__(kGradThreads, 2)
+grad_sums_kernel(const cplx<Real>* __restrict__ y, bool y_ff, const Basis<Real>* __restrict__ basis,
+                 const ParticleParams* __restrict__ params, const int64_t* __restrict__ tc, int n_det, int log_n,
+                 int log_n1, int log_n2, int log_k1b, int k_lo, int k_hi, int nseg, int blks,
+                 double* __restrict__ part) {
+    using Acc = typename grad_sum<Real>::type;
+    __shared__ Acc red[kGradThreads / 32][kGradVals];
+    const int pairs = (n_det + kGradDet - 1) / kGradDet;
+    const int seg = blockIdx.x % nseg;
+    const int i0 = (blockIdx.x / nseg) % pairs * kGradDet;
+    const int64_t p = blockIdx.x / nseg / pairs;
+    const int nd = n_det - i0 < kGradDet ? n_det - i0 : kGradDet;
+    const ParticleParams& pp = params[p];
+    const int64_t t = tc[p];
+    const int k1b = 1 << log_k1b;
+    const int64_t per_blk = (int64_t)1 << (log_n2 - 1 + log_k1b);
+    const int k2_lo = k_lo >> log_n1, rows = (k_hi >> log_n1) - k2_lo + 1;
+    const unsigned nmask = (1u << log_n) - 1u;
+    Acc acc[kGradVals];
+#pragma unroll
+    for (int q = 0; q < kGradVals; ++q) sum_zero(acc[q]);
+    if (pp.valid && t >= 0) {
+        const unsigned tu = (unsigned)t;
+        for (int blk = seg * blks; blk < (seg + 1) * blks; ++blk) {
+            const Basis<Real>* bb = basis + blk * per_blk;
+            const cplx<Real>* yb = y + ((int64_t)blk * n_det + i0) * per_blk;
+            for (int r = threadIdx.x; r < rows << log_k1b; r += kGradThreads) {
+                const int e = r + (k2_lo << log_k1b);
+                const int k = blk * k1b + (e & (k1b - 1)) + ((e >> log_k1b) << log_n1);
+                if (k < k_lo || k > k_hi) continue;
+                const Basis<Real> b = bb[e];
+                const unsigned m = ((unsigned)k * tu) & nmask;   // k t mod N (the low bits of the product)
+                if constexpr (sizeof(Real) == 4) {
+                    const float shift = (float)m * __int_as_float((127 - log_n) << 23);   // m / N, exact
+                    const ChirpPowers cpw = chirp_powers(b);
+                    float s = frac_mul_ff(pp.ch[0], pp.cl[0], cpw.b53.x, cpw.b53.y);
+                    s += frac_mul_ff(pp.ch[1], pp.cl[1], cpw.b1.x, cpw.b1.y);
+                    s += frac_mul_ff(pp.ch[2], pp.cl[2], cpw.b23.x, cpw.b23.y);
+                    s += frac_mul_ff(pp.ch[3], pp.cl[3], cpw.b13.x, cpw.b13.y);
+                    const float kk = (float)k;   // < 2^24: exact
+#pragma unroll
+                    for (int u = 0; u < kGradDet; ++u) {
+                        if (u >= nd) break;
+                        const float2 yv = yb[u * per_blk + e];
+                        float th = s + frac_mul_ff(kk, 0.0f, pp.dh[i0 + u], pp.dl[i0 + u]) + shift;
+                        th -= rintf(th);
+                        float sn, cs;
+                        sincospif(2.0f * th, &sn, &cs);
+                        const float qv[2] = {yv.x * cs - yv.y * sn, yv.x * sn + yv.y * cs};
+#pragma unroll
+                        for (int x = 0; x < 2; ++x) {
+                            sum_add(acc[u * kGradSums + x], qv[x]);
+                            sum_add_w(acc[u * kGradSums + 2 + x], kk, qv[x]);
+                            sum_add_w(acc[u * kGradSums + 4 + x], cpw.b53, qv[x]);
+                            sum_add_w(acc[u * kGradSums + 6 + x], cpw.b1, qv[x]);
+                            sum_add_w(acc[u * kGradSums + 8 + x], cpw.b23, qv[x]);
+                            sum_add_w(acc[u * kGradSums + 10 + x], cpw.b13, qv[x]);
+                        }
+                    }
+                } else {
+                    const double shift = (double)m * __hiloint2double((1023 - log_n) << 20, 0);   // m / N, exact
+                    const double s = pp.c[0] * b.a.x + pp.c[1] * b.a.y + pp.c[2] * b.b.x + pp.c[3] * b.b.y;
+                    const double kk = (double)k;
+#pragma unroll
+                    for (int u = 0; u < kGradDet; ++u) {
+                        if (u >= nd) break;
+                        double2 yv;
+                        if (y_ff) {   // float-float layout (FCAS_PREC_FF contexts): hi/lo re, hi/lo im
+                            const float4 q = reinterpret_cast<const float4*>(yb)[u * per_blk + e];
+                            yv = make_double2((double)q.x + (double)q.y, (double)q.z + (double)q.w);
+                        } else {
+                            yv = yb[u * per_blk + e];
+                        }
+                        double th = s - rint(s);
+                        const double kd = kk * pp.dturn[i0 + u];
+                        th += kd - rint(kd) + shift;
+                        th -= rint(th);
+                        double sn, cs;
+                        sincospi(2.0 * th, &sn, &cs);
+                        const double qv[2] = {yv.x * cs - yv.y * sn, yv.x * sn + yv.y * cs};
+#pragma unroll
+                        for (int x = 0; x < 2; ++x) {
+                            sum_add(acc[u * kGradSums + x], qv[x]);
+                            sum_add_w(acc[u * kGradSums + 2 + x], kk, qv[x]);
+                            sum_add_w(acc[u * kGradSums + 4 + x], b.a.x, qv[x]);
+                            sum_add_w(acc[u * kGradSums + 6 + x], b.a.y, qv[x]);
+                            sum_add_w(acc[u * kGradSums + 8 + x], b.b.x, qv[x]);
+                            sum_add_w(acc[u * kGradSums + 10 + x], b.b.y, qv[x]);
+                        }
+                    }
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kGradVals; ++q) sum_normalise(acc[q]);
+    const int lane = threadIdx.x & 31;
+    warp_sums(acc, lane);
+    if ((lane & 3) == 0) {
+        const int v0 = (lane & 16 ? 12 : 0) + (lane & 8 ? 6 : 0) + (lane & 4 ? 3 : 0);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) red[threadIdx.x >> 5][v0 + i] = acc[i];
     }
     __syncthreads();
-    if (threadIdx.x < kGradSums) {
-        double v = 0.0;
-        for (int w = 0; w < 8; ++w) v += red[threadIdx.x][w];
-        sums[(p * n_det + i) * kGradSums + threadIdx.x] = v;
+    if (threadIdx.x < nd * kGradSums) {
+        Acc v = red[0][threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < kGradThreads / 32; ++w) v = sum_of(v, red[w][threadIdx.x]);
+        const int u = threadIdx.x / kGradSums, q = threadIdx.x % kGradSums;
+        part[((p * n_det + i0 + u) * nseg + seg) * kGradSums + q] = sum_value(v);
     }
 }
 
@@ -144,59 +250,95 @@ __device__ void chirp_coeffs_dual(double tau0, double tau15, double dt0, double 
     c[3] = (3.0 * f_star) * tau2;
 }
 
-__global__ void grad_final_kernel(const double* __restrict__ theta, const int64_t* __restrict__ tc, int64_t n,
-                                  const double* __restrict__ sums, const double* __restrict__ det9,
-                                  const double* __restrict__ s2, int n_det, double f_star, double df,
-                                  double* __restrict__ grad) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
+// One CTA per particle: the segments' partial sums are added in order by all threads, the sky geometry
+// (one lane per detector) and the chirp coefficients (one lane per chirp time) by two different warps,
+// and four lanes combine them, one per component (one thread per particle did all of it serially in
+// binary64, whose every dependent instruction waits tens of cycles).
+constexpr int kFinalThreads = 128;
+__global__ void __launch_bounds__(kFinalThreads)
+grad_final_kernel(const double* __restrict__ theta, const int64_t* __restrict__ tc, const double* __restrict__ part,
+                  int nseg, const double* __restrict__ det9, const double* __restrict__ s2, int n_det, double f_star,
+                  double df, double* __restrict__ grad) {
+    __shared__ double sp[FCAS_MAX_DET * kGradSums];   // Z_i, F_i, S_ij
+    __shared__ double spart[kFinalThreads];
+    __shared__ double u[FCAS_MAX_DET][3][2];          // U^i and its alpha / delta derivatives
+    __shared__ double dd[FCAS_MAX_DET][3];            // delay in turns per bin and its derivatives
+    __shared__ double dc[2][4];                       // d c_j / d tau0, d c_j / d tau1.5
+    const int64_t p = blockIdx.x;
+    const int tid = threadIdx.x;
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     const double alpha = theta[4 * p], delta = theta[4 * p + 1], tau0 = theta[4 * p + 2], tau15 = theta[4 * p + 3];
-    for (int m = 0; m < 4; ++m) grad[4 * p + m] = nan;
-    if (!(isfinite(alpha) && isfinite(delta) && tau0 > 0.0 && tau15 > 0.0 && tc[p] >= 0)) return;
-    const double two_pi = 6.283185307179586476925286766559;
-    double sa, ca, sd, cd;
-    sincos(alpha, &sa, &ca);
-    sincos(delta, &sd, &cd);
-    // basis vectors and their derivatives: [0] value, [1] d/d alpha, [2] d/d delta
-    const double nv[3][3] = {{cd * ca, cd * sa, sd}, {-cd * sa, cd * ca, 0.0}, {-sd * ca, -sd * sa, cd}};
-    const double bx[3][3] = {{sa, -ca, 0.0}, {ca, sa, 0.0}, {0.0, 0.0, 0.0}};
-    const double by[3][3] = {{-sd * ca, -sd * sa, cd}, {sd * sa, -sd * ca, 0.0}, {-cd * ca, -cd * sa, -sd}};
-    double u[FCAS_MAX_DET][3][2];    // U^i and its alpha / delta derivatives
-    double dd[FCAS_MAX_DET][3];      // delay in turns per bin and its derivatives
-    double G[3][3] = {};             // G entries (11, 12, 22) and derivatives
-    for (int i = 0; i < n_det; ++i) {
-        const double* dv = det9 + 9 * i;
-        auto dot = [](const double* a, const double* b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; };
-        const double xX = dot(dv + 3, bx[0]), xY = dot(dv + 3, by[0]), yX = dot(dv + 6, bx[0]), yY = dot(dv + 6, by[0]);
-        u[i][0][0] = 0.5 * (xX * xX - xY * xY - yX * yX + yY * yY);
-        u[i][0][1] = xX * xY - yX * yY;
-        for (int m = 1; m < 3; ++m) {
-            const double dxX = dot(dv + 3, bx[m]), dxY = dot(dv + 3, by[m]), dyX = dot(dv + 6, bx[m]),
-                         dyY = dot(dv + 6, by[m]);
-            u[i][m][0] = xX * dxX - xY * dxY - yX * dyX + yY * dyY;
-            u[i][m][1] = dxX * xY + xX * dxY - dyX * yY - yX * dyY;
-        }
-        for (int m = 0; m < 3; ++m) dd[i][m] = -dot(dv, nv[m]) / kCLight * df;
-        for (int m = 0; m < 3; ++m) {
-            // m = 0: G itself; m = 1, 2: dG = sum s2 (dU U^T + U dU^T)
-            if (m == 0) {
-                G[0][0] += s2[i] * u[i][0][0] * u[i][0][0];
-                G[0][1] += s2[i] * u[i][0][0] * u[i][0][1];
-                G[0][2] += s2[i] * u[i][0][1] * u[i][0][1];
-            } else {
-                G[m][0] += s2[i] * 2.0 * u[i][m][0] * u[i][0][0];
-                G[m][1] += s2[i] * (u[i][m][0] * u[i][0][1] + u[i][0][0] * u[i][m][1]);
-                G[m][2] += s2[i] * 2.0 * u[i][m][1] * u[i][0][1];
+    if (!(isfinite(alpha) && isfinite(delta) && tau0 > 0.0 && tau15 > 0.0 && tc[p] >= 0)) {
+        if (tid < 4) grad[4 * p + tid] = nan;
+        return;
+    }
+    // value v of the detectors' 12 n_det sums: groups of threads add every groups-th segment, then the
+    // groups' totals in order
+    const int vals = n_det * kGradSums, groups = kFinalThreads / vals;
+    const int v = tid % vals, gr = tid / vals;
+    double acc = 0.0;
+    if (gr < groups)
+        for (int seg = gr; seg < nseg; seg += groups)
+            acc += part[((p * n_det + v / kGradSums) * nseg + seg) * kGradSums + v % kGradSums];
+    spart[tid] = acc;
+    if (tid >= 32 && tid < 34) {
+        Dual c[4];
+        chirp_coeffs_dual(tau0, tau15, tid == 32 ? 1.0 : 0.0, tid == 33 ? 1.0 : 0.0, f_star, c);
+        for (int j = 0; j < 4; ++j) dc[tid - 32][j] = c[j].d;
+    }
+    if (tid < 32) {
+        // lane 0 takes sin and cos of alpha, lane 1 of delta
+        double sn, cs;
+        sincos(tid & 1 ? delta : alpha, &sn, &cs);
+        const double sa = __shfl_sync(0xffffffffu, sn, 0), ca = __shfl_sync(0xffffffffu, cs, 0);
+        const double sd = __shfl_sync(0xffffffffu, sn, 1), cd = __shfl_sync(0xffffffffu, cs, 1);
+        if (tid < n_det) {
+            // basis vectors and their derivatives: [0] value, [1] d/d alpha, [2] d/d delta
+            const double nv[3][3] = {{cd * ca, cd * sa, sd}, {-cd * sa, cd * ca, 0.0}, {-sd * ca, -sd * sa, cd}};
+            const double bx[3][3] = {{sa, -ca, 0.0}, {ca, sa, 0.0}, {0.0, 0.0, 0.0}};
+            const double by[3][3] = {{-sd * ca, -sd * sa, cd}, {sd * sa, -sd * ca, 0.0}, {-cd * ca, -cd * sa, -sd}};
+            const double* dv = det9 + 9 * tid;
+            auto dot = [](const double* a, const double* b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; };
+            const double xX = dot(dv + 3, bx[0]), xY = dot(dv + 3, by[0]), yX = dot(dv + 6, bx[0]),
+                         yY = dot(dv + 6, by[0]);
+            u[tid][0][0] = 0.5 * (xX * xX - xY * xY - yX * yX + yY * yY);
+            u[tid][0][1] = xX * xY - yX * yY;
+            for (int m = 1; m < 3; ++m) {
+                const double dxX = dot(dv + 3, bx[m]), dxY = dot(dv + 3, by[m]), dyX = dot(dv + 6, bx[m]),
+                             dyY = dot(dv + 6, by[m]);
+                u[tid][m][0] = xX * dxX - xY * dxY - yX * dyX + yY * dyY;
+                u[tid][m][1] = dxX * xY + xX * dxY - dyX * yY - yX * dyY;
             }
+            for (int m = 0; m < 3; ++m) dd[tid][m] = -dot(dv, nv[m]) / kCLight * df;
         }
     }
-    const double det = G[0][0] * G[0][2] - G[0][1] * G[0][1];
-    const double tr = G[0][0] + G[0][2];
-    if (det < kRank1Rtol * (0.5 * tr) * (0.5 * tr)) return;   // rank-1 branch: no gradient (NaN)
-    const double gi[3] = {G[0][2] / det, -G[0][1] / det, G[0][0] / det};
-    // Z_i, F_i, S_ij
-    const double* sp = sums + p * n_det * 12;
+    __syncthreads();
+    if (tid < vals) {
+        double total = spart[tid];
+        for (int g = 1; g < groups; ++g) total += spart[g * vals + tid];
+        sp[tid] = total;
+    }
+    __syncthreads();
+    if (tid >= 4) return;
+    const int m = tid;   // the component
+    const double two_pi = 6.283185307179586476925286766559;
+    double G[3] = {}, dG[3] = {};   // G entries (11, 12, 22) and their derivative for m = 0, 1
+    const int md = m < 2 ? m + 1 : 0;
+    for (int i = 0; i < n_det; ++i) {
+        G[0] += s2[i] * u[i][0][0] * u[i][0][0];
+        G[1] += s2[i] * u[i][0][0] * u[i][0][1];
+        G[2] += s2[i] * u[i][0][1] * u[i][0][1];
+        dG[0] += s2[i] * 2.0 * u[i][md][0] * u[i][0][0];
+        dG[1] += s2[i] * (u[i][md][0] * u[i][0][1] + u[i][0][0] * u[i][md][1]);
+        dG[2] += s2[i] * 2.0 * u[i][md][1] * u[i][0][1];
+    }
+    const double det = G[0] * G[2] - G[1] * G[1];
+    const double tr = G[0] + G[2];
+    if (det < kRank1Rtol * (0.5 * tr) * (0.5 * tr)) {   // rank-1 branch: no gradient (NaN)
+        grad[4 * p + m] = nan;
+        return;
+    }
+    const double gi[3] = {G[2] / det, -G[1] / det, G[0] / det};
     double Wr[2] = {0, 0}, Wi[2] = {0, 0};
     for (int i = 0; i < n_det; ++i)
         for (int a = 0; a < 2; ++a) {
@@ -209,61 +351,77 @@ __global__ void grad_final_kernel(const double* __restrict__ theta, const int64_
         const double i0 = g[0] * bi[0] + g[1] * bi[1], i1 = g[1] * bi[0] + g[2] * bi[1];
         return ar[0] * r0 + ar[1] * r1 + ai[0] * i0 + ai[1] * i1;
     };
-    Dual c0[4], c1[4];
-    chirp_coeffs_dual(tau0, tau15, 1.0, 0.0, f_star, c0);
-    chirp_coeffs_dual(tau0, tau15, 0.0, 1.0, f_star, c1);
-    for (int m = 0; m < 4; ++m) {
-        double dWr[2] = {0, 0}, dWi[2] = {0, 0};
-        for (int i = 0; i < n_det; ++i) {
-            const double* s = sp + 12 * i;
-            // dZ_i = 2 pi i * X_i, X_i = (dd_i) F_i or sum_j dc_j S_ij
-            double xr, xi;
-            if (m < 2) {
-                xr = dd[i][m + 1] * s[2];
-                xi = dd[i][m + 1] * s[3];
-            } else {
-                const Dual* c = m == 2 ? c0 : c1;
-                xr = c[0].d * s[4] + c[1].d * s[6] + c[2].d * s[8] + c[3].d * s[10];
-                xi = c[0].d * s[5] + c[1].d * s[7] + c[2].d * s[9] + c[3].d * s[11];
-            }
-            const double dzr = -two_pi * xi, dzi = two_pi * xr;
-            for (int a = 0; a < 2; ++a) {
-                dWr[a] += u[i][0][a] * dzr;
-                dWi[a] += u[i][0][a] * dzi;
-                if (m < 2) {
-                    dWr[a] += u[i][m + 1][a] * s[0];
-                    dWi[a] += u[i][m + 1][a] * s[1];
-                }
-            }
-        }
-        double gsum = 2.0 * quad_re(dWr, dWi, Wr, Wi, gi);
+    double dWr[2] = {0, 0}, dWi[2] = {0, 0};
+    for (int i = 0; i < n_det; ++i) {
+        const double* s = sp + 12 * i;
+        // dZ_i = 2 pi i * X_i, X_i = (dd_i) F_i or sum_j dc_j S_ij
+        double xr, xi;
         if (m < 2) {
-            // - W^H Ginv dG Ginv W: Ginv W first, then the dG quadratic form
-            const double ar[2] = {gi[0] * Wr[0] + gi[1] * Wr[1], gi[1] * Wr[0] + gi[2] * Wr[1]};
-            const double ai[2] = {gi[0] * Wi[0] + gi[1] * Wi[1], gi[1] * Wi[0] + gi[2] * Wi[1]};
-            gsum -= quad_re(ar, ai, ar, ai, G[m + 1]);
+            xr = dd[i][m + 1] * s[2];
+            xi = dd[i][m + 1] * s[3];
+        } else {
+            const double* c = dc[m - 2];
+            xr = c[0] * s[4] + c[1] * s[6] + c[2] * s[8] + c[3] * s[10];
+            xi = c[0] * s[5] + c[1] * s[7] + c[2] * s[9] + c[3] * s[11];
         }
-        grad[4 * p + m] = gsum;
+        const double dzr = -two_pi * xi, dzi = two_pi * xr;
+        for (int a = 0; a < 2; ++a) {
+            dWr[a] += u[i][0][a] * dzr;
+            dWi[a] += u[i][0][a] * dzi;
+            if (m < 2) {
+                dWr[a] += u[i][m + 1][a] * s[0];
+                dWi[a] += u[i][m + 1][a] * s[1];
+            }
+        }
     }
+    double gsum = 2.0 * quad_re(dWr, dWi, Wr, Wi, gi);
+    if (m < 2) {
+        // - W^H Ginv dG Ginv W: Ginv W first, then the dG quadratic form
+        const double ar[2] = {gi[0] * Wr[0] + gi[1] * Wr[1], gi[1] * Wr[0] + gi[2] * Wr[1]};
+        const double ai[2] = {gi[0] * Wi[0] + gi[1] * Wi[1], gi[1] * Wi[0] + gi[2] * Wi[1]};
+        gsum -= quad_re(ar, ai, ar, ai, dG);
+    }
+    grad[4 * p + m] = gsum;
 }
 
-template <typename Real>
-cudaError_t launch_grad_sums(const FitnessPlan& pl, int k1b, int64_t k_lo, int64_t k_hi, const ParticleParams* params,
-                             const int64_t* tc, int64_t n, double* sums, cudaStream_t s, bool y_ff) {
-    if (n <= 0) return cudaSuccess;
-    dim3 grid((unsigned)n, (unsigned)pl.n_det);
-    grad_sums_kernel<Real><<<grid, 256, 0, s>>>(static_cast<const cplx<Real>*>(pl.y), y_ff,
-                                                static_cast<const Basis<Real>*>(pl.basis), params, tc, pl.n_det,
-                                                pl.log_n, pl.log_n1, pl.log_n2, k1b, k_lo, k_hi, sums);
-    return cudaGetLastError();
+// Segments of the band sums: ~2048 bins per CTA, at most 256 segments and one column block per segment
+// (a power of two, as the number of column blocks is).
+int grad_segments(const FitnessPlan& pl) {
+    const int nblk = (1 << pl.log_n1) / pl.k1b;
+    return imax_c(1, imin_c(imin_c(nblk, 256), pl.log_n > 12 ? 1 << (pl.log_n - 12) : 1));
 }
 
-cudaError_t launch_grad_final(const double* theta, const int64_t* tc, int64_t n, const double* sums,
-                              const double* det9, const double* s2, int n_det, double f_star, double df, double* grad,
-                              cudaStream_t s) {
-    if (n <= 0) return cudaSuccess;
-    grad_final_kernel<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(theta, tc, n, sums, det9, s2, n_det, f_star, df, grad);
-    return cudaGetLastError();
+int64_t grad_chunk(const FitnessPlan& pl) { return imax_c(1, 32768 / grad_segments(pl)); }
+
+cudaError_t launch_gradient(const FitnessPlan& pl, int precision, int64_t k_lo, int64_t k_hi,
+                            const ParticleParams* params, const double* theta, const int64_t* tc, int64_t n,
+                            double* part, const double* det9, const double* s2, double f_star, double df, double* grad,
+                            cudaStream_t s) {
+    const int nseg = grad_segments(pl), pairs = (pl.n_det + kGradDet - 1) / kGradDet;
+    const int blks = (1 << pl.log_n1) / pl.k1b / nseg;
+    int log_k1b = 0;
+    while ((1 << log_k1b) < pl.k1b) ++log_k1b;
+    const int64_t chunk = grad_chunk(pl);   // bounds the partial sums (12.6 MB with four detectors)
+    for (int64_t p0 = 0; p0 < n; p0 += chunk) {
+        const int64_t np = n - p0 < chunk ? n - p0 : chunk;
+        const unsigned ctas = (unsigned)(np * pairs * nseg);
+        if (precision == FCAS_PREC_FP32)
+            grad_sums_kernel<float><<<ctas, kGradThreads, 0, s>>>(
+                static_cast<const float2*>(pl.y), false, static_cast<const BasisF*>(pl.basis), params + p0, tc + p0,
+                pl.n_det, pl.log_n, pl.log_n1, pl.log_n2, log_k1b, (int)k_lo, (int)k_hi, nseg, blks, part);
+        else
+            grad_sums_kernel<double><<<ctas, kGradThreads, 0, s>>>(
+                static_cast<const double2*>(pl.y), precision == FCAS_PREC_FF, static_cast<const BasisD*>(pl.basis),
+                params + p0, tc + p0, pl.n_det, pl.log_n, pl.log_n1, pl.log_n2, log_k1b, (int)k_lo, (int)k_hi, nseg,
+                blks, part);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        grad_final_kernel<<<(unsigned)np, kFinalThreads, 0, s>>>(theta + 4 * p0, tc + p0, part, nseg, det9, s2,
+                                                                 pl.n_det, f_star, df, grad + 4 * p0);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -349,10 +507,5 @@ cudaError_t launch_polish_accept(double* theta, double* fit, int64_t* tc, const 
                                                                      accepted, n, searching);
     return cudaGetLastError();
 }
-
-template cudaError_t launch_grad_sums<float>(const FitnessPlan&, int, int64_t, int64_t, const ParticleParams*,
-                                             const int64_t*, int64_t, double*, cudaStream_t, bool);
-template cudaError_t launch_grad_sums<double>(const FitnessPlan&, int, int64_t, int64_t, const ParticleParams*,
-                                              const int64_t*, int64_t, double*, cudaStream_t, bool);
 
 }  // namespace fcas

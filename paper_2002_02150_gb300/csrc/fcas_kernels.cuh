@@ -142,12 +142,14 @@ bool pass_a_radix8_available(int log_n2, int precision, int k1b);
 int pass_a_default_radix_bits(int log_n2, int precision);
 
 // ---- adjoint (fcas_grad.cu) ----
-template <typename Real>
-cudaError_t launch_grad_sums(const FitnessPlan& pl, int k1b, int64_t k_lo, int64_t k_hi, const ParticleParams* params,
-                             const int64_t* tc, int64_t n, double* sums, cudaStream_t s, bool y_ff = false);
-cudaError_t launch_grad_final(const double* theta, const int64_t* tc, int64_t n, const double* sums,
-                              const double* det9, const double* s2, int n_det, double f_star, double df, double* grad,
-                              cudaStream_t s);
+// d Gamma^2 / d theta at the lags tc of n particles whose parameters (geometry) are in params. part: scratch
+// of grad_chunk() particles, grad_segments() x n_det x 12 binary64 partial sums each.
+int grad_segments(const FitnessPlan& plan);
+int64_t grad_chunk(const FitnessPlan& plan);
+cudaError_t launch_gradient(const FitnessPlan& plan, int precision, int64_t k_lo, int64_t k_hi,
+                            const ParticleParams* params, const double* theta, const int64_t* tc, int64_t n,
+                            double* part, const double* det9, const double* s2, double f_star, double df, double* grad,
+                            cudaStream_t s);
 
 // ---- gradient polishing (fcas_grad.cu) ----
 struct PolishScales {
