@@ -1,6 +1,8 @@
 // Fitness path, per-particle and host-side parts: geometry, the final argmax, the shape helpers
 // of the two passes, the per-stage twiddle tables, and the FP32 / binary64 instantiations of the
 // passes (fcas_passes.cuh).
+#include <cmath>
+
 #include "fcas_passes.cuh"
 
 namespace fcas {
@@ -9,135 +11,184 @@ namespace fcas {
 // Geometry: Sec. II eq. detresponse (U = F(alpha, delta, 0), Delta^i), Sec. II.C/II.D
 // (G = sum_i sigma_i^2 U^i U^i^T) and Sec. II.B (chirp times -> phase coefficients).
 // ------------------------------------------------------------------------------------------
-__global__ void geometry_kernel(const double* __restrict__ theta, int64_t n, ParticleParams* __restrict__ out,
-                                const double* __restrict__ det9, const double* __restrict__ s2, int n_det,
-                                double f_star, double df, int64_t kstep) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const double alpha = theta[4 * p + 0], delta = theta[4 * p + 1];
-    const double tau0 = theta[4 * p + 2], tau15 = theta[4 * p + 3];
-    ParticleParams pp;
-    for (int q = 0; q < 4; ++q) pp.c[q] = 0.0;
-    for (int i = 0; i < FCAS_MAX_DET; ++i) pp.dturn[i] = pp.u[i][0] = pp.u[i][1] = pp.w1[i] = pp.w2[i] = 0.0;
-    pp.ginv[0] = pp.ginv[1] = pp.ginv[2] = 0.0;
-    pp.chol[0] = pp.chol[1] = pp.chol[2] = 0.0;
-    pp.valid = 0;
-    pp.taylor_ok = 0;
+// Two warps per four particles, eight lanes of each per particle. The first warp takes the sky (one lane per
+// detector), the second the chirp coefficients, so that their binary64 chains run beside each other: the
+// kernel is bound by the latency of dependent binary64 instructions (a few particles) or by their number
+// per SM (a large batch), and one thread per particle issued every detector's share serially (one
+// particle on 64 s, host arrays: 89.5 -> 65.1 us a call; 40 particles 85.9 -> 62.6; the same results).
+struct TaylorBound {
+    double m[2][4];   // cm^3/6 |psi'''| <= sum_j |c_j| m[bit][j]; infinite where no anchor is allowed
+};
+
+// Remainder of psi(k + c) = psi(k) + c psi' + c^2 psi''/2 for c <= C (FP32 pass A, C + 1 adjacent columns
+// per lane group, C = 3 or 7): at most C^3/6 max |psi'''| over the band, taken at k_b = f_*/df - 2 (C + 1)
+// (the band's lowest bin, less the C by which an anchor bin may lie below it, with margin), where
+// |psi'''| <= sum_m |c_m| e_m (e_m + 1) (e_m + 2) phi^-e_m / k^3.
+static TaylorBound taylor_bound(double f_star, double df) {
+    TaylorBound t;
+    for (int bit = 0; bit < 2; ++bit) {
+        const double cm = bit == 0 ? 3.0 : 7.0;
+        const double kb = f_star / df - 2.0 * (cm + 1.0);
+        if (kb < 1.0) {
+            for (double& v : t.m[bit]) v = HUGE_VAL;
+            continue;
+        }
+        const double r = f_star / (kb * df);   // phi^-1 at k_b
+        const double r13 = std::cbrt(r);
+        const double w = cm * cm * cm / 6.0 / (kb * kb * kb);
+        t.m[bit][0] = w * (440.0 / 27.0) * r * r13 * r13;
+        t.m[bit][1] = w * 6.0 * r;
+        t.m[bit][2] = w * (80.0 / 27.0) * r13 * r13;
+        t.m[bit][3] = w * (28.0 / 27.0) * r13;
+    }
+    return t;
+}
+
+constexpr int kGeomLanes = FCAS_MAX_DET;            // lanes per particle
+constexpr int kGeomParticles = 32 / kGeomLanes;     // particles per warp
+
+__global__ void __launch_bounds__(64)
+geometry_kernel(const double* __restrict__ theta, int64_t n, ParticleParams* __restrict__ out,
+                const double* __restrict__ det9, const double* __restrict__ s2, int n_det, double f_star, double df,
+                int64_t kstep, TaylorBound tb) {
+    const int lane = threadIdx.x & 31, sub = lane % kGeomLanes, lane0 = lane - sub;
+    const int64_t p = (int64_t)blockIdx.x * kGeomParticles + lane / kGeomLanes;
+    const bool have = p < n;
+    const int64_t pc = have ? p : n - 1;   // lanes beyond the batch repeat its last particle, unwritten
+    const double alpha = theta[4 * pc + 0], delta = theta[4 * pc + 1];
+    const double tau0 = theta[4 * pc + 2], tau15 = theta[4 * pc + 3];
     const bool ok = isfinite(alpha) && isfinite(delta) && isfinite(tau0) && isfinite(tau15) && tau0 > 0.0 &&
                     tau15 > 0.0;
-    if (ok) {
-        double sa, ca, sd, cd;
-        sincos(alpha, &sa, &ca);
-        sincos(delta, &sd, &cd);
-        const double nx = cd * ca, ny = cd * sa, nz = sd;
-        const double bx[3] = {sa, -ca, 0.0};             // -alpha_hat
-        const double by[3] = {-sd * ca, -sd * sa, cd};   // delta_hat
-        double g11 = 0.0, g12 = 0.0, g22 = 0.0;
-        for (int i = 0; i < n_det; ++i) {
-            const double* d = det9 + 9 * i;
-            pp.dturn[i] = -(d[0] * nx + d[1] * ny + d[2] * nz) / kCLight * df;
-            const double xX = d[3] * bx[0] + d[4] * bx[1] + d[5] * bx[2];
-            const double xY = d[3] * by[0] + d[4] * by[1] + d[5] * by[2];
-            const double yX = d[6] * bx[0] + d[7] * bx[1] + d[8] * bx[2];
-            const double yY = d[6] * by[0] + d[7] * by[1] + d[8] * by[2];
-            const double fp = 0.5 * (xX * xX - xY * xY - yX * yX + yY * yY);
-            const double fx = xX * xY - yX * yY;
-            pp.u[i][0] = fp;
-            pp.u[i][1] = fx;
-            g11 += s2[i] * fp * fp;
-            g12 += s2[i] * fp * fx;
-            g22 += s2[i] * fx * fx;
-        }
-        const double det = g11 * g22 - g12 * g12;
-        const double tr = g11 + g22;
-        if (det < kRank1Rtol * (0.5 * tr) * (0.5 * tr)) {
-            const double lam = 0.5 * tr + sqrt(0.25 * (g11 - g22) * (g11 - g22) + g12 * g12);
-            double e1 = lam - g22, e2 = g12;
-            double f1 = g12, f2 = lam - g11;
-            if (f1 * f1 + f2 * f2 > e1 * e1 + e2 * e2) { e1 = f1; e2 = f2; }
-            const double nrm = e1 * e1 + e2 * e2;
-            if (lam > 0.0 && nrm > 0.0) {
-                pp.ginv[0] = e1 * e1 / nrm / lam;
-                pp.ginv[1] = e1 * e2 / nrm / lam;
-                pp.ginv[2] = e2 * e2 / nrm / lam;
-            }
-        } else {
-            pp.ginv[0] = g22 / det;
-            pp.ginv[1] = -g12 / det;
-            pp.ginv[2] = g11 / det;
-        }
-        // Cholesky factor of G^-1 so that Gamma^2 = |l11 W+ + l21 Wx|^2 + |l22 Wx|^2 is a sum of
-        // squares (no cancellation when F is ill-conditioned)
-        if (pp.ginv[0] > 0.0) {
-            const double l11 = sqrt(pp.ginv[0]);
-            const double l21 = pp.ginv[1] / l11;
-            pp.chol[0] = l11;
-            pp.chol[1] = l21;
-            pp.chol[2] = sqrt(fmax(0.0, pp.ginv[2] - l21 * l21));
-        } else {
-            pp.chol[2] = sqrt(fmax(0.0, pp.ginv[2]));
-        }
-        for (int i = 0; i < n_det; ++i) {
-            pp.w1[i] = pp.chol[0] * pp.u[i][0] + pp.chol[1] * pp.u[i][1];
-            pp.w2[i] = pp.chol[2] * pp.u[i][1];
-        }
-        // (tau0, tau1.5) -> x = pi M f_*, eta; then the 2PN chirp times tau1, tau2.
+    ParticleParams* pp = out + pc;
+    if (threadIdx.x >= 32) {
+        // (tau0, tau1.5) -> x = pi M f_*, eta; then the 2PN chirp times: tau1 by even lanes, tau2 by odd ones
         const double pi = 0.5 * kTwoPi;
         const double x = 5.0 * tau15 / (32.0 * pi * tau0);
         const double cx = cbrt(x);
         const double eta = 1.0 / (cx * cx) / (8.0 * f_star * tau15);
-        const double tau1 = 5.0 / (192.0 * pi * f_star * eta * x) * (743.0 / 336.0 + 11.0 * eta / 4.0);
-        const double tau2 = 5.0 / (128.0 * pi * f_star * eta * cx) *
-                            (3058673.0 / 1016064.0 + 5429.0 * eta / 1008.0 + 617.0 * eta * eta / 144.0);
-        pp.c[0] = 0.6 * f_star * tau0;
-        pp.c[1] = f_star * tau1;
-        pp.c[2] = -1.5 * f_star * tau15;
-        pp.c[3] = 3.0 * f_star * tau2;
-        pp.valid = 1;
-        // Remainder of psi(k + c) = psi(k) + c psi' + c^2 psi''/2 for c <= C (FP32 pass A, C + 1
-        // adjacent columns per lane group, C = 3 or 7): at most C^3/6 max |psi'''| over the band,
-        // taken at k_b = f_*/df - 2 (C + 1) (the band's lowest bin, less the C by which an anchor bin
-        // may lie below it, with margin), where |psi'''| <= sum_m |c_m| e_m (e_m + 1) (e_m + 2)
-        // phi^-e_m / k^3. Bit 0: C = 3; bit 1: C = 7.
+        const bool odd = sub & 1;
+        const double scale = 5.0 / ((odd ? 128.0 * pi : 192.0 * pi) * f_star * eta * (odd ? cx : x));
+        const double tau = scale * (odd ? 3058673.0 / 1016064.0 + 5429.0 * eta / 1008.0 + 617.0 * eta * eta / 144.0
+                                        : 743.0 / 336.0 + 11.0 * eta / 4.0);
+        const double tau1 = __shfl_sync(0xffffffffu, tau, lane0), tau2 = __shfl_sync(0xffffffffu, tau, lane0 + 1);
+        const double c[4] = {0.6 * f_star * tau0, f_star * tau1, -1.5 * f_star * tau15, 3.0 * f_star * tau2};
+        int taylor = 0;
+#pragma unroll
         for (int bit = 0; bit < 2; ++bit) {
-            const double cm = bit == 0 ? 3.0 : 7.0;
-            const double kb = f_star / df - 2.0 * (cm + 1.0);
-            if (kb < 1.0) continue;
-            const double r = f_star / (kb * df);   // phi^-1 at k_b
-            const double r13 = cbrt(r);
-            const double d3 = (fabs(pp.c[0]) * (440.0 / 27.0) * r * r13 * r13 + fabs(pp.c[1]) * 6.0 * r +
-                               fabs(pp.c[2]) * (80.0 / 27.0) * r13 * r13 + fabs(pp.c[3]) * (28.0 / 27.0) * r13) /
-                              (kb * kb * kb);
-            if (cm * cm * cm / 6.0 * d3 < 1e-7) pp.taylor_ok |= 1 << bit;
+            double rem = 0.0;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) rem += fabs(c[r]) * tb.m[bit][r];
+            if (rem < 1e-7) taylor |= 1 << bit;   // false for the infinite bound and for a NaN
+        }
+        if (!have) return;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (sub != r) continue;
+            const double v = ok ? c[r] : 0.0;
+            pp->c[r] = v;
+            pp->ch[r] = (float)v;
+            pp->cl[r] = (float)(v - (double)(float)v);
+        }
+        if (sub == 4) {
+            pp->valid = ok;
+            pp->taylor_ok = ok ? taylor : 0;
+        }
+        return;
+    }
+    // sky: sin and cos of alpha by even lanes, of delta by odd ones
+    double sn, cs;
+    sincos(sub & 1 ? delta : alpha, &sn, &cs);
+    const double sa = __shfl_sync(0xffffffffu, sn, lane0), ca = __shfl_sync(0xffffffffu, cs, lane0);
+    const double sd = __shfl_sync(0xffffffffu, sn, lane0 + 1), cd = __shfl_sync(0xffffffffu, cs, lane0 + 1);
+    const double nx = cd * ca, ny = cd * sa, nz = sd;
+    const double bx[3] = {sa, -ca, 0.0};             // -alpha_hat
+    const double by[3] = {-sd * ca, -sd * sa, cd};   // delta_hat
+    double dturn = 0.0, fp = 0.0, fx = 0.0, sfp = 0.0, sfx = 0.0;
+    if (sub < n_det) {
+        const double* d = det9 + 9 * sub;
+        dturn = -(d[0] * nx + d[1] * ny + d[2] * nz) / kCLight * df;
+        const double xX = d[3] * bx[0] + d[4] * bx[1] + d[5] * bx[2];
+        const double xY = d[3] * by[0] + d[4] * by[1] + d[5] * by[2];
+        const double yX = d[6] * bx[0] + d[7] * bx[1] + d[8] * bx[2];
+        const double yY = d[6] * by[0] + d[7] * by[1] + d[8] * by[2];
+        fp = 0.5 * (xX * xX - xY * xY - yX * yX + yY * yY);
+        fx = xX * xY - yX * yY;
+        sfp = s2[sub] * fp;
+        sfx = s2[sub] * fx;
+    }
+    double g11 = 0.0, g12 = 0.0, g22 = 0.0;
+    for (int i = 0; i < n_det; ++i) {
+        const double fpi = __shfl_sync(0xffffffffu, fp, lane0 + i), fxi = __shfl_sync(0xffffffffu, fx, lane0 + i);
+        const double spi = __shfl_sync(0xffffffffu, sfp, lane0 + i), sxi = __shfl_sync(0xffffffffu, sfx, lane0 + i);
+        g11 += spi * fpi;
+        g12 += spi * fxi;
+        g22 += sxi * fxi;
+    }
+    const double det = g11 * g22 - g12 * g12;
+    const double tr = g11 + g22;
+    // G^-1: lane 0 divides for its first entry, lane 1 for its second, the others for its third
+    const double quot = (sub == 0 ? g22 : sub == 1 ? -g12 : g11) / det;
+    double ginv[3] = {__shfl_sync(0xffffffffu, quot, lane0), __shfl_sync(0xffffffffu, quot, lane0 + 1),
+                      __shfl_sync(0xffffffffu, quot, lane0 + 2)};
+    if (det < kRank1Rtol * (0.5 * tr) * (0.5 * tr)) {
+        const double lam = 0.5 * tr + sqrt(0.25 * (g11 - g22) * (g11 - g22) + g12 * g12);
+        double e1 = lam - g22, e2 = g12;
+        double f1 = g12, f2 = lam - g11;
+        if (f1 * f1 + f2 * f2 > e1 * e1 + e2 * e2) { e1 = f1; e2 = f2; }
+        const double nrm = e1 * e1 + e2 * e2;
+        ginv[0] = ginv[1] = ginv[2] = 0.0;
+        if (lam > 0.0 && nrm > 0.0) {
+            ginv[0] = e1 * e1 / nrm / lam;
+            ginv[1] = e1 * e2 / nrm / lam;
+            ginv[2] = e2 * e2 / nrm / lam;
         }
     }
-    for (int r = 0; r < 4; ++r) {
-        pp.ch[r] = (float)pp.c[r];
-        pp.cl[r] = (float)(pp.c[r] - (double)pp.ch[r]);
+    // Cholesky factor of G^-1 so that Gamma^2 = |l11 W+ + l21 Wx|^2 + |l22 Wx|^2 is a sum of
+    // squares (no cancellation when F is ill-conditioned)
+    double chol[3] = {0.0, 0.0, 0.0};
+    if (ginv[0] > 0.0) {
+        const double l11 = sqrt(ginv[0]);
+        const double l21 = ginv[1] / l11;
+        chol[0] = l11;
+        chol[1] = l21;
+        chol[2] = sqrt(fmax(0.0, ginv[2] - l21 * l21));
+    } else {
+        chol[2] = sqrt(fmax(0.0, ginv[2]));
     }
-    for (int i = 0; i < FCAS_MAX_DET; ++i) {
-        if (i >= n_det) pp.w1[i] = pp.w2[i] = 0.0;
-        pp.dh[i] = (float)pp.dturn[i];
-        pp.dl[i] = (float)(pp.dturn[i] - (double)pp.dh[i]);
-        pp.w1f[i] = (float)pp.w1[i];
-        pp.w2f[i] = (float)pp.w2[i];
-        double u = (double)kstep * pp.dturn[i];   // |u| < 2^24 turns, exact to ~1e-9
-        u -= rint(u);
-        double su, cu;
-        sincospi(2.0 * u, &su, &cu);
-        pp.dstep[i] = make_float2((float)cu, (float)su);
+    const bool det_lane = ok && sub < n_det;
+    const double w1 = det_lane ? chol[0] * fp + chol[1] * fx : 0.0;
+    const double w2 = det_lane ? chol[2] * fx : 0.0;
+    if (!det_lane) dturn = fp = fx = 0.0;
+    double us = (double)kstep * dturn;   // |us| < 2^24 turns, exact to ~1e-9
+    us -= rint(us);
+    double su, cu;
+    sincospi(2.0 * us, &su, &cu);
+    if (!have) return;
+    pp->dturn[sub] = dturn;
+    pp->u[sub][0] = fp;
+    pp->u[sub][1] = fx;
+    pp->w1[sub] = w1;
+    pp->w2[sub] = w2;
+    pp->dh[sub] = (float)dturn;
+    pp->dl[sub] = (float)(dturn - (double)(float)dturn);
+    pp->w1f[sub] = (float)w1;
+    pp->w2f[sub] = (float)w2;
+    pp->dstep[sub] = make_float2((float)cu, (float)su);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        if (sub != r) continue;
+        pp->ginv[r] = ok ? ginv[r] : 0.0;
+        pp->chol[r] = ok ? chol[r] : 0.0;
     }
-    out[p] = pp;
 }
 
 cudaError_t launch_geometry(const double* theta, int64_t n, ParticleParams* out, const double* det9,
                             const double* sigma2_scaled, int n_det, double f_star, double df, int64_t kstep,
                             cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    const int threads = 128;
-    const int64_t blocks = (n + threads - 1) / threads;
-    geometry_kernel<<<(unsigned)blocks, threads, 0, s>>>(theta, n, out, det9, sigma2_scaled, n_det, f_star, df,
-                                                          kstep);
+    const int64_t blocks = (n + kGeomParticles - 1) / kGeomParticles;
+    geometry_kernel<<<(unsigned)blocks, 64, 0, s>>>(theta, n, out, det9, sigma2_scaled, n_det, f_star, df, kstep,
+                                                    taylor_bound(f_star, df));
     return cudaGetLastError();
 }
 
