@@ -283,8 +283,9 @@ int apply_layout(fcas_ctx* c, int bias, int k1b, int sub, int radix_bits_a, cuda
     c->sub = sub;
     c->radix_bits_a = radix_bits_a;
     c->nb_partials = nb;
-    cudaError_t e = launch_stage_tables(l2, radix_bits_a, c->d_stw_a64, c->d_stw_a32, st);
-    if (e == cudaSuccess) e = launch_stage_tables(l1, 4, c->d_stw_b64, c->d_stw_b32, st);
+    const bool local = c->setup.precision == FCAS_PREC_FP32;   // the form with warp-local exchanges
+    cudaError_t e = launch_stage_tables(l2, radix_bits_a, local ? k1b : 0, c->d_stw_a64, c->d_stw_a32, st);
+    if (e == cudaSuccess) e = launch_stage_tables(l1, 4, local ? 1 : 0, c->d_stw_b64, c->d_stw_b32, st);
     if (e == cudaSuccess && c->d_stw_aff) e = launch_split_ff(c->d_stw_a64, c->d_stw_aff, (int64_t)1 << l2, st);
     if (e == cudaSuccess && c->d_stw_bff) e = launch_split_ff(c->d_stw_b64, c->d_stw_bff, (int64_t)1 << l1, st);
     if (e == cudaSuccess)
@@ -741,7 +742,7 @@ int fcas_autotune(fcas_ctx* c, int64_t n_particles, const char* cache_path, void
     for (char& ch : gpu)
         if (ch == ' ') ch = '_';
     char key[512];
-    snprintf(key, sizeof(key), "fcas-tune-v3 %s %lld %d %d %lld", gpu.c_str(), (long long)c->setup.n_fft,
+    snprintf(key, sizeof(key), "fcas-tune-v4 %s %lld %d %d %lld", gpu.c_str(), (long long)c->setup.n_fft,
              c->setup.n_det, c->setup.precision, (long long)n_particles);
     if (cache_path) {
         if (FILE* f = fopen(cache_path, "r")) {
@@ -790,7 +791,7 @@ int fcas_autotune(fcas_ctx* c, int64_t n_particles, const char* cache_path, void
         if (l2 == last_l2 || c->log_n - l2 > kMaxLogPass) continue;
         last_l2 = l2;
         int ks[8], rbs[8];
-        int nk = pass_a_k1b_variants(l2, c->setup.precision, ks);   // at most 4, plus 2 radix-8 shapes below
+        int nk = pass_a_k1b_variants(l2, c->setup.precision, ks);   // at most 5, plus 2 radix-8 shapes below
         for (int q = 0; q < nk; ++q) rbs[q] = 4;
         for (int k8 : {4, 2}) {
             if (pass_a_radix8_available(l2, c->setup.precision, k8)) {

@@ -10,12 +10,13 @@
 // e^{S 2 pi i r (jj mod Ns) / (Ns R)}, applies the R-point DFT in registers and writes to
 // (jj / Ns) Ns R + (jj mod Ns) + r Ns. Consecutive stages exchange data through shared memory,
 // padded by one element every 16 so that the stride-16 writes of a stage do not share banks.
-// With PP the exchanges alternate between two buffers `alt` elements apart (exchange e of the
-// transform uses buffer (e + par0) mod 2): a buffer is rewritten only two exchanges after it was
-// last read, with a barrier in between, so the barrier before each write is dropped.
+// The threads that work on one residue class of the index (modulo 16 after the first radix-16 stage) are
+// consecutive, so that from the second exchange on all data stay within a warp: those exchanges need no
+// barrier of the CTA (see fft_local_bits).
 // Twiddles come from a per-length table laid out stage by stage as
-//   T[(Ns - 1) + (r - 1) Ns + jm] = e^{2 pi i r jm / (Ns R)},   r = 1..R-1, jm = 0..Ns-1,
-// so that a warp reads consecutive entries; the stages together use L - 1 entries.
+//   T[(Ns - 1) + (r - 1) Ns + P(jm)] = e^{2 pi i r jm / (Ns R)},   r = 1..R-1, jm = 0..Ns-1,
+// with P the order in which the stage's threads take jm (fft_tw_pos), so that a warp reads consecutive
+// entries; the stages together use L - 1 entries.
 #pragma once
 
 #include <type_traits>
@@ -57,14 +58,57 @@ __host__ __device__ constexpr int fftr_radix_bits(int log_l, int done, int maxrb
     return (log_l - done) >= maxrb ? maxrb : (log_l - done);
 }
 __host__ __device__ constexpr int fftr_v(int log_l, int maxrb) { return log_l >= maxrb ? (1 << maxrb) : (1 << log_l); }
-__host__ __device__ constexpr int fft16_radix_bits(int log_l, int done) { return fftr_radix_bits(log_l, done, 4); }
 __host__ __device__ constexpr int fft16_v(int log_l) { return fftr_v(log_l, 4); }
-__host__ __device__ constexpr int fft16_pad(int e) { return e + (e >> 4); }
-__host__ __device__ constexpr int fft16_buf_elems(int log_l) { return fft16_pad(1 << log_l); }
-// the exchange padding with one spare element per 2^PS (PS = 4 above; 3 for 16-byte elements in
-// radix-8 stages, whose first-stage writes would otherwise fall two to a bank group)
-template <int PS> __host__ __device__ constexpr int xpad(int e) { return e + (e >> PS); }
-template <int PS> __host__ __device__ constexpr int xbuf_elems(int log_l) { return xpad<PS>(1 << log_l); }
+// Warp-local exchanges. After the stages that resolve the low CB bits of the output index, every later stage
+// of the transform reads and writes only elements of one residue class modulo 2^CB; thread j then takes the
+// tasks of the permuted index fft_job(j) = class + 2^CB (position in the class), with the class in the upper
+// bits of j, so that a class belongs to G / 2^CB consecutive values of j. Where those threads (times the K
+// columns that share them) lie in one warp, the exchanges after that stage are ordered by __syncwarp alone
+// and the CTA meets once per transform instead of around every exchange. fft_local_bits is the smallest such
+// CB, or 0 where no exchange can be local; where one warp holds the whole transform (fft_one_warp) every
+// exchange is local in the plain order. K = 0: the CTA meets at every exchange. The packed FP32 form uses them (60-min
+// pass B alone 42.0 -> 40.9 us for one particle, 15-min passes 786 / 478 -> 777 / 469 us per 64 particles; no
+// change for 64 particles of the 60-min workload). The float-float form does not: its unrolled double-word
+// code no longer stays in the instruction cache when warps drift apart (60-min pass B 2.00 -> 2.35 ms per 8
+// particles); the binary64 form waits for its arithmetic unit alone and gains nothing.
+__host__ __device__ constexpr int fft_log_g(int log_l, int maxrb) { return log_l > maxrb ? log_l - maxrb : 0; }
+__host__ __device__ constexpr int fft_local_bits(int log_l, int maxrb, int k) {
+    if (k == 0 || (k << fft_log_g(log_l, maxrb)) <= 32) return 0;
+    for (int cb = maxrb; cb <= fft_log_g(log_l, maxrb) && cb + maxrb < log_l; cb += maxrb) {
+        const int threads = k << (fft_log_g(log_l, maxrb) - cb);   // of one class
+        if (threads >= 8 && threads <= 32) return cb;              // fewer: two classes would share banks
+    }
+    return 0;
+}
+// nt: threads of the CTA
+__host__ __device__ constexpr bool fft_one_warp(int log_l, int maxrb, int k, int nt) {
+    return k > 0 && (k << fft_log_g(log_l, maxrb)) <= 32 && nt >= 32;
+}
+// the task (and, for the last stage, the first output index) of thread j: outputs are fft_job(j) + q G
+template <int LOG_L, int MAXRB, int K>
+__host__ __device__ constexpr int fft_job(int j) {
+    constexpr int cb = fft_local_bits(LOG_L, MAXRB, K), gb = fft_log_g(LOG_L, MAXRB) - cb;
+    return cb == 0 ? j : (j >> gb) + ((j & ((1 << gb) - 1)) << cb);
+}
+// P(jm): the place of a stage's twiddle jm (0 <= jm < ns) in its block of the table; cb the local bits
+// above. Thread j of G takes jm = fft_job(j) mod ns (+ h G where ns > G) in the stages from cb on.
+__host__ __device__ constexpr int fft_tw_pos(int jm, int ns, int log_g, int cb) {
+    if (cb == 0 || ns < (1 << cb)) return jm;
+    const int b = ns < (1 << log_g) ? ns : 1 << log_g, lo = jm & (b - 1);
+    return jm - lo + (lo & ((1 << cb) - 1)) * (b >> cb) + (lo >> cb);
+}
+// The exchange padding: one spare element per 2^PS (4; 3 for 16-byte elements in radix-8 stages, whose
+// first-stage writes would otherwise fall two to a bank group). In a local exchange consecutive threads sit
+// 2^CB elements apart when they read and 2^(CB + MAXRB) when they write: one more element per 2^(CB + MAXRB),
+// and per 2^CB where that is not 2^PS already, keeps them in different banks.
+template <int LOG_L, int MAXRB, int K, int PS> __host__ __device__ constexpr int fft_pad(int e) {
+    constexpr int cb = fft_local_bits(LOG_L, MAXRB, K);
+    return e + (e >> PS) + (cb > PS ? e >> cb : 0) + (cb > 0 ? e >> (cb + MAXRB) : 0);
+}
+// elements of one transform's exchange buffer
+template <int LOG_L, int MAXRB, int K, int PS> __host__ __device__ constexpr int fft_buf_elems() {
+    return fft_pad<LOG_L, MAXRB, K, PS>(1 << LOG_L);
+}
 
 // Checked build (FCAS_CHECKED): the fitness kernels recompute each shared-memory, table and global
 // index from its definition and range-test it; a failed test sets bit `bit` of this flag (read and
@@ -230,9 +274,12 @@ __device__ __forceinline__ void dft_r(C (&a)[R]) {
 // LH (first stage only): the upper half of the input (v[V/2 ..]) is zero. TWL: the stage twiddles
 // w^r (r < 4) and w^{4h} come from the table and the rest as one product each (instead of w and w^4
 // loaded and the other powers formed by products); fewer instructions, a few more registers.
-template <typename Real, int S, int LOG_L, int DONE, int MAXRB, bool PP, bool LH = false, bool TWL = false, int PS = 4>
-__device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)], cplx<Real>* buf0, int es, int j,
-                                           const fft_tw<Real>* __restrict__ stw, int alt, int par0) {
+// j: the stage's task, jr: the thread's number. K: columns that share it (consecutive threads) where exchanges
+// may be local, 0 otherwise; NT: threads of the CTA. FRESH: nothing has read the exchange buffer yet (no
+// barrier before the first write: 15-min pass B 495 -> 478 us per 64 particles).
+template <typename Real, int S, int LOG_L, int DONE, int MAXRB, int K, int NT, bool LH, bool TWL, int PS, bool FRESH>
+__device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)], cplx<Real>* buf, int es, int j,
+                                           int jr, const fft_tw<Real>* __restrict__ stw) {
     using C = cplx<Real>;
     using W = fft_tw<Real>;
     constexpr int L = 1 << LOG_L;
@@ -244,23 +291,28 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
     constexpr int NS = 1 << DONE;
     constexpr bool FIRST = DONE == 0;
     constexpr bool LAST = DONE + RB == LOG_L;
-    constexpr int ST = DONE / MAXRB;
+    constexpr int BUF = fft_buf_elems<LOG_L, MAXRB, K, PS>();
+    constexpr auto pad = fft_pad<LOG_L, MAXRB, K, PS>;
+    // the exchange after this stage is local when the stage itself already works on one residue class
+    constexpr int CB = fft_local_bits(LOG_L, MAXRB, K);
+    constexpr bool PERM = CB != 0 && DONE >= CB;
+    constexpr bool LOCAL = PERM || fft_one_warp(LOG_L, MAXRB, K, NT);
     if constexpr (!FIRST) {
-        const cplx<Real>* buf = (PP && ((ST - 1 + par0) & 1)) ? buf0 + alt : buf0;
         if constexpr (G % (1 << PS) == 0) {
-            // pad(j + q G) = pad(j) + q (G + G / 2^PS): one base address, constant offsets
-            const C* rb = buf + xpad<PS>(j) * es;
+            // pad(j + q G) = pad(j) + pad(q G): one base address, constant offsets (j < G, and G is a multiple of
+            // 2^PS and a multiple or a divisor of the larger groups)
+            const C* rb = buf + pad(j) * es;
 #pragma unroll
             for (int q = 0; q < V; ++q) {
-                const int e = xpad<PS>(j) + q * (G + (G >> PS));
-                if (FCAS_CHECK(e == xpad<PS>(j + q * G) && e < xbuf_elems<PS>(LOG_L), kCheckExchangeRead))
-                    v[q] = rb[q * (G + (G >> PS)) * es];
+                const int e = pad(j) + pad(q * G);
+                if (FCAS_CHECK((e == pad(j + q * G) && e < BUF), kCheckExchangeRead))
+                    v[q] = rb[pad(q * G) * es];
             }
         } else {
 #pragma unroll
             for (int q = 0; q < V; ++q)
-                if (FCAS_CHECK(xpad<PS>(j + q * G) < xbuf_elems<PS>(LOG_L), kCheckExchangeRead))
-                    v[q] = buf[xpad<PS>(j + q * G) * es];
+                if (FCAS_CHECK((pad(j + q * G) < BUF), kCheckExchangeRead))
+                    v[q] = buf[pad(j + q * G) * es];
         }
     }
 #pragma unroll
@@ -270,7 +322,12 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
 #pragma unroll
         for (int r = 0; r < R; ++r) a[r] = v[h + r * T];
         if constexpr (NS > 1) {
-            const int jm = jj & (NS - 1);
+            // the twiddle's place P(jm) from the thread's own number: j itself where the block holds G entries
+            // or more, class-major within the block otherwise
+            constexpr int LG = fft_log_g(LOG_L, MAXRB);
+            const int jm = !PERM || NS < (1 << CB) ? jj & (NS - 1)
+                           : NS >= G                ? jr + h * G
+                                                    : (jr >> (LG - CB)) * (NS >> CB) + (jr & ((NS >> CB) - 1));
             const W* t = stw + (NS - 1) + jm;
             if constexpr (R >= 8 && TWL && !std::is_same<Real, ffloat>::value) {
                 W wl[4], wh[R / 4];
@@ -339,51 +396,50 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
         for (int r = 0; r < R; ++r) v[h + r * T] = a[r];
     }
     if constexpr (!LAST) {
-        if constexpr (!PP) __syncthreads();
-        cplx<Real>* buf = (PP && ((ST + par0) & 1)) ? buf0 + alt : buf0;
+        // every read of the buffer's previous contents done
+        if constexpr (LOCAL) __syncwarp();
+        else if constexpr (!(FIRST && FRESH)) __syncthreads();
 #pragma unroll
         for (int h = 0; h < T; ++h) {
             const int jj = j + h * G;
             const int dst = (jj / NS) * NS * R + (jj & (NS - 1));
-            // pad(dst + r NS) = pad(dst) + r NS + (r NS >> PS) when adding r NS to dst never carries
-            // into a new group of 2^PS differently from r NS itself: NS a multiple of 2^PS, or NS
-            // dividing 2^PS with NS R a multiple of 2^PS (dst mod 2^PS < NS), or PS = 4, NS = 1 and
-            // R = 8 (dst mod 16 in {0, 8})
+            // pad(dst + r NS) = pad(dst) + pad(r NS) when adding r NS to dst never carries into a new group of
+            // 2^PS differently from r NS itself: NS a multiple of 2^PS, or NS dividing 2^PS with NS R a multiple
+            // of 2^PS (dst mod 2^PS < NS), or PS = 4, NS = 1 and R = 8 (dst mod 16 in {0, 8}). The larger groups
+            // never do: they, NS and NS R are powers of two and dst mod (NS R) < NS.
             constexpr int GP = 1 << PS;
             if constexpr (NS % GP == 0 || (GP % NS == 0 && (NS * R) % GP == 0) || (PS == 4 && NS == 1 && R == 8)) {
-                C* wb = buf + xpad<PS>(dst) * es;
+                C* wb = buf + pad(dst) * es;
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    const int e = xpad<PS>(dst) + r * NS + ((r * NS) >> PS);
-                    if (FCAS_CHECK(e == xpad<PS>(dst + r * NS) && e < xbuf_elems<PS>(LOG_L), kCheckExchangeWrite))
-                        wb[(r * NS + ((r * NS) >> PS)) * es] = v[h + r * T];
+                    const int e = pad(dst) + pad(r * NS);
+                    if (FCAS_CHECK((e == pad(dst + r * NS) && e < BUF),
+                                   kCheckExchangeWrite))
+                        wb[pad(r * NS) * es] = v[h + r * T];
                 }
             } else {
 #pragma unroll
                 for (int r = 0; r < R; ++r)
-                    if (FCAS_CHECK(xpad<PS>(dst + r * NS) < xbuf_elems<PS>(LOG_L), kCheckExchangeWrite))
-                        buf[xpad<PS>(dst + r * NS) * es] = v[h + r * T];
+                    if (FCAS_CHECK((pad(dst + r * NS) < BUF), kCheckExchangeWrite))
+                        buf[pad(dst + r * NS) * es] = v[h + r * T];
             }
         }
-        __syncthreads();
+        if constexpr (LOCAL) __syncwarp();
+        else __syncthreads();
     }
 }
 
-template <typename Real, int S, int LOG_L, int MAXRB, bool PP = false, int DONE = 0, bool LH = false, bool TWL = false,
-          int PS = 4>
+// The whole transform: v holds x[j + q G] on entry and X[fft_job(j) + q G] on exit.
+template <typename Real, int S, int LOG_L, int MAXRB, int K, int NT, bool LH, bool TWL, int PS, bool FRESH, int DONE = 0>
 __device__ __forceinline__ void fftr(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)], cplx<Real>* buf, int es, int j,
-                                     const fft_tw<Real>* __restrict__ stw, int alt = 0, int par0 = 0) {
+                                     const fft_tw<Real>* __restrict__ stw) {
     if constexpr (DONE < LOG_L) {
-        fftr_stage<Real, S, LOG_L, DONE, MAXRB, PP, LH, TWL, PS>(v, buf, es, j, stw, alt, par0);
-        fftr<Real, S, LOG_L, MAXRB, PP, DONE + fftr_radix_bits(LOG_L, DONE, MAXRB), false, TWL, PS>(v, buf, es, j, stw,
-                                                                                                  alt, par0);
+        constexpr int CB = fft_local_bits(LOG_L, MAXRB, K);
+        const int jt = CB != 0 && DONE >= CB ? fft_job<LOG_L, MAXRB, K>(j) : j;   // permuted from stage CB on
+        fftr_stage<Real, S, LOG_L, DONE, MAXRB, K, NT, LH, TWL, PS, FRESH>(v, buf, es, jt, j, stw);
+        fftr<Real, S, LOG_L, MAXRB, K, NT, LH, TWL, PS, FRESH, DONE + fftr_radix_bits(LOG_L, DONE, MAXRB)>(
+            v, buf, es, j, stw);
     }
-}
-
-template <typename Real, int S, int LOG_L, bool PP = false>
-__device__ __forceinline__ void fft16(cplx<Real> (&v)[fft16_v(LOG_L)], cplx<Real>* buf, int es, int j,
-                                      const fft_tw<Real>* __restrict__ stw, int alt = 0, int par0 = 0) {
-    fftr<Real, S, LOG_L, 4, PP>(v, buf, es, j, stw, alt, par0);
 }
 
 }  // namespace fcas

@@ -75,27 +75,32 @@ struct ParticleParams {
 // ------------------------------------------------------------------------------------------
 __host__ __device__ constexpr int imin_c(int a, int b) { return a < b ? a : b; }
 __host__ __device__ constexpr int imax_c(int a, int b) { return a > b ? a : b; }
-#ifndef FCAS_PASS_A_THREADS_F32
-#define FCAS_PASS_A_THREADS_F32 512   // target CTA size of pass A, FP32 form
-#endif
 #ifndef FCAS_PASS_A_SUB
-#define FCAS_PASS_A_SUB 8             // adjacent column blocks of one particle scheduled together
+#define FCAS_PASS_A_SUB 16            // adjacent column blocks of one particle scheduled together
 #endif
 #ifndef FCAS_SPLIT_BIAS
 #define FCAS_SPLIT_BIAS 0             // N2 = 2^(floor(log2 N / 2) - bias): a smaller pass-A transform
 #endif
 #ifndef FCAS_PASS_B_THREADS_F32
-#define FCAS_PASS_B_THREADS_F32 256   // target CTA size of pass B, FP32 form
+#define FCAS_PASS_B_THREADS_F32 64    // target CTA size of pass B, FP32 form
 #endif
 __host__ __device__ constexpr int shape_v(int log_l) { return log_l >= 4 ? 16 : (1 << log_l); }
+// Columns per pass-A CTA. FP32: CTAs of 128 threads, but at least 4 columns (row pieces of 64 bytes; 2 columns
+// write 32-byte pieces and lose 12 % at 2^11 points) while a CTA stays within 512 threads. Several small CTAs
+// per SM are in different phases (loads, arithmetic, exchanges) at any time, one large one is in the same
+// phase throughout: us per 64 particles with 4 / 8 / 16 columns, 2^8 points 28.2 / 27.4 / 29.6, 2^9 points
+// 101 / 110 / 121, 2^10 points 778 / 827 / -.
 __host__ __device__ constexpr int pass_a_k1b(int log_l, int real_bytes) {
-    return imin_c(imin_c(16, imax_c(1, (real_bytes == 4 ? FCAS_PASS_A_THREADS_F32 : 256) /
-                                           ((1 << log_l) / shape_v(log_l)))),
-                  1 << log_l);
+    const int g = (1 << log_l) / shape_v(log_l);   // threads per column
+    const int k = real_bytes == 4 ? imax_c(128 / g, imin_c(4, 512 / g)) : 256 / g;
+    return imin_c(imin_c(16, imax_c(1, k)), 1 << log_l);
 }
 __host__ __device__ constexpr int pass_a_threads(int log_l, int real_bytes) {
     return pass_a_k1b(log_l, real_bytes) * ((1 << log_l) / shape_v(log_l));
 }
+// Rows per pass-B CTA. FP32: one row where a row takes 64 threads or more, for the same reason: us per 64
+// particles with CTAs of 256 / 128 / 64 threads, 2^8 points 19.9 / 17.3 / 16.8, 2^9 points 80 / 76 / 75, 2^11
+// points 469 / 411 / 411.
 __host__ __device__ constexpr int pass_b_tb(int log_l, int real_bytes) {
     return imin_c(imin_c(16, imax_c(1, (real_bytes == 4 ? FCAS_PASS_B_THREADS_F32 : 128) /
                                            ((1 << log_l) / shape_v(log_l)))),

@@ -277,6 +277,7 @@ int pass_a_k1b_variants(int log_n2, int precision, int* out) {
         if (rb == 4 && LG >= 8) {                                                           \
             if (x2_k1b_ok<LG>(kd / 2)) out[n++] = kd / 2;                                   \
             if (x2_k1b_ok<LG>(kd * 2)) out[n++] = kd * 2;                                   \
+            if (x2_k1b_ok<LG>(kd * 4)) out[n++] = kd * 4;                                   \
             if (LG >= 10 && kd / 2 > 1) out[n++] = 1;                                       \
         }                                                                                   \
         return n;                                                                           \
@@ -297,7 +298,8 @@ template cudaError_t launch_pass_b<double>(const FitnessPlan&, const ParticlePar
 // ------------------------------------------------------------------------------------------
 // per-stage twiddle tables of the radix-16 transforms (create time)
 // ------------------------------------------------------------------------------------------
-__global__ void stage_table_kernel(int log_l, int maxrb, double2* t64, float2* t32) {
+// entry order: fft_tw_pos of transforms whose exchanges are local from bit cb on
+__global__ void stage_table_kernel(int log_l, int maxrb, int cb, double2* t64, float2* t32) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     const int l = 1 << log_l;
     if (m >= l) return;
@@ -309,7 +311,10 @@ __global__ void stage_table_kernel(int log_l, int maxrb, double2* t64, float2* t
         if (ns > 1 && m >= ns - 1 && m < ns * r_ - 1) {
             const int off = m - (ns - 1);
             const int r = off / ns + 1;
-            const int jm = off % ns;
+            // the inverse of fft_tw_pos on 0..ns-1
+            const int pos = off % ns;
+            const int b = ns < (1 << fft_log_g(log_l, maxrb)) ? ns : 1 << fft_log_g(log_l, maxrb), lo = pos & (b - 1);
+            const int jm = cb == 0 || ns < (1 << cb) ? pos : pos - lo + lo / (b >> cb) + ((lo & ((b >> cb) - 1)) << cb);
             double sn, cs;
             // e^{2 pi i r jm / (Ns R)}, argument reduced exactly before sincospi
             const long long num = ((long long)r * jm) % ((long long)ns * r_);
@@ -334,9 +339,9 @@ unsigned int take_index_checks(cudaStream_t s) {
 #endif
 }
 
-cudaError_t launch_stage_tables(int log_l, int maxrb, double2* t64, float2* t32, cudaStream_t s) {
+cudaError_t launch_stage_tables(int log_l, int maxrb, int k, double2* t64, float2* t32, cudaStream_t s) {
     const int l = 1 << log_l;
-    stage_table_kernel<<<(l + 255) / 256, 256, 0, s>>>(log_l, maxrb, t64, t32);
+    stage_table_kernel<<<(l + 255) / 256, 256, 0, s>>>(log_l, maxrb, fft_local_bits(log_l, maxrb, k), t64, t32);
     return cudaGetLastError();
 }
 

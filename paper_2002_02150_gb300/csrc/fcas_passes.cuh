@@ -112,21 +112,15 @@ __device__ __forceinline__ ffloat ff_frac_mul_int(int k, float d1, float d2, flo
 // W_a(t) = sum_i w_a,i Z_i(t) are the transforms of P_a (Sec. II.C projection applied before the
 // t_c scan instead of after it).
 // ------------------------------------------------------------------------------------------
-// Pass A's exchange padding: one spare element per 8 for 16-byte elements in radix-8 stages (their
-// first-stage writes would otherwise fall two to a bank group), per 16 otherwise.
+// Exchange padding: one spare element per 8 for 16-byte elements in radix-8 stages (their first-stage
+// writes would otherwise fall two to a bank group), per 16 otherwise.
 template <typename Real, int MAXRB>
 __host__ __device__ constexpr int pass_a_pad_shift() {
     return sizeof(cplx<Real>) == 16 && MAXRB == 3 ? 3 : 4;
 }
 template <typename Real, int LOG_L, int K1B, int MAXRB>
 __host__ __device__ constexpr int pass_a_buf_elems() {
-    return K1B * xbuf_elems<pass_a_pad_shift<Real, MAXRB>()>(LOG_L);
-}
-
-// Pass A keeps two FFT exchange buffers when both fit in 200 KB of shared memory.
-template <typename Real, int LOG_L, int K1B, int MAXRB>
-__host__ __device__ constexpr bool pass_a_pingpong() {
-    return 2 * sizeof(cplx<Real>) * (size_t)pass_a_buf_elems<Real, LOG_L, K1B, MAXRB>() <= 200 * 1024;
+    return K1B * fft_buf_elems<LOG_L, MAXRB, 0, pass_a_pad_shift<Real, MAXRB>()>();
 }
 
 // The float-float form reduces the chirp phase in binary64 (basis as in the binary64 form) and the
@@ -325,15 +319,10 @@ pass_a_kernel(const cplx<Real>* __restrict__ y, const Basis<phase_t<Real>>* __re
         for (int q = 0; q < VH; ++q) v[q] = a == 0 ? r1[q] : r2[q];
 #pragma unroll
         for (int q = VH; q < V; ++q) v[q] = mkc(Real(0.0f), Real(0.0f));
-        // two exchange buffers where shared memory allows (no barrier before each exchange write); the
-        // exchange count is continued across the series so that a buffer is never rewritten before
-        // all its reads of the previous exchange are done
-        constexpr int NX = (LOG_L + MAXRB - 1) / MAXRB - 1;
         // FP32: stage twiddles mostly loaded (60-min pass A 4.11 -> 4.07 ms; pass B keeps the
         // products, which need fewer registers than its three CTAs per SM allow for the loads)
-        fftr<Real, +1, LOG_L, MAXRB, pass_a_pingpong<Real, LOG_L, K1B, MAXRB>(), 0, true, sizeof(Real) == 4,
-             pass_a_pad_shift<Real, MAXRB>()>(v, smem + c, K1B, j, stw, pass_a_buf_elems<Real, LOG_L, K1B, MAXRB>(),
-                                              (a * NX) & 1);
+        fftr<Real, +1, LOG_L, MAXRB, 0, 0, true, sizeof(Real) == 4, pass_a_pad_shift<Real, MAXRB>(), false>(
+            v, smem + c, K1B, j, stw);
         C* orow = out + ((p * kSeries + a) * L) * (int64_t)n1 + k1;
         // e^{2 pi i k1 ta / N} for ta = j + q G: the value at q = 0 times powers of the step e^{2 pi i k1 G / N}
         const int m0 = k1 * j, ms = k1 * G;   // < N
@@ -383,6 +372,14 @@ __device__ __forceinline__ void cta_argmax_store(Real best, int bt, Real* red_v,
         *out = Partial{bt == INT_MAX ? -DBL_MAX : to_double(best), bt == INT_MAX ? INT64_MAX : (int64_t)bt};
 }
 
+// The rows of the intermediate are in the order of pass A's threads (adjacent threads write adjacent rows):
+// row j + q G holds ta = fft_job(j) + q G of pass A's transform (G = 2^log_ga, local from bit cb_a).
+__device__ __forceinline__ int pass_b_ta(int row, int log_ga, int cb_a) {
+    if (cb_a == 0) return row;
+    const int j = row & ((1 << log_ga) - 1), gb = log_ga - cb_a;
+    return row - j + (j >> gb) + ((j & ((1 << gb) - 1)) << cb_a);
+}
+
 // ------------------------------------------------------------------------------------------
 // Pass B: transforms every row ta of both series over k1 (length N1), Gamma^2(t) = |W1(t)|^2 +
 // |W2(t)|^2 for t = ta + N2 tb (Sec. II.C, the maximisation over A_k in closed form), and the
@@ -404,7 +401,7 @@ pass_b_kernel(const cplx<Real>* __restrict__ inter, const ParticleParams* __rest
     constexpr int G = L / V;
     constexpr int TB = pass_b_tb(LOG_L, sizeof(Real));
     constexpr int NT = TB * G;
-    constexpr int BUF = fft16_buf_elems(LOG_L);
+    constexpr int BUF = fft_buf_elems<LOG_L, 4, 0, 4>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* smem = reinterpret_cast<C*>(smem_raw);
     constexpr int NRED = NT >= 32 ? NT / 32 : NT;
@@ -441,7 +438,7 @@ pass_b_kernel(const cplx<Real>* __restrict__ inter, const ParticleParams* __rest
             if (FCAS_CHECK(((p * kSeries + a) * n2 + ta) * (int64_t)L + j + q * G < (int64_t)gridDim.y * kSeries * n2 * L,
                            kCheckInterRead))
                 v[q] = row[j + q * G];
-        fft16<Real, +1, LOG_L>(v, smem + c * BUF, 1, j, stw);
+        fftr<Real, +1, LOG_L, 4, 0, 0, false, false, 4, false>(v, smem + c * BUF, 1, j, stw);
 #pragma unroll
         for (int q = 0; q < V; ++q) g[q] += v[q].x * v[q].x + v[q].y * v[q].y;
     }
@@ -467,15 +464,10 @@ pass_b_kernel(const cplx<Real>* __restrict__ inter, const ParticleParams* __rest
 __host__ __device__ constexpr int x2_a_threads(int log_l, int k1b, int maxrb = 4) {
     return k1b * ((1 << log_l) / fftr_v(log_l, maxrb));
 }
-// exchange padding: one spare element per 8 in radix-8 stages (their first-stage writes of 16-byte
-// elements would otherwise fall two to a bank group), per 16 in radix-16 stages
 __host__ __device__ constexpr int x2_pad_shift(int maxrb) { return maxrb == 3 ? 3 : 4; }
-__host__ __device__ constexpr int x2_buf_elems(int log_l, int k1b, int maxrb = 4) {
-    return maxrb == 3 ? k1b * xbuf_elems<3>(log_l) : k1b * xbuf_elems<4>(log_l);
-}
-// two exchange buffers when both fit in 200 KB of shared memory
-__host__ __device__ constexpr bool x2_a_pingpong(int log_l, int k1b, int maxrb = 4) {
-    return 2 * sizeof(c32x2) * (size_t)x2_buf_elems(log_l, k1b, maxrb) <= 200 * 1024;
+template <int LOG_L, int K1B, int MAXRB>
+__host__ __device__ constexpr int x2_buf_elems() {
+    return K1B * fft_buf_elems<LOG_L, MAXRB, K1B, x2_pad_shift(MAXRB)>();
 }
 // resident CTAs the compiler is held to: 512 threads' worth per SM with radix-16 stages (16 values per
 // thread), 1024 threads' worth with radix-8 stages (8 values per thread)
@@ -487,8 +479,9 @@ __host__ __device__ constexpr int x2_min_blocks(int threads, int maxrb = 4) {
 // (particle, column block) blockIdx.x, blockIdx.x + gridDim.x, ... in the order of the other forms
 // (SUB adjacent column blocks of one particle, then the particles of the chunk, then the next group of
 // column blocks), so that one item's stores drain while the next item loads (60-min pass A 4.27 ->
-// 4.07 ms per 64 particles against one item per CTA). Shapes with two exchange buffers run one item
-// per CTA (the exchange parity restarts with every item). Each item requests its chirp basis and its
+// 4.07 ms per 64 particles against one item per CTA). One exchange buffer: with a second
+// one (no barrier before an exchange's writes) fewer CTAs fit an SM (64-s pass A 42.0 -> 29.9 us per 64
+// particles without it). Each item requests its chirp basis and its
 // first detector's spectrum before its particle's constants arrive (3.98 -> 3.83 ms; requesting more
 // detectors early costs more in registers than it saves).
 template <int LOG_L, int K1B, int MAXRB = 4>
@@ -671,37 +664,40 @@ pass_a_x2_kernel(const float2* __restrict__ y, const BasisF* __restrict__ basis,
         for (int q = VH; q < V; ++q) v[q] = zero_c32x2();
         // one transform of both series; stage twiddles w^r (r < 4) and w^{4h} loaded, the rest one
         // product each (formed once for both series)
-        fftr<x2f, +1, LOG_L, MAXRB, x2_a_pingpong(LOG_L, K1B, MAXRB), 0, true, true, x2_pad_shift(MAXRB)>(
-            v, smem + c, K1B, j, stw, x2_buf_elems(LOG_L, K1B, MAXRB), 0);
+        fftr<x2f, +1, LOG_L, MAXRB, K1B, x2_a_threads(LOG_L, K1B, MAXRB), true, true, x2_pad_shift(MAXRB), false>(
+            v, smem + c, K1B, j, stw);
+        const int jo = fft_job<LOG_L, MAXRB, K1B>(j);
         c32x2* orow = out + ((int64_t)p * L) * n1 + k1;
-        // e^{2 pi i k1 ta / N} for ta = j + q G: the value at q = 0 times powers of the step e^{2 pi i k1 G / N}
-        const int m0 = k1 * j, ms = k1 * G;   // < N
+        // e^{2 pi i k1 ta / N} for ta = jo + q G: the value at q = 0 times powers of the step e^{2 pi i k1 G / N}
+        const int m0 = k1 * jo, ms = k1 * G;   // < N
         float2 w = cmul(__ldg(tw_hi + (m0 >> kTwLoBits)), __ldg(tw_lo + (m0 & ((1 << kTwLoBits) - 1))));
         const float2 step = cmul(__ldg(tw_hi + (ms >> kTwLoBits)), __ldg(tw_lo + (ms & ((1 << kTwLoBits) - 1))));
 #pragma unroll
         for (int q = 0; q < V; ++q) {
-            const int ta = j + q * G;
-            if (FCAS_CHECK((int64_t)p * L * n1 + k1 + (int64_t)ta * n1 < np * (int64_t)L * n1, kCheckInterWrite))
-                st_stream_x2(orow + (int64_t)ta * n1, cmul(v[q], w));   // streamed: read back only by pass B
+            const int row = j + q * G;   // holds ta = jo + q G (pass_b_ta)
+            if (FCAS_CHECK((int64_t)p * L * n1 + k1 + (int64_t)row * n1 < np * (int64_t)L * n1, kCheckInterWrite))
+                st_stream_x2(orow + (int64_t)row * n1, cmul(v[q], w));   // streamed: read back only by pass B
             if (q + 1 < V) w = cmul(w, step);
         }
     }
 }
 
 __host__ __device__ constexpr int x2_b_threads(int log_l) { return pass_b_threads(log_l, 4); }
-// resident pass-B CTAs the compiler is held to: two of 256 threads (16 values per thread)
-__host__ __device__ constexpr int x2_b_min_blocks(int log_l) { return x2_b_threads(log_l) > 256 ? 1 : 2; }
+// resident pass-B CTAs the compiler is held to: 512 threads' worth (16 values per thread)
+__host__ __device__ constexpr int x2_b_min_blocks(int log_l) {
+    return imin_c(16, imax_c(1, 512 / x2_b_threads(log_l)));
+}
 
 template <int LOG_L>
 __global__ void __launch_bounds__(x2_b_threads(LOG_L), x2_b_min_blocks(LOG_L))
 pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restrict__ params, int64_t p0, int log_n2,
-                 int64_t n_samples, const float2* __restrict__ stw, Partial* __restrict__ partials, int64_t ahead) {
+                 int log_ga, int cb_a, int64_t n_samples, const float2* __restrict__ stw, Partial* __restrict__ partials, int64_t ahead) {
     constexpr int L = 1 << LOG_L;
     constexpr int V = shape_v(LOG_L);
     constexpr int G = L / V;
     constexpr int TB = pass_b_tb(LOG_L, 4);
     constexpr int NT = TB * G;
-    constexpr int BUF = fft16_buf_elems(LOG_L);
+    constexpr int BUF = fft_buf_elems<LOG_L, 4, 1, 4>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     c32x2* smem = reinterpret_cast<c32x2*>(smem_raw);
     constexpr int NRED = NT >= 32 ? NT / 32 : NT;
@@ -711,7 +707,7 @@ pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restri
     const int j = threadIdx.x % G;
     const int c = threadIdx.x / G;
     const int n2 = 1 << log_n2;
-    const int ta = blockIdx.x * TB + c;
+    const int row_a = blockIdx.x * TB + c, ta = pass_b_ta(row_a, log_ga, cb_a);
     const int64_t p = blockIdx.y;
     // The rows of the CTA `ahead` places later in launch order (one wave of resident CTAs) are requested
     // into L2 by one bulk prefetch per warp, so that DRAM keeps streaming while the resident CTAs
@@ -732,7 +728,7 @@ pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restri
         }
     }
     if (!params[p0 + p].valid) return;   // the final reduce reports NaN for it
-    const int64_t row0 = ((int64_t)p * n2 + ta) * L;
+    const int64_t row0 = ((int64_t)p * n2 + row_a) * L;
     const c32x2* row = inter + row0;
     c32x2 v[V];
 #pragma unroll
@@ -741,8 +737,9 @@ pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restri
         if (FCAS_CHECK(row0 + j + q * G < (int64_t)gridDim.y * n2 * L, kCheckInterRead))
             v[q] = ld_na(row + j + q * G);   // read once: no L1 allocation (60-min pass B 2.13 -> 2.10 ms)
     }
-    fft16<x2f, +1, LOG_L>(v, smem + c * BUF, 1, j, stw);
-    // Gamma^2(t) = |W_1(t)|^2 + |W_2(t)|^2; t = ta + N2 (j + q G) grows with q, so a strict
+    fftr<x2f, +1, LOG_L, 4, 1, NT, false, false, 4, true>(v, smem + c * BUF, 1, j, stw);
+    const int jo = fft_job<LOG_L, 4, 1>(j);
+    // Gamma^2(t) = |W_1(t)|^2 + |W_2(t)|^2; t = ta + N2 (jo + q G) grows with q, so a strict
     // comparison keeps the lowest t among equal values
     float best = -1.0f;
     int bt = INT_MAX;
@@ -751,7 +748,7 @@ pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restri
     const int ns = n_samples < (int64_t)INT_MAX ? (int)n_samples : INT_MAX;
 #pragma unroll
     for (int q = 0; q < V; ++q) {
-        const int t = ta + n2 * (j + q * G);
+        const int t = ta + n2 * (jo + q * G);
         const float g = norm2_sum(v[q]);
         if (t < ns && g > best) {
             best = g;
@@ -762,7 +759,7 @@ pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restri
 }
 
 // Column-block widths of the packed FP32 pass A: the default of the length and, from 2^8 points on,
-// half and twice it while a CTA stays within 512 threads.
+// half, twice and four times it while a CTA stays within 512 threads.
 template <int LG>
 constexpr bool x2_k1b_ok(int k) {
     return k >= 1 && k <= 16 && k <= (1 << LG) && x2_a_threads(LG, k) <= 512;
@@ -772,23 +769,19 @@ template <int LG, int K1B, int MAXRB = 4>
 static cudaError_t pass_a_x2_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
                                 void* inter, cudaStream_t s) {
     constexpr int THREADS = x2_a_threads(LG, K1B, MAXRB);
-    const size_t smem =
-        (x2_a_pingpong(LG, K1B, MAXRB) ? 2 : 1) * sizeof(c32x2) * (size_t)x2_buf_elems(LG, K1B, MAXRB);
+    const size_t smem = sizeof(c32x2) * (size_t)x2_buf_elems<LG, K1B, MAXRB>();
     auto kern = pass_a_x2_kernel<LG, K1B, MAXRB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t items = np * ((1 << pl.log_n1) / K1B);
-    int64_t ctas = items;
-    if constexpr (!x2_a_pingpong(LG, K1B, MAXRB)) {
-        // one wave: the resident CTAs of every SM
-        int dev = 0, sms = 0, per_sm = 0;
-        e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem);
-        if (e != cudaSuccess) return e;
-        const int64_t wave = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-        if (wave < ctas) ctas = wave;
-    }
+    // one wave: the resident CTAs of every SM
+    int dev = 0, sms = 0, per_sm = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t wave = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+    const int64_t ctas = wave < items ? wave : items;
     kern<<<(unsigned)ctas, THREADS, smem, s>>>(static_cast<const float2*>(pl.y), static_cast<const BasisF*>(pl.basis),
                                                params, p0, np, pl.n_det, pl.log_n1, pl.sub, static_cast<c32x2*>(inter),
                                                static_cast<const float2*>(pl.stw_a), static_cast<const float2*>(pl.tw_lo),
@@ -817,6 +810,8 @@ static cudaError_t pass_a_x2_lg(const FitnessPlan& pl, const ParticleParams* par
             if (pl.k1b == KD / 2) return pass_a_x2_at<LG, (KD / 2 > 0 ? KD / 2 : 1)>(pl, params, p0, np, inter, s);
         if constexpr (x2_k1b_ok<LG>(KD * 2))
             if (pl.k1b == KD * 2) return pass_a_x2_at<LG, (KD * 2 <= 16 ? KD * 2 : 16)>(pl, params, p0, np, inter, s);
+        if constexpr (x2_k1b_ok<LG>(KD * 4))
+            if (pl.k1b == KD * 4) return pass_a_x2_at<LG, (KD * 4 <= 16 ? KD * 4 : 16)>(pl, params, p0, np, inter, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -825,7 +820,7 @@ template <int LG>
 static cudaError_t pass_b_x2_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
                                 const void* inter, Partial* partials, cudaStream_t s) {
     constexpr int TB = pass_b_tb(LG, 4);
-    const size_t smem = sizeof(c32x2) * (size_t)TB * fft16_buf_elems(LG);
+    const size_t smem = sizeof(c32x2) * (size_t)TB * fft_buf_elems<LG, 4, 1, 4>();
     auto kern = pass_b_x2_kernel<LG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -835,8 +830,9 @@ static cudaError_t pass_b_x2_at(const FitnessPlan& pl, const ParticleParams* par
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, x2_b_threads(LG), smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((1 << pl.log_n2) / TB), (unsigned)np);
-    kern<<<grid, x2_b_threads(LG), smem, s>>>(static_cast<const c32x2*>(inter), params, p0, pl.log_n2, pl.n_samples,
-                                              static_cast<const float2*>(pl.stw_b), partials,
+    const int log_ga = fft_log_g(pl.log_n2, pl.radix_bits_a), cb_a = fft_local_bits(pl.log_n2, pl.radix_bits_a, pl.k1b);
+    kern<<<grid, x2_b_threads(LG), smem, s>>>(static_cast<const c32x2*>(inter), params, p0, pl.log_n2, log_ga, cb_a,
+                                              pl.n_samples, static_cast<const float2*>(pl.stw_b), partials,
                                               (int64_t)sms * (per_sm > 0 ? per_sm : 1));
     return cudaGetLastError();
 }
@@ -850,8 +846,7 @@ template <typename Real, int LG, int K1B, int MAXRB = 4>
 static cudaError_t pass_a_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np, void* inter,
                              cudaStream_t s) {
     constexpr int THREADS = K1B * ((1 << LG) / fftr_v(LG, MAXRB));
-    const size_t smem = (pass_a_pingpong<Real, LG, K1B, MAXRB>() ? 2 : 1) * sizeof(cplx<Real>) *
-                        (size_t)pass_a_buf_elems<Real, LG, K1B, MAXRB>();
+    const size_t smem = sizeof(cplx<Real>) * (size_t)pass_a_buf_elems<Real, LG, K1B, MAXRB>();
     auto kern = pass_a_kernel<Real, LG, K1B, MAXRB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -900,7 +895,7 @@ static cudaError_t pass_b_at(const FitnessPlan& pl, const ParticleParams* params
                              const void* inter, Partial* partials, cudaStream_t s) {
     constexpr int TB = pass_b_tb(LG, sizeof(Real));
     constexpr int THREADS = pass_b_threads(LG, sizeof(Real));
-    const size_t smem = sizeof(cplx<Real>) * (size_t)TB * fft16_buf_elems(LG);
+    const size_t smem = sizeof(cplx<Real>) * (size_t)TB * fft_buf_elems<LG, 4, 0, 4>();
     auto kern = pass_b_kernel<Real, LG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
