@@ -99,7 +99,7 @@ namespace {
 void free_ctx(fcas_ctx* c) {
     void* ptrs[] = {c->d_det, c->d_sigma2s, c->d_y, c->d_basis, c->d_tw64, c->d_twlo64, c->d_twhi64,
                     c->d_tw32, c->d_twlo32, c->d_twhi32, c->d_stw_a64, c->d_stw_a32, c->d_stw_b64, c->d_stw_b32,
-                    c->d_twloff, c->d_twhiff, c->d_stw_aff, c->d_stw_bff, c->d_phff,
+                    c->d_twloff, c->d_twhiff, c->d_stw_aff, c->d_stw_bff, c->d_phtab,
                     c->d_params, c->d_theta, c->d_fit, c->d_tc, c->d_inter, c->d_partials, c->d_pso,
                     c->d_gsums, c->d_gstage, c->d_ynat, c->d_polish};
     for (void* p : ptrs)
@@ -237,7 +237,7 @@ int ensure_grad(fcas_ctx* c, int64_t n) {
 cudaError_t gradient_device(fcas_ctx* c, int64_t n, const double* d_theta, const int64_t* d_tc, double* d_grad,
                             cudaStream_t st) {
     const cudaError_t e = launch_geometry(d_theta, n, c->d_params, c->d_det, c->d_sigma2s, c->setup.n_det,
-                                          c->setup.f_low, c->df, pass_a_kstep(c), st);
+                                          c->setup.f_low, c->df, pass_a_kstep(c), c->setup.precision, st);
     if (e != cudaSuccess) return e;
     return launch_gradient(make_plan(c), c->setup.precision, c->k_lo, c->k_hi, c->d_params, d_theta, d_tc, n,
                            c->d_gsums, c->d_det, c->d_sigma2s, c->setup.f_low, c->df, d_grad, st);
@@ -501,8 +501,10 @@ int create_impl(fcas_ctx** out, const fcas_setup* setup, const fcas_detector* de
         FCAS_TRY(dev_alloc(&c->d_stw_bff, sizeof(double2) << kMaxLogPass, "float-float stage twiddles"));
         FCAS_TRYCUDA(launch_split_ff(c->d_twlo64, c->d_twloff, (int64_t)nlo, st));
         FCAS_TRYCUDA(launch_split_ff(c->d_twhi64, c->d_twhiff, (int64_t)nhi, st));
-        FCAS_TRY(dev_alloc(&c->d_phff, sizeof(double2) * 1024, "float-float phasor table"));
-        FCAS_TRYCUDA(launch_phase_table_ff(c->d_phff, 1024, st));
+    }
+    if (!fp32) {
+        FCAS_TRY(dev_alloc(&c->d_phtab, sizeof(double2) * 1024, "phasor table"));
+        FCAS_TRYCUDA(launch_phase_table(c->d_phtab, 1024, s.precision == FCAS_PREC_FF, st));
     }
 
     // forward FFT of the data (binary64) and the whitened, re-laid-out band spectrum
@@ -589,7 +591,7 @@ int fcas_fitness(fcas_ctx* c, int64_t n, const double* theta, double* fitness, i
     size_t slot;
     prof_begin(c, FCAS_KERNEL_GEOMETRY, st, &slot);
     FCAS_CUDA(launch_geometry(d_theta, n, c->d_params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low, c->df,
-                              pass_a_kstep(c), st));
+                              pass_a_kstep(c), c->setup.precision, st));
     prof_end(c, slot, st);
     FCAS_CUDA(launch_passes(c, n, d_fit, d_tc, st));
     if (!f_dev) FCAS_CUDA(cudaMemcpyAsync(fitness, d_fit, sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost, st));
@@ -647,7 +649,7 @@ cudaError_t swarm_iteration(fcas_ctx* c, const PsoDev& g, const Swarm& w, Partic
     cudaError_t x = launch_pso_theta(g, w.s, w.theta, st);
     if (x == cudaSuccess)
         x = launch_geometry(w.theta, rows, params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low, c->df,
-                            pass_a_kstep(c), st);
+                            pass_a_kstep(c), c->setup.precision, st);
     if (x == cudaSuccess) x = launch_passes_with(c, params, inter, partials, chunk, rows, w.fit, w.tcs, st);
     if (x == cudaSuccess) x = launch_pso_update(g, 0, w.fit, w.tcs, w.s, st);
     return x;
@@ -776,7 +778,7 @@ int fcas_autotune(fcas_ctx* c, int64_t n_particles, const char* cache_path, void
     }
     FCAS_CUDA(cudaMemcpyAsync(c->d_theta, th.data(), sizeof(double) * th.size(), cudaMemcpyHostToDevice, st));
     FCAS_CUDA(launch_geometry(c->d_theta, n_particles, c->d_params, c->d_det, c->d_sigma2s, c->setup.n_det,
-                              c->setup.f_low, c->df, pass_a_kstep(c), st));
+                              c->setup.f_low, c->df, pass_a_kstep(c), c->setup.precision, st));
     cudaEvent_t e0, e1;
     FCAS_CUDA(cudaEventCreate(&e0));
     FCAS_CUDA(cudaEventCreate(&e1));
@@ -1112,7 +1114,7 @@ int fcas_polish(fcas_ctx* c, int64_t n, double* theta, double* fitness, int64_t*
     FCAS_CUDA(cudaMemsetAsync(w_acc, 0, sizeof(int32_t) * (size_t)n, st));
     // the fitness at the starting points
     FCAS_CUDA(launch_geometry(w_th, n, c->d_params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low, c->df,
-                              pass_a_kstep(c), st));
+                              pass_a_kstep(c), c->setup.precision, st));
     FCAS_CUDA(launch_passes(c, n, w_fit, w_tc, st));
     for (int32_t step = 0; step < steps; ++step) {
         FCAS_CUDA(gradient_device(c, n, w_th, w_tc, w_grad, st));
@@ -1121,7 +1123,7 @@ int fcas_polish(fcas_ctx* c, int64_t n, double* theta, double* fitness, int64_t*
             FCAS_CUDA(cudaMemsetAsync(w_searching, 0, sizeof(int32_t), st));
             FCAS_CUDA(launch_polish_candidate(w_th, w_dir, w_step, w_done, n, w_cand, st));
             FCAS_CUDA(launch_geometry(w_cand, n, c->d_params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low,
-                                      c->df, pass_a_kstep(c), st));
+                                      c->df, pass_a_kstep(c), c->setup.precision, st));
             FCAS_CUDA(launch_passes(c, n, w_cfit, w_ctc, st));
             FCAS_CUDA(launch_polish_accept(w_th, w_fit, w_tc, w_cand, w_cfit, w_ctc, w_step, w_done, w_acc, n,
                                            w_searching, st));

@@ -86,18 +86,18 @@ __global__ void split_ff_kernel(const double2* __restrict__ src, float4* __restr
     }
 }
 
-__global__ void phase_table_ff_kernel(float4* __restrict__ dst, int n) {
+__global__ void phase_table_kernel(void* __restrict__ dst, int n, bool ff) {
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n; m += gridDim.x * blockDim.x) {
         double sn, cs;
         sincospi(2.0 * (double)m / (double)n, &sn, &cs);
         const float xh = (float)cs, yh = (float)sn;
-        dst[m] = make_float4(xh, (float)(cs - (double)xh), yh, (float)(sn - (double)yh));
+        if (ff) static_cast<float4*>(dst)[m] = make_float4(xh, (float)(cs - (double)xh), yh, (float)(sn - (double)yh));
+        else static_cast<double2*>(dst)[m] = make_double2(cs, sn);
     }
 }
-
-cudaError_t launch_phase_table_ff(void* dst, int n, cudaStream_t s) {
+cudaError_t launch_phase_table(void* dst, int n, bool ff, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    phase_table_ff_kernel<<<(n + 255) / 256, 256, 0, s>>>(static_cast<float4*>(dst), n);
+    phase_table_kernel<<<(n + 255) / 256, 256, 0, s>>>(dst, n, ff);
     return cudaGetLastError();
 }
 

@@ -126,9 +126,18 @@ __device__ __forceinline__ bool index_check(bool ok, int bit) {
 enum IndexCheck { kCheckExchangeRead = 0, kCheckExchangeWrite = 1, kCheckTwiddle = 2, kCheckSpectrum = 3,
                   kCheckBasis = 4, kCheckInterWrite = 5, kCheckInterRead = 6 };
 
+// first-layer sums of a four-point transform: float-float ones stay unnormalised pairs, normalised by the
+// second layer (8 instructions instead of 11)
+template <typename C> __device__ __forceinline__ C add_in(C a, C b) { return a + b; }
+template <typename C> __device__ __forceinline__ C sub_in(C a, C b) { return a - b; }
+__device__ __forceinline__ ff2 add_in(ff2 a, ff2 b) { return ff2{ff_add_pair(a.x, b.x), ff_add_pair(a.y, b.y)}; }
+__device__ __forceinline__ ff2 sub_in(ff2 a, ff2 b) {
+    return ff2{ff_add_pair(a.x, ff_neg(b.x)), ff_add_pair(a.y, ff_neg(b.y))};
+}
+
 template <int S, typename C>
 __device__ __forceinline__ void r16_dft4(C& a0, C& a1, C& a2, C& a3) {
-    C t0 = a0 + a2, t1 = a0 - a2, t2 = a1 + a3, t3 = a1 - a3;
+    C t0 = add_in(a0, a2), t1 = sub_in(a0, a2), t2 = add_in(a1, a3), t3 = sub_in(a1, a3);
     a0 = t0 + t2;
     a2 = t0 - t2;
     a1 = add_si<S>(t1, t3);
@@ -329,7 +338,8 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
                            : NS >= G                ? jr + h * G
                                                     : (jr >> (LG - CB)) * (NS >> CB) + (jr & ((NS >> CB) - 1));
             const W* t = stw + (NS - 1) + jm;
-            if constexpr (R >= 8 && TWL && !std::is_same<Real, ffloat>::value) {
+            constexpr bool kLoadAll = std::is_same<Real, ffloat>::value || std::is_same<Real, double>::value;
+            if constexpr (R >= 8 && TWL && !kLoadAll) {
                 W wl[4], wh[R / 4];
                 wl[0] = wh[0] = tw_one(W{});
 #pragma unroll
@@ -353,10 +363,10 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
 #pragma unroll
                     for (int r = 1; r < 4; ++r) a[4 * hi + r] = cmul(a[4 * hi + r], cmul(wh[hi], wl[r]));
                 }
-            } else if constexpr (R >= 8 && !std::is_same<Real, ffloat>::value) {
+            } else if constexpr (R >= 8 && !kLoadAll) {
                 // w^r for r = 1..R-1 from two table entries: w and w^4 (powers by products, <= 3 roundings);
-                // the float-float form loads every power instead (a double-word product costs more
-                // than a load)
+                // the binary64 and float-float forms load every power instead (a product costs more than
+                // a load there: binary64 60-min pass B 5.82 -> 5.05 ms per 4 particles)
                 W w1 = tw_one(W{}), w4 = w1;
                 if (FCAS_CHECK((NS - 1) + jm + 3 * NS < L, kCheckTwiddle)) {
                     w1 = ldg_c(t);

@@ -63,6 +63,10 @@ struct ParticleParams {
     float w1f[FCAS_MAX_DET], w2f[FCAS_MAX_DET];
     float2 dstep[FCAS_MAX_DET];    // e^{2 pi i S Delta^i df}, S = N / V_A: the FP32 pass A's step of the
                                    // delay phasor between a thread's consecutive bins (binary64 phase)
+    // binary64 and float-float pass A: delays relative to detector 0's (whose own phase joins the chirp
+    // phase) and the phasor of the same step, e^{2 pi i S rturn}; filled for those forms only
+    double rturn[FCAS_MAX_DET];
+    double2 rstep[FCAS_MAX_DET];
     int32_t valid;                 // 0: non-finite / non-positive input -> fitness NaN, tc -1
     int32_t taylor_ok;             // FP32 pass A may step the chirp phase from an anchor bin to the
                                    // next 3 (bit 0) or 7 (bit 1) bins: remainder below 1e-7 turns
@@ -81,33 +85,30 @@ __host__ __device__ constexpr int imax_c(int a, int b) { return a > b ? a : b; }
 #ifndef FCAS_SPLIT_BIAS
 #define FCAS_SPLIT_BIAS 0             // N2 = 2^(floor(log2 N / 2) - bias): a smaller pass-A transform
 #endif
-#ifndef FCAS_PASS_B_THREADS_F32
-#define FCAS_PASS_B_THREADS_F32 64    // target CTA size of pass B, FP32 form
-#endif
 __host__ __device__ constexpr int shape_v(int log_l) { return log_l >= 4 ? 16 : (1 << log_l); }
-// Columns per pass-A CTA. FP32: CTAs of 128 threads, but at least 4 columns (row pieces of 64 bytes; 2 columns
-// write 32-byte pieces and lose 12 % at 2^11 points) while a CTA stays within 512 threads. Several small CTAs
-// per SM are in different phases (loads, arithmetic, exchanges) at any time, one large one is in the same
-// phase throughout: us per 64 particles with 4 / 8 / 16 columns, 2^8 points 28.2 / 27.4 / 29.6, 2^9 points
-// 101 / 110 / 121, 2^10 points 778 / 827 / -.
-__host__ __device__ constexpr int pass_a_k1b(int log_l, int real_bytes) {
+// Columns per pass-A CTA of a form (FCAS_PREC_*). FP32: CTAs of 128 threads, but at least 4 columns (row pieces
+// of 64 bytes; 2 columns write 32-byte pieces and lose 12 % at 2^11 points) while a CTA stays within 512
+// threads. Several small CTAs per SM are in different phases (loads, arithmetic, exchanges) at any time, one
+// large one is in the same phase throughout: us per 64 particles with 4 / 8 / 16 columns, 2^8 points 28.2 /
+// 27.4 / 29.6, 2^9 points 101 / 110 / 121, 2^10 points 778 / 827 / -. Binary64: 128 threads for the same reason
+// (2^8 points, 40 particles: 8 / 16 columns 463 / 520 us; 2^11 points, 4 particles: 1 / 2 columns 6.78 / 6.92
+// ms). Float-float: 256 threads, whose warps share the instruction fetches of its long unrolled code.
+__host__ __device__ constexpr int pass_a_k1b(int log_l, int form) {
     const int g = (1 << log_l) / shape_v(log_l);   // threads per column
-    const int k = real_bytes == 4 ? imax_c(128 / g, imin_c(4, 512 / g)) : 256 / g;
+    const int k = form == FCAS_PREC_FP32 ? imax_c(128 / g, imin_c(4, 512 / g)) : (form == FCAS_PREC_FP64 ? 128 : 256) / g;
     return imin_c(imin_c(16, imax_c(1, k)), 1 << log_l);
 }
-__host__ __device__ constexpr int pass_a_threads(int log_l, int real_bytes) {
-    return pass_a_k1b(log_l, real_bytes) * ((1 << log_l) / shape_v(log_l));
+// Threads a pass-B CTA holds where rows are shorter: FP32 64 (us per 64 particles with CTAs of 256 / 128 / 64
+// threads: 2^8 points 19.9 / 17.3 / 16.8, 2^9 points 80 / 76 / 75, 2^11 points 469 / 411 / 411), binary64 128,
+// float-float 256 (2^11 points, 16 particles: 128 / 256 threads 1076 / 929 us; shared instruction fetches).
+__host__ __device__ constexpr int pass_b_target(int form) {
+    return form == FCAS_PREC_FP32 ? 64 : form == FCAS_PREC_FP64 ? 128 : 256;
 }
-// Rows per pass-B CTA. FP32: one row where a row takes 64 threads or more, for the same reason: us per 64
-// particles with CTAs of 256 / 128 / 64 threads, 2^8 points 19.9 / 17.3 / 16.8, 2^9 points 80 / 76 / 75, 2^11
-// points 469 / 411 / 411.
-__host__ __device__ constexpr int pass_b_tb(int log_l, int real_bytes) {
-    return imin_c(imin_c(16, imax_c(1, (real_bytes == 4 ? FCAS_PASS_B_THREADS_F32 : 128) /
-                                           ((1 << log_l) / shape_v(log_l)))),
-                  (1 << log_l) / 2);
+__host__ __device__ constexpr int pass_b_tb(int log_l, int form) {
+    return imin_c(imin_c(16, imax_c(1, pass_b_target(form) / ((1 << log_l) / shape_v(log_l)))), (1 << log_l) / 2);
 }
-__host__ __device__ constexpr int pass_b_threads(int log_l, int real_bytes) {
-    return pass_b_tb(log_l, real_bytes) * ((1 << log_l) / shape_v(log_l));
+__host__ __device__ constexpr int pass_b_threads(int log_l, int form) {
+    return pass_b_tb(log_l, form) * ((1 << log_l) / shape_v(log_l));
 }
 // Transforms per particle between the passes: the two network-weighted series.
 constexpr int kSeries = 2;

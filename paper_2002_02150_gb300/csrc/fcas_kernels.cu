@@ -50,7 +50,7 @@ constexpr int kGeomParticles = 32 / kGeomLanes;     // particles per warp
 __global__ void __launch_bounds__(64)
 geometry_kernel(const double* __restrict__ theta, int64_t n, ParticleParams* __restrict__ out,
                 const double* __restrict__ det9, const double* __restrict__ s2, int n_det, double f_star, double df,
-                int64_t kstep, TaylorBound tb) {
+                int64_t kstep, bool wide, TaylorBound tb) {
     const int lane = threadIdx.x & 31, sub = lane % kGeomLanes, lane0 = lane - sub;
     const int64_t p = (int64_t)blockIdx.x * kGeomParticles + lane / kGeomLanes;
     const bool have = p < n;
@@ -163,6 +163,18 @@ geometry_kernel(const double* __restrict__ theta, int64_t n, ParticleParams* __r
     us -= rint(us);
     double su, cu;
     sincospi(2.0 * us, &su, &cu);
+    if (wide) {
+        const double d0 = __shfl_sync(0xffffffffu, dturn, lane0);
+        const double rel = det_lane ? dturn - d0 : 0.0;
+        double ur = (double)kstep * rel;
+        ur -= rint(ur);
+        double sr, cr;
+        sincospi(2.0 * ur, &sr, &cr);
+        if (have) {
+            pp->rturn[sub] = rel;
+            pp->rstep[sub] = make_double2(cr, sr);
+        }
+    }
     if (!have) return;
     pp->dturn[sub] = dturn;
     pp->u[sub][0] = fp;
@@ -184,11 +196,11 @@ geometry_kernel(const double* __restrict__ theta, int64_t n, ParticleParams* __r
 
 cudaError_t launch_geometry(const double* theta, int64_t n, ParticleParams* out, const double* det9,
                             const double* sigma2_scaled, int n_det, double f_star, double df, int64_t kstep,
-                            cudaStream_t s) {
+                            int precision, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int64_t blocks = (n + kGeomParticles - 1) / kGeomParticles;
     geometry_kernel<<<(unsigned)blocks, 64, 0, s>>>(theta, n, out, det9, sigma2_scaled, n_det, f_star, df, kstep,
-                                                    taylor_bound(f_star, df));
+                                                    precision != FCAS_PREC_FP32, taylor_bound(f_star, df));
     return cudaGetLastError();
 }
 
@@ -236,24 +248,9 @@ cudaError_t launch_reduce(const Partial* partials, int64_t nb, const ParticlePar
 // ------------------------------------------------------------------------------------------
 // shape helpers of the passes
 // ------------------------------------------------------------------------------------------
-int pass_a_k1b_for(int log_n2, int precision) {
-    const int rb = precision == FCAS_PREC_FP32 ? 4 : 8;
-    switch (log_n2) {
-#define FCAS_CASE(LG) case LG: return pass_a_k1b(LG, rb);
-        FCAS_LOG_CASES(FCAS_CASE)
-#undef FCAS_CASE
-        default: return -1;
-    }
-}
-
 int pass_b_blocks_per_particle(int log_n1, int log_n2, int precision) {
-    const bool fp32 = precision == FCAS_PREC_FP32;
-    switch (log_n1) {
-#define FCAS_CASE(LG) case LG: return (1 << log_n2) / pass_b_tb(LG, fp32 ? 4 : 8);
-        FCAS_LOG_CASES(FCAS_CASE)
-#undef FCAS_CASE
-        default: return -1;
-    }
+    if (log_n1 < 2 || log_n1 > kMaxLogPass) return -1;
+    return (1 << log_n2) / pass_b_tb(log_n1, precision);
 }
 
 bool pass_a_radix8_available(int log_n2, int precision, int k1b) {
@@ -267,25 +264,18 @@ int pass_a_default_radix_bits(int log_n2, int precision) {
 }
 
 int pass_a_k1b_variants(int log_n2, int precision, int* out) {
-    const int rb = precision == FCAS_PREC_FP32 ? 4 : 8;
+    if (log_n2 < 2 || log_n2 > kMaxLogPass) return 0;
+    const int kd = pass_a_k1b(log_n2, precision);
     int n = 0;
-    switch (log_n2) {
-#define FCAS_CASE(LG)                                                                       \
-    case LG: {                                                                              \
-        const int kd = pass_a_k1b(LG, rb);                                                  \
-        out[n++] = kd;                                                                      \
-        if (rb == 4 && LG >= 8) {                                                           \
-            if (x2_k1b_ok<LG>(kd / 2)) out[n++] = kd / 2;                                   \
-            if (x2_k1b_ok<LG>(kd * 2)) out[n++] = kd * 2;                                   \
-            if (x2_k1b_ok<LG>(kd * 4)) out[n++] = kd * 4;                                   \
-            if (LG >= 10 && kd / 2 > 1) out[n++] = 1;                                       \
-        }                                                                                   \
-        return n;                                                                           \
+    out[n++] = kd;
+    if (log_n2 >= 8 && precision == FCAS_PREC_FP32) {
+        if (x2_k1b_ok(log_n2, kd / 2)) out[n++] = kd / 2;
+        if (x2_k1b_ok(log_n2, kd * 2)) out[n++] = kd * 2;
+        if (x2_k1b_ok(log_n2, kd * 4)) out[n++] = kd * 4;
+        if (log_n2 >= 10 && kd / 2 > 1) out[n++] = 1;
     }
-        FCAS_LOG_CASES(FCAS_CASE)
-#undef FCAS_CASE
-        default: return 0;
-    }
+    if (precision == FCAS_PREC_FP64 && fp64_k1b_double(log_n2)) out[n++] = kd * 2;
+    return n;
 }
 
 template cudaError_t launch_pass_a<float>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, void*, cudaStream_t);

@@ -102,14 +102,14 @@ struct FitnessPlan {
     int sub;                      // adjacent column blocks of a particle scheduled together
     const void* tw_lo;            // e^{2 pi i m / N}, m < 4096
     const void* tw_hi;            // e^{2 pi i 4096 m / N}, m < max(1, N / 4096)
-    const void* ptab;             // float-float e^{2 pi i m / 1024}, m < 1024 (FCAS_PREC_FF only)
+    const void* ptab;             // e^{2 pi i m / 1024}, m < 1024 (binary64 and float-float forms)
 };
 
 // Per-particle geometry (binary64): chirp coefficients, delays, antenna patterns, G^-1.
 // kstep: the bin step between a pass-A thread's consecutive values (N / V_A, pass_a_kstep).
 cudaError_t launch_geometry(const double* theta, int64_t n, ParticleParams* out, const double* det9,
                             const double* sigma2_scaled, int n_det, double f_star, double df, int64_t kstep,
-                            cudaStream_t s);
+                            int precision, cudaStream_t s);
 
 // Pass A for particles [p0, p0 + np): writes the intermediate [np][2][N2][N1].
 template <typename Real>
@@ -129,10 +129,9 @@ int pass_b_blocks_per_particle(int log_n1, int log_n2, int precision);
 unsigned int take_index_checks(cudaStream_t s);
 // float-float copy (16-byte entries: hi/lo of re, hi/lo of im) of a binary64 complex table
 cudaError_t launch_split_ff(const double2* src, void* dst, int64_t n, cudaStream_t s);
-// float-float table of e^{2 pi i m / n}, m < n (16-byte entries as above)
-cudaError_t launch_phase_table_ff(void* dst, int n, cudaStream_t s);
+// table of e^{2 pi i m / n}, m < n, in binary64 or float-float (16-byte entries as above)
+cudaError_t launch_phase_table(void* dst, int n, bool ff, cudaStream_t s);
 unsigned int take_index_checks_ff(cudaStream_t s);   // the float-float passes' translation unit
-int pass_a_k1b_for(int log_n2, int precision);
 // compiled pass-A column-block widths (radix-16 stages) for a length: writes up to 5 values, returns the count
 int pass_a_k1b_variants(int log_n2, int precision, int* out);
 // per-stage twiddles of length-2^log_l transforms, in the order of threads shared by k columns (0: jm's own)

@@ -26,11 +26,9 @@ namespace fcas {
 // Phase of Q_i[k] = Y_i[k] e^{2 pi i (psi(f_k)/2pi + f_k Delta^i)} (Sec. II.B, eq. data_template_innprod)
 // ------------------------------------------------------------------------------------------
 
-__device__ __forceinline__ float round_nearest(float x) { return rintf(x); }
-__device__ __forceinline__ double round_nearest(double x) { return rint(x); }
-
-__device__ __forceinline__ double chirp_frac(const BasisD& b, const ParticleParams& pp) {
-    double s = pp.c[0] * b.a.x + pp.c[1] * b.a.y + pp.c[2] * b.b.x + pp.c[3] * b.b.y;
+// chirp phase [turns] of a bin, reduced by an integer
+__device__ __forceinline__ double chirp_frac(const BasisD& b, const double* c) {
+    double s = c[0] * b.a.x + c[1] * b.a.y + c[2] * b.b.x + c[3] * b.b.y;
     return s - rint(s);
 }
 
@@ -42,18 +40,7 @@ __device__ __forceinline__ float2 fast_phasor(float turns) {
     return make_float2(cs, sn);
 }
 
-__device__ __forceinline__ float2 unit_phasor(float turns) {
-    float sn, cs;
-    sincospif(2.0f * turns, &sn, &cs);
-    return make_float2(cs, sn);
-}
-__device__ __forceinline__ double2 unit_phasor(double turns) {
-    double sn, cs;
-    sincospi(2.0 * turns, &sn, &cs);
-    return make_double2(cs, sn);
-}
-
-// Entries of the float-float phasor table: e^{2 pi i m / kPhaseTab}, m < kPhaseTab.
+// Entries of the phasor table of the binary64 and float-float forms: e^{2 pi i m / kPhaseTab}, m < kPhaseTab.
 constexpr int kPhaseTabBits = 10;
 constexpr int kPhaseTab = 1 << kPhaseTabBits;
 
@@ -82,9 +69,22 @@ __device__ __forceinline__ ff2 ff_unit_phasor(ffloat u, const ff2* __restrict__ 
     const ff2 t = ldg_c(tab + ((int)m & (kPhaseTab - 1)));
     return cmul(t, ff2{ffloat(c, cl), sn});
 }
-__device__ __forceinline__ ff2 ff_unit_phasor(double u, const ff2* __restrict__ tab) {
+__device__ __forceinline__ ff2 unit_phasor(double u, const ff2* __restrict__ tab) {   // |u| <= 1/2
     const float uh = __double2float_rn(u);
     return ff_unit_phasor(ffloat(uh, __double2float_rn(u - (double)uh)), tab);
+}
+// e^{2 pi i u} in binary64 for |u| < 2^30, by the same reduction: the nearest table point m from adding
+// 1.5 2^52 (the low word of the sum is m), the remainder exact, cos x and sin x to x^4 and x^5 (the first
+// omitted terms are below 2e-18). 14 binary64 instructions; sincospi took about three times as many, and
+// the binary64 unit is what the binary64 form waits for.
+__device__ __forceinline__ double2 unit_phasor(double u, const double2* __restrict__ tab) {
+    constexpr double kMagic = 6755399441055744.0;   // 1.5 2^52
+    const double t = fma(u, (double)kPhaseTab, kMagic);
+    const double x = fma(t - kMagic, -1.0 / (double)kPhaseTab, u) * kTwoPi;
+    const double x2 = x * x;
+    const double sn = fma(x * x2, fma(x2, 1.0 / 120.0, -1.0 / 6.0), x);
+    const double cs = fma(x2, fma(x2, 1.0 / 24.0, -0.5), 1.0);
+    return cmul(__ldg(tab + (__double2loint(t) & (kPhaseTab - 1))), make_double2(cs, sn));
 }
 
 // frac(k d) in float-float for an integer 0 <= k < 2^24 and d = d1 + d2 + d3 (three floats, each
@@ -123,35 +123,85 @@ __host__ __device__ constexpr int pass_a_buf_elems() {
     return K1B * fft_buf_elems<LOG_L, MAXRB, 0, pass_a_pad_shift<Real, MAXRB>()>();
 }
 
-// The float-float form reduces the chirp phase in binary64 (basis as in the binary64 form) and the
-// delay phase from a three-float split of the delay, and forms the phasors, the detector sums and
-// everything after them in float-float.
-template <typename Real> struct phase_of { using type = Real; };
-template <> struct phase_of<ffloat> { using type = double; };
-template <typename Real> using phase_t = typename phase_of<Real>::type;
-
 // streamed store (evict-first): the intermediate is read back only by pass B
-__device__ __forceinline__ void st_stream(float2* p, float2 v) { __stcs(p, v); }
 __device__ __forceinline__ void st_stream(double2* p, double2 v) { __stcs(p, v); }
 __device__ __forceinline__ void st_stream(ff2* p, ff2 v) {
     __stcs(reinterpret_cast<float4*>(p), make_float4(v.x.h, v.x.l, v.y.h, v.y.l));
 }
 
+// a x + y and the next value of a three-term recurrence, c2 b - a per component
+__device__ __forceinline__ double axpy(double a, double x, double y) { return fma(a, x, y); }
+__device__ __forceinline__ ffloat axpy(ffloat a, ffloat x, ffloat y) { return ff_fma(a, x, y); }
+template <typename Real>
+__device__ __forceinline__ cplx<Real> three_term(Real c2, cplx<Real> b, cplx<Real> a) {
+    return mkc(axpy(c2, b.x, -a.x), axpy(c2, b.y, -a.y));
+}
+__device__ __forceinline__ double twice(double a) { return 2.0 * a; }
+__device__ __forceinline__ ffloat twice(ffloat a) { return ffloat(2.0f * a.h, 2.0f * a.l); }
+
+// N phasors e^{i (phi + q theta)}, q = 0..N-1, given to use(q, phasor): at_mid = e^{i (phi + (N/2 - 1) theta)}
+// and one product give the two middle ones, the others follow outwards by p(q +- 1) = 2 cos(theta) p(q) -
+// p(q -+ 1), half the arithmetic of a product each. The recurrence loses at most N/2 + 1 units of rounding
+// over its N/2 - 1 steps, as many as N - 1 products in a row.
+template <typename Real, int N, typename F>
+__device__ __forceinline__ void phasor_run(cplx<Real> at_mid, cplx<Real> step, F&& use) {
+    using C = cplx<Real>;
+    if constexpr (N >= 4) {
+        constexpr int M = N / 2;
+        const Real c2 = twice(step.x);
+        const C up = cmul(at_mid, step);
+        use(M - 1, at_mid);
+        use(M, up);
+        C a = at_mid, b = up;
+#pragma unroll
+        for (int q = M + 1; q < N; ++q) {
+            const C n = three_term<Real>(c2, b, a);
+            use(q, n);
+            a = b;
+            b = n;
+        }
+        a = up;
+        b = at_mid;
+#pragma unroll
+        for (int q = M - 2; q >= 0; --q) {
+            const C n = three_term<Real>(c2, b, a);
+            use(q, n);
+            a = b;
+            b = n;
+        }
+    } else {
+        C w = at_mid;   // N / 2 - 1 = 0, or N = 1
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            use(q, w);
+            if (q + 1 < N) w = cmul(w, step);
+        }
+    }
+}
+__host__ __device__ constexpr int phasor_mid(int n) { return n >= 4 ? n / 2 - 1 : 0; }
+
 template <typename Real>
 struct DetConst {
-    phase_t<Real> dh[FCAS_MAX_DET], dl[FCAS_MAX_DET];
+    double rturn[FCAS_MAX_DET];          // delay relative to detector 0's [turns per bin]
+    cplx<Real> step[FCAS_MAX_DET];       // its phasor over a thread's bin step
     Real w1[FCAS_MAX_DET], w2[FCAS_MAX_DET];
 };
 
+// Pass A of the binary64 and float-float forms. The binary64 form waits for the binary64 unit alone (two
+// lanes per SM and clock), the float-float form for FP32 issue and instruction fetch: both follow the number
+// of real operations. Detector 0 needs no phasor (its delay joins the chirp phase), phasors along a thread's
+// bins and outputs come from three-term recurrences, accurate phasors from a table, the step phasors from
+// the geometry kernel: binary64 60-min pass A 9.15 -> 6.78 ms per 4 particles (with 128-thread CTAs), 64-s
+// 704 -> 463 us per 40; float-float 4.00 -> 3.63 ms per 8 particles of the 60-min workload, 15-min 2.69 ->
+// 1.86 ms per 16; errors against the oracle unchanged.
 template <typename Real, int LOG_L, int K1B, int MAXRB>
 __global__ void __launch_bounds__(K1B * ((1 << LOG_L) / fftr_v(LOG_L, MAXRB)), 1)
-pass_a_kernel(const cplx<Real>* __restrict__ y, const Basis<phase_t<Real>>* __restrict__ basis,
+pass_a_kernel(const cplx<Real>* __restrict__ y, const BasisD* __restrict__ basis,
               const ParticleParams* __restrict__ params, int64_t p0, int64_t np, int n_det, int log_n1, int sub_req,
               cplx<Real>* __restrict__ out, const cplx<Real>* __restrict__ stw,
               const cplx<Real>* __restrict__ tw_lo, const cplx<Real>* __restrict__ tw_hi,
               const cplx<Real>* __restrict__ ptab) {
     using C = cplx<Real>;
-    using P = phase_t<Real>;      // the real type of the phase reduction (binary64 for the float-float form)
     constexpr bool kFF = std::is_same<Real, ffloat>::value;
     constexpr int L = 1 << LOG_L;
     constexpr int V = fftr_v(LOG_L, MAXRB);
@@ -160,7 +210,7 @@ pass_a_kernel(const cplx<Real>* __restrict__ y, const Basis<phase_t<Real>>* __re
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* smem = reinterpret_cast<C*>(smem_raw);
     __shared__ DetConst<Real> sc;
-    __shared__ float dsplit[3][FCAS_MAX_DET];   // float-float form: Delta^i df as three floats
+    __shared__ float dsplit[3][FCAS_MAX_DET];   // float-float form: the relative delay as three floats
 
     const int c = threadIdx.x % K1B;
     const int j = threadIdx.x / K1B;
@@ -177,138 +227,93 @@ pass_a_kernel(const cplx<Real>* __restrict__ y, const Basis<phase_t<Real>>* __re
     const int k1 = blk * K1B + c;
     const ParticleParams* pp = params + p0 + p;
     if (!pp->valid) return;   // not evaluated (invalid input, or a PSO particle outside its box)
-    if (threadIdx.x < FCAS_MAX_DET) {
-        const int i = threadIdx.x;
-        if constexpr (sizeof(P) == 4) {
-            sc.dh[i] = pp->dh[i];
-            sc.dl[i] = pp->dl[i];
-            sc.w1[i] = pp->w1f[i];
-            sc.w2[i] = pp->w2f[i];
-        } else {
-            sc.dh[i] = pp->dturn[i];
-            sc.dl[i] = 0.0;
-            sc.w1[i] = Real(pp->w1[i]);
-            sc.w2[i] = Real(pp->w2[i]);
-            if constexpr (kFF) {
-                const double d = pp->dturn[i];
-                const float d1 = (float)d;
-                const float d2 = (float)(d - (double)d1);
-                dsplit[0][i] = d1;
-                dsplit[1][i] = d2;
-                dsplit[2][i] = (float)(d - (double)d1 - (double)d2);
-            }
+    // (CTAs of fewer than 8 threads fill the constants in turns)
+    for (int i = threadIdx.x; i < FCAS_MAX_DET; i += blockDim.x) {
+        const double d = pp->rturn[i];
+        const double2 st = pp->rstep[i];
+        sc.rturn[i] = d;
+        sc.step[i] = mkc(Real(st.x), Real(st.y));
+        sc.w1[i] = Real(pp->w1[i]);
+        sc.w2[i] = Real(pp->w2[i]);
+        if constexpr (kFF) {
+            const float d1 = (float)d;
+            const float d2 = (float)(d - (double)d1);
+            dsplit[0][i] = d1;
+            dsplit[1][i] = d2;
+            dsplit[2][i] = (float)(d - (double)d1 - (double)d2);
         }
     }
     __syncthreads();
     const int n1 = 1 << log_n1;
 
-    // Thread (c, j) owns the bins k = k1 + N1 (j + q G), q < VH. The delay phasors e^{2 pi i k Delta^i / T}
-    // of consecutive q differ by the constant factor e^{2 pi i N1 G Delta^i / T}: one accurate phasor
-    // and one step per detector, then products. The chirp phasor multiplies the detector sums last:
-    // P_a[k] = e^{i psi(f_k)} sum_i w_a,i Y_i[k] e^{2 pi i f_k Delta^i}.
-    C r1[VH], r2[VH];
-#pragma unroll
-    for (int q = 0; q < VH; ++q) r1[q] = r2[q] = mkc(Real(0.0f), Real(0.0f));
-    // the chirp basis of the thread's bins is requested first: its latency overlaps the detector sums
-    const Basis<P>* bb = basis + ((int64_t)blk * (L / 2) + j) * K1B + c;
-    Basis<P> bq[sizeof(P) == 4 ? VH : 1];
-    if constexpr (sizeof(P) == 4) {
-#pragma unroll
-        for (int q = 0; q < VH; ++q)
-            if (FCAS_CHECK(((int64_t)blk * (L / 2) + j) * K1B + c + (int64_t)q * G * K1B < ((int64_t)L / 2 << log_n1),
-                           kCheckBasis))
-                bq[q] = bb[(int64_t)q * G * K1B];
-    }
+    // Thread (c, j) owns the bins k = k1 + N1 (j + q G), q < VH:
+    // P_a[k] = e^{i (psi(f_k) + 2 pi k Delta^0)} sum_i w_a,i Y_i[k] e^{2 pi i k (Delta^i - Delta^0)}.
+    const BasisD* bb = basis + ((int64_t)blk * (L / 2) + j) * K1B + c;
     const int kbase = k1 + n1 * j;
     const int kstep = n1 * G;
     const int64_t col0 = (int64_t)blk * n_det;
+    const double dturn0 = pp->dturn[0];
+    auto chirp_phasor = [&](int q) {
+        BasisD b{};
+        if (FCAS_CHECK(((int64_t)blk * (L / 2) + j) * K1B + c + (int64_t)q * G * K1B < ((int64_t)L / 2 << log_n1),
+                       kCheckBasis))
+            b = bb[(int64_t)q * G * K1B];
+        const double u = fma((double)(kbase + q * kstep), dturn0, chirp_frac(b, pp->c));
+        if constexpr (kFF) return unit_phasor(u - rint(u), ptab);
+        else return unit_phasor(u, ptab);
+    };
+    auto spectrum = [&](int i, int q) {
+        C yv = mkc(Real(0.0f), Real(0.0f));
+        const int64_t at = ((col0 + i) * (L / 2) + j) * K1B + c + (int64_t)q * G * K1B;
+        if (FCAS_CHECK(at < (int64_t)n_det * ((int64_t)L / 2 << log_n1), kCheckSpectrum)) {
+            if constexpr (kFF) yv = ldg_c(y + at);
+            else yv = y[at];
+        }
+        return yv;
+    };
     // The float-float form keeps its code small (its fully unrolled double-word arithmetic would not
     // fit the instruction cache): the chirp phasors are formed in a loop into shared memory (the
     // transforms' exchange buffers, not yet in use) and the detector loop is not unrolled.
     if constexpr (kFF) {
 #pragma unroll 1
         for (int q = 0; q < VH; ++q) {
-            Basis<P> b{};
-            if (FCAS_CHECK(((int64_t)blk * (L / 2) + j) * K1B + c + (int64_t)q * G * K1B < ((int64_t)L / 2 << log_n1),
-                           kCheckBasis))
-                b = bb[(int64_t)q * G * K1B];
+            const C cp = chirp_phasor(q);
             if (FCAS_CHECK((q * (int)blockDim.x + (int)threadIdx.x < pass_a_buf_elems<Real, LOG_L, K1B, MAXRB>()),
                            kCheckExchangeWrite))
-                smem[q * blockDim.x + threadIdx.x] = ff_unit_phasor(chirp_frac(b, *pp), ptab);
+                smem[q * blockDim.x + threadIdx.x] = cp;
         }
+    }
+    C r1[VH], r2[VH];
+#pragma unroll
+    for (int q = 0; q < VH; ++q) {
+        const C yv = spectrum(0, q);
+        r1[q] = mkc(sc.w1[0] * yv.x, sc.w1[0] * yv.y);
+        r2[q] = mkc(sc.w2[0] * yv.x, sc.w2[0] * yv.y);
     }
     constexpr int kDetUnroll = kFF ? 1 : FCAS_MAX_DET;
 #pragma unroll kDetUnroll
-    for (int i = 0; i < FCAS_MAX_DET; ++i) {
+    for (int i = 1; i < FCAS_MAX_DET; ++i) {
         if (i >= n_det) break;
-        C dph, dstep;
-        if constexpr (sizeof(P) == 4) {
-            float fb = frac_mul_ff((float)kbase, 0.0f, sc.dh[i], sc.dl[i]);
-            float fs = frac_mul_ff((float)kstep, 0.0f, sc.dh[i], sc.dl[i]);
-            fb -= rintf(fb);
-            fs -= rintf(fs);
-            dph = fast_phasor(fb);
-            dstep = fast_phasor(fs);
-        } else {
-            if constexpr (kFF) {
-                // the delay fraction without binary64 arithmetic (60-min pass A 34.7 -> 32.0 ms)
-                dph = ff_unit_phasor(ff_frac_mul_int(kbase, dsplit[0][i], dsplit[1][i], dsplit[2][i]), ptab);
-                dstep = ff_unit_phasor(ff_frac_mul_int(kstep, dsplit[0][i], dsplit[1][i], dsplit[2][i]), ptab);
-            } else {
-                const double fb = (double)kbase * sc.dh[i], fs = (double)kstep * sc.dh[i];
-                dph = unit_phasor(fb - rint(fb));
-                dstep = unit_phasor(fs - rint(fs));
-            }
-        }
-        const C* yd = y + ((col0 + i) * (L / 2) + j) * K1B + c;
+        const int kmid = kbase + phasor_mid(VH) * kstep;
+        C dph;
+        if constexpr (kFF)
+            dph = ff_unit_phasor(ff_frac_mul_int(kmid, dsplit[0][i], dsplit[1][i], dsplit[2][i]), ptab);
+        else
+            dph = unit_phasor((double)kmid * sc.rturn[i], ptab);
         const Real w1 = sc.w1[i], w2 = sc.w2[i];
-#pragma unroll
-        for (int q = 0; q < VH; ++q) {
-            C yv = mkc(Real(0.0f), Real(0.0f));
-            if (FCAS_CHECK(((col0 + i) * (L / 2) + j) * K1B + c + (int64_t)q * G * K1B <
-                               (int64_t)n_det * ((int64_t)L / 2 << log_n1), kCheckSpectrum)) {
-                if constexpr (kFF) yv = ldg_c(yd + (int64_t)q * G * K1B);
-                else yv = yd[(int64_t)q * G * K1B];
-            }
-            const C t = cmul(yv, dph);
-            r1[q].x += w1 * t.x;
-            r1[q].y += w1 * t.y;
-            r2[q].x += w2 * t.x;
-            r2[q].y += w2 * t.y;
-            if (q + 1 < VH) dph = cmul(dph, dstep);
-        }
+        phasor_run<Real, VH>(dph, sc.step[i], [&](int q, C ph) {
+            const C t = cmul(spectrum(i, q), ph);
+            r1[q] = mkc(axpy(w1, t.x, r1[q].x), axpy(w1, t.y, r1[q].y));
+            r2[q] = mkc(axpy(w2, t.x, r2[q].x), axpy(w2, t.y, r2[q].y));
+        });
     }
-    {
-        float cfh[4], cfl[4];
-        if constexpr (sizeof(P) == 4) {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                cfh[r] = pp->ch[r];
-                cfl[r] = pp->cl[r];
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < VH; ++q) {
-            C cp;
-            if constexpr (sizeof(P) == 4) {
-                const ChirpPowers b = chirp_powers_lean(bq[q]);
-                float s = frac_mul_ff(cfh[0], cfl[0], b.b53.x, b.b53.y);
-                s += frac_mul_ff(cfh[1], cfl[1], b.b1.x, b.b1.y);
-                s += frac_mul_ff(cfh[2], cfl[2], b.b23.x, b.b23.y);
-                s += frac_mul_ff(cfh[3], cfl[3], b.b13.x, b.b13.y);
-                cp = fast_phasor(s - rintf(s));
-            } else if constexpr (kFF) {
-                cp = smem[q * blockDim.x + threadIdx.x];
-            } else {
-                Basis<P> b{};
-                if (FCAS_CHECK(((int64_t)blk * (L / 2) + j) * K1B + c + (int64_t)q * G * K1B <
-                                   ((int64_t)L / 2 << log_n1), kCheckBasis))
-                    b = bb[(int64_t)q * G * K1B];
-                cp = unit_phasor(chirp_frac(b, *pp));
-            }
-            r1[q] = cmul(r1[q], cp);
-            r2[q] = cmul(r2[q], cp);
-        }
+    for (int q = 0; q < VH; ++q) {
+        C cp;
+        if constexpr (kFF) cp = smem[q * blockDim.x + threadIdx.x];
+        else cp = chirp_phasor(q);
+        r1[q] = cmul(r1[q], cp);
+        r2[q] = cmul(r2[q], cp);
     }
     if constexpr (kFF) __syncthreads();   // every chirp phasor read before the exchange buffers are reused
 
@@ -319,23 +324,18 @@ pass_a_kernel(const cplx<Real>* __restrict__ y, const Basis<phase_t<Real>>* __re
         for (int q = 0; q < VH; ++q) v[q] = a == 0 ? r1[q] : r2[q];
 #pragma unroll
         for (int q = VH; q < V; ++q) v[q] = mkc(Real(0.0f), Real(0.0f));
-        // FP32: stage twiddles mostly loaded (60-min pass A 4.11 -> 4.07 ms; pass B keeps the
-        // products, which need fewer registers than its three CTAs per SM allow for the loads)
-        fftr<Real, +1, LOG_L, MAXRB, 0, 0, true, sizeof(Real) == 4, pass_a_pad_shift<Real, MAXRB>(), false>(
-            v, smem + c, K1B, j, stw);
+        fftr<Real, +1, LOG_L, MAXRB, 0, 0, true, false, pass_a_pad_shift<Real, MAXRB>(), false>(v, smem + c, K1B, j, stw);
         C* orow = out + ((p * kSeries + a) * L) * (int64_t)n1 + k1;
-        // e^{2 pi i k1 ta / N} for ta = j + q G: the value at q = 0 times powers of the step e^{2 pi i k1 G / N}
-        const int m0 = k1 * j, ms = k1 * G;   // < N
-        C w = cmul(ldg_c(tw_hi + (m0 >> kTwLoBits)), ldg_c(tw_lo + (m0 & ((1 << kTwLoBits) - 1))));
+        // e^{2 pi i k1 ta / N} for ta = j + q G, steps of e^{2 pi i k1 G / N}
+        const int m0 = k1 * (j + phasor_mid(V) * G), ms = k1 * G;   // < N
+        const C w0 = cmul(ldg_c(tw_hi + (m0 >> kTwLoBits)), ldg_c(tw_lo + (m0 & ((1 << kTwLoBits) - 1))));
         const C step = cmul(ldg_c(tw_hi + (ms >> kTwLoBits)), ldg_c(tw_lo + (ms & ((1 << kTwLoBits) - 1))));
-#pragma unroll
-        for (int q = 0; q < V; ++q) {
+        phasor_run<Real, V>(w0, step, [&](int q, C w) {
             const int ta = j + q * G;
             if (FCAS_CHECK((p * kSeries + a) * (int64_t)L * n1 + k1 + (int64_t)ta * n1 < np * kSeries * (int64_t)L * n1,
                            kCheckInterWrite))
                 st_stream(orow + (int64_t)ta * n1, cmul(v[q], w));   // streamed: read back only by pass B
-            if (q + 1 < V) w = cmul(w, step);
-        }
+        });
     }
 }
 
@@ -385,21 +385,20 @@ __device__ __forceinline__ int pass_b_ta(int row, int log_ga, int cb_a) {
 // |W2(t)|^2 for t = ta + N2 tb (Sec. II.C, the maximisation over A_k in closed form), and the
 // argmax over the CTA's rows (lowest t on ties).
 // ------------------------------------------------------------------------------------------
-// Resident pass-B CTAs per SM the compiler is held to: three for the FP32 form's 2^11- and
-// 2^12-point rows (76-77 registers, no spills), two for other CTAs of up to 256 threads.
-__host__ __device__ constexpr int pass_b_min_blocks(int log_l, int real_bytes) {
-    return pass_b_threads(log_l, real_bytes) > 256 ? 1 : (real_bytes == 4 && (log_l == 11 || log_l == 12)) ? 3 : 2;
-}
+template <typename Real> constexpr int form_of = std::is_same<Real, double>::value ? FCAS_PREC_FP64 : FCAS_PREC_FF;
+// resident pass-B CTAs per SM the compiler is held to: two of up to 256 threads
+__host__ __device__ constexpr int pass_b_min_blocks(int threads) { return threads > 256 ? 1 : 2; }
 
 template <typename Real, int LOG_L>
-__global__ void __launch_bounds__(pass_b_threads(LOG_L, sizeof(Real)), pass_b_min_blocks(LOG_L, sizeof(Real)))
+__global__ void __launch_bounds__(pass_b_threads(LOG_L, form_of<Real>),
+                                  pass_b_min_blocks(pass_b_threads(LOG_L, form_of<Real>)))
 pass_b_kernel(const cplx<Real>* __restrict__ inter, const ParticleParams* __restrict__ params, int64_t p0,
               int log_n2, int64_t n_samples, const cplx<Real>* __restrict__ stw, Partial* __restrict__ partials) {
     using C = cplx<Real>;
     constexpr int L = 1 << LOG_L;
     constexpr int V = shape_v(LOG_L);
     constexpr int G = L / V;
-    constexpr int TB = pass_b_tb(LOG_L, sizeof(Real));
+    constexpr int TB = pass_b_tb(LOG_L, form_of<Real>);
     constexpr int NT = TB * G;
     constexpr int BUF = fft_buf_elems<LOG_L, 4, 0, 4>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -682,7 +681,7 @@ pass_a_x2_kernel(const float2* __restrict__ y, const BasisF* __restrict__ basis,
     }
 }
 
-__host__ __device__ constexpr int x2_b_threads(int log_l) { return pass_b_threads(log_l, 4); }
+__host__ __device__ constexpr int x2_b_threads(int log_l) { return pass_b_threads(log_l, FCAS_PREC_FP32); }
 // resident pass-B CTAs the compiler is held to: 512 threads' worth (16 values per thread)
 __host__ __device__ constexpr int x2_b_min_blocks(int log_l) {
     return imin_c(16, imax_c(1, 512 / x2_b_threads(log_l)));
@@ -695,7 +694,7 @@ pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restri
     constexpr int L = 1 << LOG_L;
     constexpr int V = shape_v(LOG_L);
     constexpr int G = L / V;
-    constexpr int TB = pass_b_tb(LOG_L, 4);
+    constexpr int TB = pass_b_tb(LOG_L, FCAS_PREC_FP32);
     constexpr int NT = TB * G;
     constexpr int BUF = fft_buf_elems<LOG_L, 4, 1, 4>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -760,10 +759,7 @@ pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restri
 
 // Column-block widths of the packed FP32 pass A: the default of the length and, from 2^8 points on,
 // half, twice and four times it while a CTA stays within 512 threads.
-template <int LG>
-constexpr bool x2_k1b_ok(int k) {
-    return k >= 1 && k <= 16 && k <= (1 << LG) && x2_a_threads(LG, k) <= 512;
-}
+constexpr bool x2_k1b_ok(int lg, int k) { return k >= 1 && k <= 16 && k <= (1 << lg) && x2_a_threads(lg, k) <= 512; }
 
 template <int LG, int K1B, int MAXRB = 4>
 static cudaError_t pass_a_x2_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
@@ -792,7 +788,7 @@ static cudaError_t pass_a_x2_at(const FitnessPlan& pl, const ParticleParams* par
 template <int LG>
 static cudaError_t pass_a_x2_lg(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
                                 void* inter, cudaStream_t s) {
-    constexpr int KD = pass_a_k1b(LG, 4);
+    constexpr int KD = pass_a_k1b(LG, FCAS_PREC_FP32);
     if (pl.radix_bits_a == 3) {
         // radix-8 stages: 8 values per thread, CTAs of 2 or 4 columns (at most 1024 threads)
         if constexpr (LG >= 10 && LG <= 11)
@@ -806,11 +802,11 @@ static cudaError_t pass_a_x2_lg(const FitnessPlan& pl, const ParticleParams* par
     if constexpr (LG >= 10 && KD > 1)
         if (pl.k1b == 1) return pass_a_x2_at<LG, 1>(pl, params, p0, np, inter, s);   // one column per CTA
     if constexpr (LG >= 8) {
-        if constexpr (x2_k1b_ok<LG>(KD / 2))
+        if constexpr (x2_k1b_ok(LG, KD / 2))
             if (pl.k1b == KD / 2) return pass_a_x2_at<LG, (KD / 2 > 0 ? KD / 2 : 1)>(pl, params, p0, np, inter, s);
-        if constexpr (x2_k1b_ok<LG>(KD * 2))
+        if constexpr (x2_k1b_ok(LG, KD * 2))
             if (pl.k1b == KD * 2) return pass_a_x2_at<LG, (KD * 2 <= 16 ? KD * 2 : 16)>(pl, params, p0, np, inter, s);
-        if constexpr (x2_k1b_ok<LG>(KD * 4))
+        if constexpr (x2_k1b_ok(LG, KD * 4))
             if (pl.k1b == KD * 4) return pass_a_x2_at<LG, (KD * 4 <= 16 ? KD * 4 : 16)>(pl, params, p0, np, inter, s);
     }
     return cudaErrorInvalidValue;
@@ -819,7 +815,7 @@ static cudaError_t pass_a_x2_lg(const FitnessPlan& pl, const ParticleParams* par
 template <int LG>
 static cudaError_t pass_b_x2_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
                                 const void* inter, Partial* partials, cudaStream_t s) {
-    constexpr int TB = pass_b_tb(LG, 4);
+    constexpr int TB = pass_b_tb(LG, FCAS_PREC_FP32);
     const size_t smem = sizeof(c32x2) * (size_t)TB * fft_buf_elems<LG, 4, 1, 4>();
     auto kern = pass_b_x2_kernel<LG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -852,49 +848,37 @@ static cudaError_t pass_a_at(const FitnessPlan& pl, const ParticleParams* params
     if (e != cudaSuccess) return e;
     const int64_t ctas = np * ((1 << pl.log_n1) / K1B);
     kern<<<(unsigned)ctas, THREADS, smem, s>>>(static_cast<const cplx<Real>*>(pl.y),
-                                     static_cast<const Basis<phase_t<Real>>*>(pl.basis),
+                                     static_cast<const BasisD*>(pl.basis),
                                      params, p0, np, pl.n_det, pl.log_n1, pl.sub, static_cast<cplx<Real>*>(inter),
                                      static_cast<const cplx<Real>*>(pl.stw_a), static_cast<const cplx<Real>*>(pl.tw_lo),
                                      static_cast<const cplx<Real>*>(pl.tw_hi), static_cast<const cplx<Real>*>(pl.ptab));
     return cudaGetLastError();
 }
 
-// Column-block widths compiled for pass A: the default of the length and, for the FP32 form at
-// lengths >= 2^8, half and twice it (the autotuner's choices).
-template <int LG, int RB>
-constexpr bool k1b_variant_ok(int k) {
-    return k >= 1 && k <= 16 && k <= (1 << LG) && k * ((1 << LG) / shape_v(LG)) <= 1024;
-}
+// binary64 form: CTAs of twice the default's columns are compiled for 2^8- to 2^11-point columns
+constexpr bool fp64_k1b_double(int lg) { return lg >= 8 && lg <= 11; }
 
 template <typename Real, int LG>
 static cudaError_t pass_a_lg(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
                              void* inter, cudaStream_t s) {
-    constexpr int RB = sizeof(Real);
-    constexpr int KD = pass_a_k1b(LG, RB);
+    constexpr int KD = pass_a_k1b(LG, form_of<Real>);
     if (pl.radix_bits_a == 3) {
-        // radix-8 stages: 8 values per thread, 1024-thread CTAs of 4 columns (FP32, >= 2^10 points)
-        if constexpr (RB == 4 && LG >= 10 && LG <= 12)
-            if (pl.k1b == 4) return pass_a_at<Real, LG, 4, 3>(pl, params, p0, np, inter, s);
-        // float-float: 512-thread CTAs of 2 columns (half the registers per thread of radix 16)
+        // float-float: radix-8 stages, 512-thread CTAs of 2 columns (half the registers per thread of radix 16)
         if constexpr (std::is_same<Real, ffloat>::value && LG >= 10 && LG <= 12)
             if (pl.k1b == 2) return pass_a_at<Real, LG, 2, 3>(pl, params, p0, np, inter, s);
         return cudaErrorInvalidValue;
     }
     if (pl.k1b == KD) return pass_a_at<Real, LG, KD>(pl, params, p0, np, inter, s);
-    if constexpr (RB == 4 && LG >= 8) {
-        if constexpr (k1b_variant_ok<LG, RB>(KD / 2))
-            if (pl.k1b == KD / 2) return pass_a_at<Real, LG, (KD / 2 > 0 ? KD / 2 : 1)>(pl, params, p0, np, inter, s);
-        if constexpr (k1b_variant_ok<LG, RB>(KD * 2))
-            if (pl.k1b == KD * 2) return pass_a_at<Real, LG, (KD * 2 <= 16 ? KD * 2 : 16)>(pl, params, p0, np, inter, s);
-    }
+    if constexpr (std::is_same<Real, double>::value && fp64_k1b_double(LG))
+        if (pl.k1b == KD * 2) return pass_a_at<Real, LG, KD * 2>(pl, params, p0, np, inter, s);
     return cudaErrorInvalidValue;
 }
 
 template <typename Real, int LG>
 static cudaError_t pass_b_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
                              const void* inter, Partial* partials, cudaStream_t s) {
-    constexpr int TB = pass_b_tb(LG, sizeof(Real));
-    constexpr int THREADS = pass_b_threads(LG, sizeof(Real));
+    constexpr int TB = pass_b_tb(LG, form_of<Real>);
+    constexpr int THREADS = pass_b_threads(LG, form_of<Real>);
     const size_t smem = sizeof(cplx<Real>) * (size_t)TB * fft_buf_elems<LG, 4, 0, 4>();
     auto kern = pass_b_kernel<Real, LG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
