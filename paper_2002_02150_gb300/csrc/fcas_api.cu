@@ -180,13 +180,16 @@ void prof_end(fcas_ctx* c, size_t slot, cudaStream_t s) {
     if (slot != SIZE_MAX) cudaEventRecord(c->events[slot].b, s);
 }
 
-// Passes A, B and the final argmax over chunks of particle parameters, with the given scratch.
+// Passes A, B and the final argmax over chunks of particle parameters, with the given scratch: as many
+// equal chunks as needed (77 particles by 64: 39 + 38 instead of 64 + 13, whose last waves are emptier).
 cudaError_t launch_passes_with(fcas_ctx* c, const ParticleParams* params, void* inter, Partial* partials,
                                int64_t chunk, int64_t n, double* d_fit, int64_t* d_tc, cudaStream_t st) {
     const FitnessPlan plan = make_plan(c);
     const int prec = c->setup.precision;
     size_t slot;
     cudaError_t e = cudaSuccess;
+    const int64_t nch = (n + chunk - 1) / chunk;
+    chunk = nch > 0 ? (n + nch - 1) / nch : chunk;
     for (int64_t p0 = 0; p0 < n && e == cudaSuccess; p0 += chunk) {
         const int64_t np = (n - p0) < chunk ? (n - p0) : chunk;
         prof_begin(c, FCAS_KERNEL_PASS_A, st, &slot);
@@ -241,6 +244,16 @@ cudaError_t gradient_device(fcas_ctx* c, int64_t n, const double* d_theta, const
     if (e != cudaSuccess) return e;
     return launch_gradient(make_plan(c), c->setup.precision, c->k_lo, c->k_hi, c->d_params, d_theta, d_tc, n,
                            c->d_gsums, c->d_det, c->d_sigma2s, c->setup.f_low, c->df, d_grad, st);
+}
+
+// Particles per chunk when the caller leaves it open: at least 64, and for short segments as many as 512 MB of
+// scratch hold (a chunk's launches have fixed costs and a last wave: 320 particles on 64 s take 239 us in
+// chunks of 64 and 195 us in one, on 4096 points 95 and 38 us; from 2^19 points on 64 is enough). Bounded by
+// 16 GB, and by 2048 (the passes' grids have one row of CTAs per particle).
+int64_t auto_chunk(size_t per_particle) {
+    const int64_t most = (int64_t)(((size_t)16 << 30) / per_particle);
+    const int64_t want = std::min<int64_t>(2048, std::max<int64_t>(64, (int64_t)(((size_t)512 << 20) / per_particle)));
+    return std::max<int64_t>(1, std::min(want, most));
 }
 
 // Scratch of the fitness path (allocated at create unless FCAS_SETUP_LAZY_SCRATCH, else on first use).
@@ -528,13 +541,7 @@ int create_impl(fcas_ctx** out, const fcas_setup* setup, const fcas_detector* de
 
     // scratch for the fitness path (partials sized for every split the tuner may choose)
     const size_t per_particle = inter_bytes_per_particle(s.precision, n);
-    int64_t chunk = s.max_batch;
-    if (chunk == 0) {
-        const size_t budget = (size_t)16 << 30;
-        chunk = (int64_t)(budget / per_particle);
-        if (chunk > 64) chunk = 64;
-        if (chunk < 1) chunk = 1;
-    }
+    const int64_t chunk = s.max_batch > 0 ? s.max_batch : auto_chunk(per_particle);
     c->chunk = chunk;
     c->nb_cap = 0;
     for (int bias = 0; bias <= 1; ++bias) {
@@ -864,6 +871,9 @@ int fcas_set_shape(fcas_ctx* c, int32_t split_bias, int32_t k1b, int32_t sub, in
 struct fcas_group {
     std::vector<fcas_ctx*> ctxs;
     int64_t chunk = 0;
+    int64_t auto_cap = 0;           // largest chunk a search may grow the scratch to (0: the caller fixed it)
+    size_t inter_pp = 0;            // scratch per particle: intermediate bytes and argmax partials
+    int64_t nb = 0;
     void* d_inter = nullptr;
     Partial* d_partials = nullptr;
     ParticleParams* d_params = nullptr;
@@ -891,9 +901,11 @@ int fcas_group_create(fcas_group** out, int32_t n_ctx, fcas_ctx* const* ctxs, in
     }
     fcas_group* g = new fcas_group();
     g->ctxs.assign(ctxs, ctxs + n_ctx);
-    int64_t chunk = max_batch;
-    if (chunk == 0) chunk = std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)(((size_t)16 << 30) / inter_pp)));
+    const int64_t chunk = max_batch > 0 ? max_batch : std::min<int64_t>(64, auto_chunk(inter_pp));
     g->chunk = chunk;
+    g->auto_cap = max_batch > 0 ? 0 : auto_chunk(inter_pp);
+    g->inter_pp = inter_pp;
+    g->nb = nb;
     int rc = dev_alloc(&g->d_inter, inter_pp * (size_t)chunk, "group intermediate transform");
     if (!rc) rc = dev_alloc(&g->d_partials, sizeof(Partial) * (size_t)chunk * nb, "group argmax partials");
     if (!rc) {
@@ -940,6 +952,22 @@ int fcas_group_search_boxes(fcas_group* g, const fcas_pso_config* cfg, const dou
         rc = dev_alloc(&g->d_params, sizeof(ParticleParams) * (size_t)rows, "group particle parameters");
         if (rc) return rc;
         g->params_cap = rows;
+    }
+    if (const int64_t want = std::min(rows, g->auto_cap); want > g->chunk) {
+        // larger swarms in fewer chunks; the present scratch stays when the device has no room for more
+        void* inter = nullptr;
+        Partial* partials = nullptr;
+        if (cudaMalloc(&inter, g->inter_pp * (size_t)want) == cudaSuccess &&
+            cudaMalloc(&partials, sizeof(Partial) * (size_t)want * g->nb) == cudaSuccess) {
+            cudaFree(g->d_inter);
+            cudaFree(g->d_partials);
+            g->d_inter = inter;
+            g->d_partials = partials;
+            g->chunk = want;
+        } else {
+            cudaGetLastError();
+            if (inter) cudaFree(inter);
+        }
     }
     const size_t per = align256(swarm_bytes(rows, cfg->n_runs));
     if (per * n_ctx > g->pso_bytes) {
