@@ -201,7 +201,7 @@ cudaError_t launch_passes_with(fcas_ctx* c, const ParticleParams* params, void* 
         prof_end(c, slot, st);
         if (e != cudaSuccess) break;
         prof_begin(c, FCAS_KERNEL_REDUCE, st, &slot);
-        e = launch_reduce(partials, c->nb_partials, params, p0, np, d_fit, d_tc, st);
+        e = launch_reduce(partials, c->nb_partials, params, p0, np, d_fit, d_tc, chain_pays(np, c->log_n), st);
         prof_end(c, slot, st);
     }
     return e;
@@ -636,7 +636,7 @@ Swarm carve_swarm(unsigned char* b, int64_t rows, int runs) {
     w.s.x = reinterpret_cast<double*>(b);
     w.s.v = reinterpret_cast<double*>(b + r4);
     w.s.pbest_x = reinterpret_cast<double*>(b + 2 * r4);
-    w.theta = reinterpret_cast<double*>(b + 3 * r4);
+    w.theta = w.s.theta = reinterpret_cast<double*>(b + 3 * r4);
     w.s.pbest_f = reinterpret_cast<double*>(b + 4 * r4);
     w.fit = reinterpret_cast<double*>(b + 4 * r4 + r1);
     w.s.pbest_tc = reinterpret_cast<int64_t*>(b + 4 * r4 + 2 * r1);
@@ -653,12 +653,11 @@ Swarm carve_swarm(unsigned char* b, int64_t rows, int runs) {
 // One PSO iteration of one segment: parameters of the particles inside the box, their fitness, update.
 cudaError_t swarm_iteration(fcas_ctx* c, const PsoDev& g, const Swarm& w, ParticleParams* params, void* inter,
                             Partial* partials, int64_t chunk, int64_t rows, cudaStream_t st) {
-    cudaError_t x = launch_pso_theta(g, w.s, w.theta, st);
-    if (x == cudaSuccess)
-        x = launch_geometry(w.theta, rows, params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low, c->df,
+    // (w.theta holds the positions' parameters: written by the initialisation and by every update)
+    cudaError_t x = launch_geometry(w.theta, rows, params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low, c->df,
                             pass_a_kstep(c), c->setup.precision, st);
     if (x == cudaSuccess) x = launch_passes_with(c, params, inter, partials, chunk, rows, w.fit, w.tcs, st);
-    if (x == cudaSuccess) x = launch_pso_update(g, 0, w.fit, w.tcs, w.s, st);
+    if (x == cudaSuccess) x = launch_pso_update(g, 0, w.fit, w.tcs, w.s, st, chain_pays(rows, c->log_n));
     return x;
 }
 

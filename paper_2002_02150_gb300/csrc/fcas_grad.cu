@@ -108,10 +108,12 @@ __device__ __forceinline__ void warp_sums(Acc (&v)[kGradVals], int lane) {
 template <typename Real>
 __global__ void __launch_bounds__(kGradThreads, 2)
 grad_sums_kernel(const cplx<Real>* __restrict__ y, bool y_ff, const Basis<Real>* __restrict__ basis,
-                 const ParticleParams* __restrict__ params, const int64_t* __restrict__ tc, int n_det, int log_n,
+                 const ParticleParams* params, const int64_t* __restrict__ tc, int n_det, int log_n,
                  int log_n1, int log_n2, int log_k1b, int k_lo, int k_hi, int nseg, int blks,
-                 double* __restrict__ part) {
+                 double* part) {
     using Acc = typename grad_sum<Real>::type;
+    chain_wait();
+    chain_go();
     __shared__ Acc red[kGradThreads / 32][kGradVals];
     const int pairs = (n_det + kGradDet - 1) / kGradDet;
     const int seg = blockIdx.x % nseg;
@@ -256,7 +258,7 @@ __device__ void chirp_coeffs_dual(double tau0, double tau15, double dt0, double 
 // binary64, whose every dependent instruction waits tens of cycles).
 constexpr int kFinalThreads = 128;
 __global__ void __launch_bounds__(kFinalThreads)
-grad_final_kernel(const double* __restrict__ theta, const int64_t* __restrict__ tc, const double* __restrict__ part,
+grad_final_kernel(const double* __restrict__ theta, const int64_t* __restrict__ tc, const double* part,
                   int nseg, const double* __restrict__ det9, const double* __restrict__ s2, int n_det, double f_star,
                   double df, double* __restrict__ grad) {
     __shared__ double sp[FCAS_MAX_DET * kGradSums];   // Z_i, F_i, S_ij
@@ -266,6 +268,8 @@ grad_final_kernel(const double* __restrict__ theta, const int64_t* __restrict__ 
     __shared__ double dc[2][4];                       // d c_j / d tau0, d c_j / d tau1.5
     const int64_t p = blockIdx.x;
     const int tid = threadIdx.x;
+    chain_wait();
+    chain_go();
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     const double alpha = theta[4 * p], delta = theta[4 * p + 1], tau0 = theta[4 * p + 2], tau15 = theta[4 * p + 3];
     if (!(isfinite(alpha) && isfinite(delta) && tau0 > 0.0 && tau15 > 0.0 && tc[p] >= 0)) {
@@ -405,20 +409,20 @@ cudaError_t launch_gradient(const FitnessPlan& pl, int precision, int64_t k_lo, 
     for (int64_t p0 = 0; p0 < n; p0 += chunk) {
         const int64_t np = n - p0 < chunk ? n - p0 : chunk;
         const unsigned ctas = (unsigned)(np * pairs * nseg);
+        cudaError_t e;
         if (precision == FCAS_PREC_FP32)
-            grad_sums_kernel<float><<<ctas, kGradThreads, 0, s>>>(
-                static_cast<const float2*>(pl.y), false, static_cast<const BasisF*>(pl.basis), params + p0, tc + p0,
-                pl.n_det, pl.log_n, pl.log_n1, pl.log_n2, log_k1b, (int)k_lo, (int)k_hi, nseg, blks, part);
+            e = launch_chained(true, grad_sums_kernel<float>, dim3(ctas), dim3(kGradThreads), 0, s,
+                               static_cast<const float2*>(pl.y), false, static_cast<const BasisF*>(pl.basis),
+                               params + p0, tc + p0, pl.n_det, pl.log_n, pl.log_n1, pl.log_n2, log_k1b, (int)k_lo,
+                               (int)k_hi, nseg, blks, part);
         else
-            grad_sums_kernel<double><<<ctas, kGradThreads, 0, s>>>(
-                static_cast<const double2*>(pl.y), precision == FCAS_PREC_FF, static_cast<const BasisD*>(pl.basis),
-                params + p0, tc + p0, pl.n_det, pl.log_n, pl.log_n1, pl.log_n2, log_k1b, (int)k_lo, (int)k_hi, nseg,
-                blks, part);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        grad_final_kernel<<<(unsigned)np, kFinalThreads, 0, s>>>(theta + 4 * p0, tc + p0, part, nseg, det9, s2,
-                                                                 pl.n_det, f_star, df, grad + 4 * p0);
-        e = cudaGetLastError();
+            e = launch_chained(true, grad_sums_kernel<double>, dim3(ctas), dim3(kGradThreads), 0, s,
+                               static_cast<const double2*>(pl.y), precision == FCAS_PREC_FF,
+                               static_cast<const BasisD*>(pl.basis), params + p0, tc + p0, pl.n_det, pl.log_n,
+                               pl.log_n1, pl.log_n2, log_k1b, (int)k_lo, (int)k_hi, nseg, blks, part);
+        if (e == cudaSuccess)
+            e = launch_chained(true, grad_final_kernel, dim3((unsigned)np), dim3(kFinalThreads), 0, s, theta + 4 * p0,
+                               tc + p0, part, nseg, det9, s2, pl.n_det, f_star, df, grad + 4 * p0);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(64)
 geometry_kernel(const double* __restrict__ theta, int64_t n, ParticleParams* __restrict__ out,
                 const double* __restrict__ det9, const double* __restrict__ s2, int n_det, double f_star, double df,
                 int64_t kstep, bool wide, TaylorBound tb) {
+    chain_go();
     const int lane = threadIdx.x & 31, sub = lane % kGeomLanes, lane0 = lane - sub;
     const int64_t p = (int64_t)blockIdx.x * kGeomParticles + lane / kGeomLanes;
     const bool have = p < n;
@@ -209,11 +210,13 @@ __device__ __forceinline__ bool better(double v, int64_t t, double bv, int64_t b
 }
 
 
-__global__ void reduce_kernel(const Partial* __restrict__ partials, int64_t nb, const ParticleParams* __restrict__ params,
+__global__ void reduce_kernel(const Partial* partials, int64_t nb, const ParticleParams* params,
                               int64_t p0, double* __restrict__ fitness, int64_t* __restrict__ tc) {
     __shared__ double sv[32];
     __shared__ int64_t st[32];
     const int64_t p = blockIdx.x;
+    chain_wait();
+    chain_go();
     double best = -DBL_MAX;
     int64_t bt = INT64_MAX;
     for (int64_t b = threadIdx.x; b < nb; b += blockDim.x) {
@@ -239,10 +242,10 @@ __global__ void reduce_kernel(const Partial* __restrict__ partials, int64_t nb, 
 }
 
 cudaError_t launch_reduce(const Partial* partials, int64_t nb, const ParticleParams* params, int64_t p0, int64_t np,
-                          double* fitness, int64_t* tc, cudaStream_t s) {
+                          double* fitness, int64_t* tc, bool chained, cudaStream_t s) {
     if (np <= 0) return cudaSuccess;
-    reduce_kernel<<<(unsigned)np, 256, 0, s>>>(partials, nb, params, p0, fitness, tc);
-    return cudaGetLastError();
+    return launch_chained(chained, reduce_kernel, dim3((unsigned)np), dim3(256), 0, s, partials, nb, params, p0, fitness,
+                          tc);
 }
 
 // ------------------------------------------------------------------------------------------

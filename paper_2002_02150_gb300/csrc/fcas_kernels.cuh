@@ -121,7 +121,7 @@ cudaError_t launch_pass_b(const FitnessPlan& plan, const ParticleParams* params,
                           const void* inter, Partial* partials, cudaStream_t s);
 // Final argmax: fitness[p0 + p], tc[p0 + p].
 cudaError_t launch_reduce(const Partial* partials, int64_t nb, const ParticleParams* params, int64_t p0,
-                          int64_t np, double* fitness, int64_t* tc, cudaStream_t s);
+                          int64_t np, double* fitness, int64_t* tc, bool chained, cudaStream_t s);
 
 int pass_b_blocks_per_particle(int log_n1, int log_n2, int precision);
 // Checked build (FCAS_CHECKED): waits for the stream, returns and clears the bits of the index

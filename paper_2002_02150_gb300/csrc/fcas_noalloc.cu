@@ -97,7 +97,8 @@ extern "C" int fcas_fitness_noalloc(const fcas_ctx* c, int64_t n, const double* 
         if (e == cudaSuccess)
             e = launch_pass_a_prec(c->setup.precision, plan, params, 0, np, inter, st);
         if (e == cudaSuccess) e = launch_pass_b_prec(c->setup.precision, plan, params, 0, np, inter, partials, st);
-        if (e == cudaSuccess) e = launch_reduce(partials, c->nb_partials, params, 0, np, fitness + p0, tc + p0, st);
+        if (e == cudaSuccess)
+            e = launch_reduce(partials, c->nb_partials, params, 0, np, fitness + p0, tc + p0, chain_pays(np, c->log_n), st);
     }
     if (e != cudaSuccess) return report_error(FCAS_ERR_CUDA, cudaGetErrorString(e));
     // checked build (FCAS_CHECKED): wait for the launches and report a failed index check as this

@@ -197,7 +197,7 @@ struct DetConst {
 template <typename Real, int LOG_L, int K1B, int MAXRB>
 __global__ void __launch_bounds__(K1B * ((1 << LOG_L) / fftr_v(LOG_L, MAXRB)), 1)
 pass_a_kernel(const cplx<Real>* __restrict__ y, const BasisD* __restrict__ basis,
-              const ParticleParams* __restrict__ params, int64_t p0, int64_t np, int n_det, int log_n1, int sub_req,
+              const ParticleParams* params, int64_t p0, int64_t np, int n_det, int log_n1, int sub_req,
               cplx<Real>* __restrict__ out, const cplx<Real>* __restrict__ stw,
               const cplx<Real>* __restrict__ tw_lo, const cplx<Real>* __restrict__ tw_hi,
               const cplx<Real>* __restrict__ ptab) {
@@ -226,6 +226,8 @@ pass_a_kernel(const cplx<Real>* __restrict__ y, const BasisD* __restrict__ basis
     const int blk = (int)((rest / np) * sub + lin % sub);
     const int k1 = blk * K1B + c;
     const ParticleParams* pp = params + p0 + p;
+    chain_wait();
+    chain_go();
     if (!pp->valid) return;   // not evaluated (invalid input, or a PSO particle outside its box)
     // (CTAs of fewer than 8 threads fill the constants in turns)
     for (int i = threadIdx.x; i < FCAS_MAX_DET; i += blockDim.x) {
@@ -392,8 +394,8 @@ __host__ __device__ constexpr int pass_b_min_blocks(int threads) { return thread
 template <typename Real, int LOG_L>
 __global__ void __launch_bounds__(pass_b_threads(LOG_L, form_of<Real>),
                                   pass_b_min_blocks(pass_b_threads(LOG_L, form_of<Real>)))
-pass_b_kernel(const cplx<Real>* __restrict__ inter, const ParticleParams* __restrict__ params, int64_t p0,
-              int log_n2, int64_t n_samples, const cplx<Real>* __restrict__ stw, Partial* __restrict__ partials) {
+pass_b_kernel(const cplx<Real>* inter, const ParticleParams* params, int64_t p0,
+              int log_n2, int64_t n_samples, const cplx<Real>* __restrict__ stw, Partial* partials) {
     using C = cplx<Real>;
     constexpr int L = 1 << LOG_L;
     constexpr int V = shape_v(LOG_L);
@@ -412,6 +414,8 @@ pass_b_kernel(const cplx<Real>* __restrict__ inter, const ParticleParams* __rest
     const int n2 = 1 << log_n2;
     const int ta = blockIdx.x * TB + c;
     const int64_t p = blockIdx.y;
+    chain_wait();
+    chain_go();
     if (!params[p0 + p].valid) return;   // the final reduce reports NaN for it
     if constexpr (sizeof(Real) != 4) {
         // binary64 and float-float: the second series' row is requested into L2 now, so that its
@@ -487,7 +491,7 @@ template <int LOG_L, int K1B, int MAXRB = 4>
 __global__ void __launch_bounds__(x2_a_threads(LOG_L, K1B, MAXRB),
                                   x2_min_blocks(x2_a_threads(LOG_L, K1B, MAXRB), MAXRB))
 pass_a_x2_kernel(const float2* __restrict__ y, const BasisF* __restrict__ basis,
-                 const ParticleParams* __restrict__ params, int64_t p0, int64_t np, int n_det, int log_n1, int sub_req,
+                 const ParticleParams* params, int64_t p0, int64_t np, int n_det, int log_n1, int sub_req,
                  c32x2* __restrict__ out, const float2* __restrict__ stw, const float2* __restrict__ tw_lo,
                  const float2* __restrict__ tw_hi, int64_t items) {
     constexpr int L = 1 << LOG_L;
@@ -546,6 +550,10 @@ pass_a_x2_kernel(const float2* __restrict__ y, const BasisF* __restrict__ basis,
         // The particle's constants are read where they are used, straight from its parameter record
         // (the same address across the CTA, cached in L1): no shared-memory copy and no barrier before
         // the detector sums (60-min pass A 3.75 -> 3.67 ms per 64 particles).
+        if (lin == blockIdx.x) {   // the spectrum and basis above do not depend on the call
+            chain_wait();
+            chain_go();
+        }
         const int taylor_ok = pp->taylor_ok;
         if (!pp->valid) continue;   // not evaluated (invalid input, or a PSO particle outside its box)
 
@@ -560,13 +568,13 @@ pass_a_x2_kernel(const float2* __restrict__ y, const BasisF* __restrict__ basis,
             if (i >= n_det) break;
             // the phasor at the thread's first bin; its step to the next bin (kstep further) is the
             // particle's (formed once by the geometry kernel for this shape)
-            float fb = frac_mul_ff((float)kbase, 0.0f, __ldg(&pp->dh[i]), __ldg(&pp->dl[i]));
+            float fb = frac_mul_ff((float)kbase, 0.0f, pp->dh[i], pp->dl[i]);
             fb -= rintf(fb);
             float2 dph = fast_phasor(fb);
-            const float2 dstep = __ldg(&pp->dstep[i]);
+            const float2 dstep = pp->dstep[i];
             const int64_t yidx0 = ((col0 + i) * (L / 2) + j) * K1B + c;
             const float2* yd = y + yidx0;
-            const float w1 = __ldg(&pp->w1f[i]), w2 = __ldg(&pp->w2f[i]);
+            const float w1 = pp->w1f[i], w2 = pp->w2f[i];
 #pragma unroll
             for (int q = 0; q < VH; ++q) {
                 float2 yv = make_float2(0.0f, 0.0f);
@@ -588,8 +596,8 @@ pass_a_x2_kernel(const float2* __restrict__ y, const BasisF* __restrict__ basis,
             float cfh[4], cfl[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                cfh[r] = __ldg(&pp->ch[r]);
-                cfl[r] = __ldg(&pp->cl[r]);
+                cfh[r] = pp->ch[r];
+                cfl[r] = pp->cl[r];
             }
             if (kLane && (taylor_ok & (K1B <= 4 ? 1 : 2))) {
                 // The K1B lanes of a group (consecutive lanes, one per column) hold the adjacent bins
@@ -689,8 +697,8 @@ __host__ __device__ constexpr int x2_b_min_blocks(int log_l) {
 
 template <int LOG_L>
 __global__ void __launch_bounds__(x2_b_threads(LOG_L), x2_b_min_blocks(LOG_L))
-pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restrict__ params, int64_t p0, int log_n2,
-                 int log_ga, int cb_a, int64_t n_samples, const float2* __restrict__ stw, Partial* __restrict__ partials, int64_t ahead) {
+pass_b_x2_kernel(const c32x2* inter, const ParticleParams* params, int64_t p0, int log_n2,
+                 int log_ga, int cb_a, int64_t n_samples, const float2* __restrict__ stw, Partial* partials, int64_t ahead) {
     constexpr int L = 1 << LOG_L;
     constexpr int V = shape_v(LOG_L);
     constexpr int G = L / V;
@@ -708,6 +716,8 @@ pass_b_x2_kernel(const c32x2* __restrict__ inter, const ParticleParams* __restri
     const int n2 = 1 << log_n2;
     const int row_a = blockIdx.x * TB + c, ta = pass_b_ta(row_a, log_ga, cb_a);
     const int64_t p = blockIdx.y;
+    chain_wait();
+    chain_go();
     // The rows of the CTA `ahead` places later in launch order (one wave of resident CTAs) are requested
     // into L2 by one bulk prefetch per warp, so that DRAM keeps streaming while the resident CTAs
     // transform (60-min pass B 2.10 -> 1.94 ms per 64 particles).
@@ -778,11 +788,10 @@ static cudaError_t pass_a_x2_at(const FitnessPlan& pl, const ParticleParams* par
     if (e != cudaSuccess) return e;
     const int64_t wave = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
     const int64_t ctas = wave < items ? wave : items;
-    kern<<<(unsigned)ctas, THREADS, smem, s>>>(static_cast<const float2*>(pl.y), static_cast<const BasisF*>(pl.basis),
-                                               params, p0, np, pl.n_det, pl.log_n1, pl.sub, static_cast<c32x2*>(inter),
-                                               static_cast<const float2*>(pl.stw_a), static_cast<const float2*>(pl.tw_lo),
-                                               static_cast<const float2*>(pl.tw_hi), items);
-    return cudaGetLastError();
+    return launch_chained(chain_pays(np, pl.log_n), kern, dim3((unsigned)ctas), dim3(THREADS), smem, s,
+                          static_cast<const float2*>(pl.y), static_cast<const BasisF*>(pl.basis), params, p0, np, pl.n_det, pl.log_n1, pl.sub,
+                          static_cast<c32x2*>(inter), static_cast<const float2*>(pl.stw_a),
+                          static_cast<const float2*>(pl.tw_lo), static_cast<const float2*>(pl.tw_hi), items);
 }
 
 template <int LG>
@@ -827,10 +836,9 @@ static cudaError_t pass_b_x2_at(const FitnessPlan& pl, const ParticleParams* par
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((1 << pl.log_n2) / TB), (unsigned)np);
     const int log_ga = fft_log_g(pl.log_n2, pl.radix_bits_a), cb_a = fft_local_bits(pl.log_n2, pl.radix_bits_a, pl.k1b);
-    kern<<<grid, x2_b_threads(LG), smem, s>>>(static_cast<const c32x2*>(inter), params, p0, pl.log_n2, log_ga, cb_a,
-                                              pl.n_samples, static_cast<const float2*>(pl.stw_b), partials,
-                                              (int64_t)sms * (per_sm > 0 ? per_sm : 1));
-    return cudaGetLastError();
+    return launch_chained(chain_pays(np, pl.log_n), kern, grid, dim3(x2_b_threads(LG)), smem, s,
+                          static_cast<const c32x2*>(inter), params, p0, pl.log_n2, log_ga, cb_a, pl.n_samples, static_cast<const float2*>(pl.stw_b), partials,
+                          (int64_t)sms * (per_sm > 0 ? per_sm : 1));
 }
 
 // ------------------------------------------------------------------------------------------
@@ -847,12 +855,11 @@ static cudaError_t pass_a_at(const FitnessPlan& pl, const ParticleParams* params
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t ctas = np * ((1 << pl.log_n1) / K1B);
-    kern<<<(unsigned)ctas, THREADS, smem, s>>>(static_cast<const cplx<Real>*>(pl.y),
-                                     static_cast<const BasisD*>(pl.basis),
-                                     params, p0, np, pl.n_det, pl.log_n1, pl.sub, static_cast<cplx<Real>*>(inter),
-                                     static_cast<const cplx<Real>*>(pl.stw_a), static_cast<const cplx<Real>*>(pl.tw_lo),
-                                     static_cast<const cplx<Real>*>(pl.tw_hi), static_cast<const cplx<Real>*>(pl.ptab));
-    return cudaGetLastError();
+    return launch_chained(chain_pays(np, pl.log_n), kern, dim3((unsigned)ctas), dim3(THREADS), smem, s,
+                          static_cast<const cplx<Real>*>(pl.y), static_cast<const BasisD*>(pl.basis), params, p0, np, pl.n_det, pl.log_n1, pl.sub,
+                          static_cast<cplx<Real>*>(inter), static_cast<const cplx<Real>*>(pl.stw_a),
+                          static_cast<const cplx<Real>*>(pl.tw_lo), static_cast<const cplx<Real>*>(pl.tw_hi),
+                          static_cast<const cplx<Real>*>(pl.ptab));
 }
 
 // binary64 form: CTAs of twice the default's columns are compiled for 2^8- to 2^11-point columns
@@ -884,9 +891,8 @@ static cudaError_t pass_b_at(const FitnessPlan& pl, const ParticleParams* params
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((1 << pl.log_n2) / TB), (unsigned)np);
-    kern<<<grid, THREADS, smem, s>>>(static_cast<const cplx<Real>*>(inter), params, p0, pl.log_n2, pl.n_samples,
-                                     static_cast<const cplx<Real>*>(pl.stw_b), partials);
-    return cudaGetLastError();
+    return launch_chained(chain_pays(np, pl.log_n), kern, grid, dim3(THREADS), smem, s,
+                          static_cast<const cplx<Real>*>(inter), params, p0, pl.log_n2, pl.n_samples, static_cast<const cplx<Real>*>(pl.stw_b), partials);
 }
 
 template <typename Real>

@@ -47,6 +47,16 @@ __device__ __forceinline__ bool in_box(const double* x) {
            x[3] <= 1.0;
 }
 
+// Parameters of position x (NaN outside the box, so that the fitness path skips the particle).
+__device__ __forceinline__ void store_theta(const PsoDev& g, const double* x, double* __restrict__ theta) {
+    const bool inside = in_box(x);
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+        const double lo = g.box[2 * d], hi = g.box[2 * d + 1];
+        theta[d] = inside ? __dadd_rn(lo, __dmul_rn(__dsub_rn(hi, lo), x[d])) : NAN;
+    }
+}
+
 __global__ void pso_init_kernel(PsoDev g, PsoStateDev s) {
     const int64_t rows = (int64_t)g.n_runs * g.n_particles;
     const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -63,13 +73,14 @@ __global__ void pso_init_kernel(PsoDev g, PsoStateDev s) {
     }
     s.pbest_f[row] = -INFINITY;
     s.pbest_tc[row] = -1;
+    if (s.theta) store_theta(g, x, s.theta + 4 * row);
     if (p == 0) {
         if (s.iter) s.iter[run] = 0;
         if (s.evals) s.evals[run] = 0;
     }
 }
 
-// Parameters of every particle; NaN outside the box so that the fitness path skips it.
+// Parameters of every particle.
 __global__ void pso_theta_kernel(PsoDev g, PsoStateDev s, double* __restrict__ theta) {
     const int64_t rows = (int64_t)g.n_runs * g.n_particles;
     const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -77,22 +88,18 @@ __global__ void pso_theta_kernel(PsoDev g, PsoStateDev s, double* __restrict__ t
     double x[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) x[d] = s.x[4 * row + d];
-    const bool inside = in_box(x);
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        const double lo = g.box[2 * d], hi = g.box[2 * d + 1];
-        theta[4 * row + d] = inside ? __dadd_rn(lo, __dmul_rn(__dsub_rn(hi, lo), x[d])) : NAN;
-    }
+    store_theta(g, x, theta + 4 * row);
 }
 
 // One CTA per run, one thread per particle.
-__global__ void pso_update_kernel(PsoDev g, int32_t iter_arg, const double* __restrict__ fitness,
-                                  const int64_t* __restrict__ tc, PsoStateDev s) {
+__global__ void pso_update_kernel(PsoDev g, int32_t iter_arg, const double* fitness, const int64_t* tc,
+                                  PsoStateDev s) {
     __shared__ double s_pf[1024];
     __shared__ int s_count;
     const int run = blockIdx.x;
     const int p = threadIdx.x;
     const int P = g.n_particles;
+    chain_wait();
     const int it = s.iter ? s.iter[run] : iter_arg;
     if (p == 0) s_count = 0;
     __syncthreads();
@@ -143,6 +150,7 @@ __global__ void pso_update_kernel(PsoDev g, int32_t iter_arg, const double* __re
     if (p < P) {
 #pragma unroll
         for (int d = 0; d < 4; ++d) s.x[4 * row + d] = x[d];
+        if (s.theta) store_theta(g, x, s.theta + 4 * row);   // the next iteration's (one launch fewer)
     }
     if (p == 0) {
         if (s.iter) s.iter[run] = it + 1;
@@ -220,10 +228,9 @@ cudaError_t launch_pso_theta(const PsoDev& g, const PsoStateDev& s, double* thet
 }
 
 cudaError_t launch_pso_update(const PsoDev& g, int32_t iter, const double* fitness, const int64_t* tc,
-                              const PsoStateDev& s, cudaStream_t st) {
+                              const PsoStateDev& s, cudaStream_t st, bool chained) {
     const int threads = ((g.n_particles + 31) / 32) * 32;
-    pso_update_kernel<<<g.n_runs, threads, 0, st>>>(g, iter, fitness, tc, s);
-    return cudaGetLastError();
+    return launch_chained(chained, pso_update_kernel, dim3(g.n_runs), dim3(threads), 0, st, g, iter, fitness, tc, s);
 }
 
 cudaError_t launch_pso_result(const PsoDev& g, const PsoStateDev& s, fcas_search_result* out, cudaStream_t st) {

@@ -113,10 +113,11 @@ __device__ __forceinline__ c32x2 rot16_x2(c32x2 x) {
     }
 }
 
-// read-only load that does not allocate in L1 (pass B reads each intermediate element once)
+// load that does not allocate in L1 (pass B reads each intermediate element once); volatile, so that it stays
+// behind the wait for the kernel that writes the data
 __device__ __forceinline__ c32x2 ld_na(const c32x2* p) {
     c32x2 r;
-    asm("ld.global.nc.L1::no_allocate.v2.b64 {%0, %1}, [%2];" : "=l"(r.x.v), "=l"(r.y.v) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v2.b64 {%0, %1}, [%2];" : "=l"(r.x.v), "=l"(r.y.v) : "l"(p));
     return r;
 }
 // streamed store (evict-first): pass A's output is read back once, by pass B
