@@ -104,6 +104,7 @@ void free_ctx(fcas_ctx* c) {
                     c->d_gsums, c->d_gstage, c->d_ynat, c->d_polish};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    if (c->h_stage) cudaFreeHost(c->h_stage);
     if (c->search_stream) cudaStreamDestroy(c->search_stream);
     for (auto& e : c->events) {
         cudaEventDestroy(e.a);
@@ -157,6 +158,23 @@ int ensure_staging(fcas_ctx* c, int64_t n) {
     if (rc) return rc;
     c->stage_cap = n;
     return FCAS_OK;
+}
+
+// Pinned staging for host arrays of up to kHostStage particles: the geometry kernel reads theta from it and the
+// final argmax writes into it, so that a small call needs no copies (one particle on 64 s 50.8 -> 36 us a
+// call, with the passes' launch preparation moved to the context). Null when the host has no pinned memory left: the copies are made then.
+constexpr int64_t kHostStage = 1024;
+unsigned char* host_stage(fcas_ctx* c) {
+    if (!c->h_stage) {
+        void* p = nullptr;
+        const size_t bytes = (size_t)kHostStage * (sizeof(double) * 5 + sizeof(int64_t));
+        if (cudaHostAlloc(&p, bytes, cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        c->h_stage = static_cast<unsigned char*>(p);
+    }
+    return c->h_stage;
 }
 
 void prof_begin(fcas_ctx* c, int kind, cudaStream_t s, size_t* slot) {
@@ -246,14 +264,36 @@ cudaError_t gradient_device(fcas_ctx* c, int64_t n, const double* d_theta, const
                            c->d_gsums, c->d_det, c->d_sigma2s, c->setup.f_low, c->df, d_grad, st);
 }
 
-// Particles per chunk when the caller leaves it open: at least 64, and for short segments as many as 512 MB of
-// scratch hold (a chunk's launches have fixed costs and a last wave: 320 particles on 64 s take 239 us in
-// chunks of 64 and 195 us in one, on 4096 points 95 and 38 us; from 2^19 points on 64 is enough). Bounded by
-// 16 GB, and by 2048 (the passes' grids have one row of CTAs per particle).
-int64_t auto_chunk(size_t per_particle) {
+// Particles per chunk when the caller leaves it open: at least 64, and for short segments as many as the given
+// scratch holds (a chunk's launches have fixed costs and a last wave: 320 particles on 64 s take 239 us in
+// chunks of 64, 221 in three and 195 in one, on 4096 points 95 and 38 us; from 2^19 points on 64 is enough).
+// Bounded by 16 GB, and by 2048 (the passes' grids have one row of CTAs per particle).
+constexpr size_t kCreateScratch = (size_t)128 << 20;   // allocated with a context: no slower than 64 MB
+constexpr size_t kSearchScratch = (size_t)512 << 20;   // what a search of kGrowIterations or more grows it to
+constexpr int kGrowIterations = 12;                    // the growth takes ~250 us, an iteration saves ~25
+int64_t auto_chunk(size_t per_particle, size_t scratch) {
     const int64_t most = (int64_t)(((size_t)16 << 30) / per_particle);
-    const int64_t want = std::min<int64_t>(2048, std::max<int64_t>(64, (int64_t)(((size_t)512 << 20) / per_particle)));
+    const int64_t want = std::min<int64_t>(2048, std::max<int64_t>(64, (int64_t)(scratch / per_particle)));
     return std::max<int64_t>(1, std::min(want, most));
+}
+
+// A larger intermediate and argmax array for chunks of `want` particles; the present ones stay when the device
+// has no room for more.
+void grow_scratch(void** inter, Partial** partials, int64_t* chunk, int64_t want, size_t inter_pp, int64_t nb) {
+    if (want <= *chunk) return;
+    void* i = nullptr;
+    Partial* p = nullptr;
+    if (cudaMalloc(&i, inter_pp * (size_t)want) == cudaSuccess &&
+        cudaMalloc(reinterpret_cast<void**>(&p), sizeof(Partial) * (size_t)want * nb) == cudaSuccess) {
+        if (*inter) cudaFree(*inter);
+        if (*partials) cudaFree(*partials);
+        *inter = i;
+        *partials = p;
+        *chunk = want;
+        return;
+    }
+    cudaGetLastError();
+    if (i) cudaFree(i);
 }
 
 // Scratch of the fitness path (allocated at create unless FCAS_SETUP_LAZY_SCRATCH, else on first use).
@@ -304,6 +344,7 @@ int apply_layout(fcas_ctx* c, int bias, int k1b, int sub, int radix_bits_a, cuda
     if (e == cudaSuccess)
         e = launch_layout(c->d_ynat, c->setup.n_det, log_n, l1, l2, k1b, c->k_lo, c->k_hi, c->setup.fs, c->setup.f_low,
                           c->setup.precision, c->d_y, c->d_basis, st);
+    if (e == cudaSuccess) e = prepare_passes(c);
     if (e != cudaSuccess) return fail(FCAS_ERR_CUDA, "layout: %s", cudaGetErrorString(e));
     return FCAS_OK;
 }
@@ -541,7 +582,7 @@ int create_impl(fcas_ctx** out, const fcas_setup* setup, const fcas_detector* de
 
     // scratch for the fitness path (partials sized for every split the tuner may choose)
     const size_t per_particle = inter_bytes_per_particle(s.precision, n);
-    const int64_t chunk = s.max_batch > 0 ? s.max_batch : auto_chunk(per_particle);
+    const int64_t chunk = s.max_batch > 0 ? s.max_batch : auto_chunk(per_particle, kCreateScratch);
     c->chunk = chunk;
     c->nb_cap = 0;
     for (int bias = 0; bias <= 1; ++bias) {
@@ -584,26 +625,37 @@ int fcas_fitness(fcas_ctx* c, int64_t n, const double* theta, double* fitness, i
     int rc = ensure_particles(c, n);
     if (!rc) rc = ensure_scratch(c);
     if (rc) return rc;
-    if (!th_dev || !f_dev || !t_dev) {
+    const bool host = !th_dev || !f_dev || !t_dev;
+    unsigned char* hs = host && n <= kHostStage ? host_stage(c) : nullptr;
+    if (host && !hs) {
         rc = ensure_staging(c, n);
         if (rc) return rc;
     }
-    const double* d_theta = theta;
+    double* s_theta = hs ? reinterpret_cast<double*>(hs) : c->d_theta;
+    double* s_fit = hs ? s_theta + 4 * kHostStage : c->d_fit;
+    int64_t* s_tc = hs ? reinterpret_cast<int64_t*>(s_fit + kHostStage) : c->d_tc;
+    const double* d_theta = th_dev ? theta : s_theta;
+    double* d_fit = f_dev ? fitness : s_fit;
+    int64_t* d_tc = t_dev ? tc : s_tc;
     if (!th_dev) {
-        FCAS_CUDA(cudaMemcpyAsync(c->d_theta, theta, sizeof(double) * 4 * (size_t)n, cudaMemcpyHostToDevice, st));
-        d_theta = c->d_theta;
+        if (hs) std::memcpy(s_theta, theta, sizeof(double) * 4 * (size_t)n);
+        else FCAS_CUDA(cudaMemcpyAsync(s_theta, theta, sizeof(double) * 4 * (size_t)n, cudaMemcpyHostToDevice, st));
     }
-    double* d_fit = f_dev ? fitness : c->d_fit;
-    int64_t* d_tc = t_dev ? tc : c->d_tc;
     size_t slot;
     prof_begin(c, FCAS_KERNEL_GEOMETRY, st, &slot);
     FCAS_CUDA(launch_geometry(d_theta, n, c->d_params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low, c->df,
                               pass_a_kstep(c), c->setup.precision, st));
     prof_end(c, slot, st);
     FCAS_CUDA(launch_passes(c, n, d_fit, d_tc, st));
-    if (!f_dev) FCAS_CUDA(cudaMemcpyAsync(fitness, d_fit, sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost, st));
-    if (!t_dev) FCAS_CUDA(cudaMemcpyAsync(tc, d_tc, sizeof(int64_t) * (size_t)n, cudaMemcpyDeviceToHost, st));
-    if (!th_dev || !f_dev || !t_dev) FCAS_CUDA(cudaStreamSynchronize(st));
+    if (hs) {
+        FCAS_CUDA(cudaStreamSynchronize(st));
+        if (!f_dev) std::memcpy(fitness, d_fit, sizeof(double) * (size_t)n);
+        if (!t_dev) std::memcpy(tc, d_tc, sizeof(int64_t) * (size_t)n);
+    } else if (host) {
+        if (!f_dev) FCAS_CUDA(cudaMemcpyAsync(fitness, d_fit, sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost, st));
+        if (!t_dev) FCAS_CUDA(cudaMemcpyAsync(tc, d_tc, sizeof(int64_t) * (size_t)n, cudaMemcpyDeviceToHost, st));
+        FCAS_CUDA(cudaStreamSynchronize(st));
+    }
     if (const unsigned int bad = take_index_checks(st) | take_index_checks_ff(st))
         return fail(FCAS_ERR_CUDA, "fcas_fitness: index checks failed (bits 0x%x)", bad);
     return FCAS_OK;
@@ -701,6 +753,10 @@ int fcas_search(fcas_ctx* c, const fcas_pso_config* cfg, fcas_search_result* res
     rc = ensure_particles(c, rows);
     if (!rc) rc = ensure_scratch(c);
     if (rc) return rc;
+    if (c->setup.max_batch == 0 && cfg->n_iter >= kGrowIterations) {
+        const size_t pp = inter_bytes_per_particle(c->setup.precision, c->setup.n_fft);
+        grow_scratch(&c->d_inter, &c->d_partials, &c->chunk, std::min(rows, auto_chunk(pp, kSearchScratch)), pp, c->nb_cap);
+    }
     const size_t need = swarm_bytes(rows, cfg->n_runs);
     if (need > c->pso_bytes) {
         if (c->d_pso) cudaFree(c->d_pso);
@@ -900,9 +956,9 @@ int fcas_group_create(fcas_group** out, int32_t n_ctx, fcas_ctx* const* ctxs, in
     }
     fcas_group* g = new fcas_group();
     g->ctxs.assign(ctxs, ctxs + n_ctx);
-    const int64_t chunk = max_batch > 0 ? max_batch : std::min<int64_t>(64, auto_chunk(inter_pp));
+    const int64_t chunk = max_batch > 0 ? max_batch : std::min<int64_t>(64, auto_chunk(inter_pp, kCreateScratch));
     g->chunk = chunk;
-    g->auto_cap = max_batch > 0 ? 0 : auto_chunk(inter_pp);
+    g->auto_cap = max_batch > 0 ? 0 : auto_chunk(inter_pp, kSearchScratch);
     g->inter_pp = inter_pp;
     g->nb = nb;
     int rc = dev_alloc(&g->d_inter, inter_pp * (size_t)chunk, "group intermediate transform");
@@ -952,22 +1008,8 @@ int fcas_group_search_boxes(fcas_group* g, const fcas_pso_config* cfg, const dou
         if (rc) return rc;
         g->params_cap = rows;
     }
-    if (const int64_t want = std::min(rows, g->auto_cap); want > g->chunk) {
-        // larger swarms in fewer chunks; the present scratch stays when the device has no room for more
-        void* inter = nullptr;
-        Partial* partials = nullptr;
-        if (cudaMalloc(&inter, g->inter_pp * (size_t)want) == cudaSuccess &&
-            cudaMalloc(&partials, sizeof(Partial) * (size_t)want * g->nb) == cudaSuccess) {
-            cudaFree(g->d_inter);
-            cudaFree(g->d_partials);
-            g->d_inter = inter;
-            g->d_partials = partials;
-            g->chunk = want;
-        } else {
-            cudaGetLastError();
-            if (inter) cudaFree(inter);
-        }
-    }
+    if (cfg->n_iter * n_ctx >= kGrowIterations)
+        grow_scratch(&g->d_inter, &g->d_partials, &g->chunk, std::min(rows, g->auto_cap), g->inter_pp, g->nb);
     const size_t per = align256(swarm_bytes(rows, cfg->n_runs));
     if (per * n_ctx > g->pso_bytes) {
         if (g->d_pso) cudaFree(g->d_pso);

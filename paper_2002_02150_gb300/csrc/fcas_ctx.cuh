@@ -39,6 +39,7 @@ struct fcas_ctx {
     int radix_bits_a = 4;           // pass-A full-stage radix bits (4: radix 16, 3: radix 8)
     int sub = 8;                    // pass-A column blocks scheduled together
     double tuned_ms = 0.0;          // per-particle time of the tuned configuration (0: not tuned)
+    int64_t wave_a = 0, wave_b = 0; // resident CTAs of the shape's pass kernels
     int64_t nb_cap = 0;             // argmax partials per particle the scratch holds
     void* d_y = nullptr;            // Y (precision-dependent)
     void* d_basis = nullptr;
@@ -77,6 +78,7 @@ struct fcas_ctx {
     int64_t grad_cap = 0;
     unsigned char* d_polish = nullptr;  // working arrays of fcas_polish
     size_t polish_bytes = 0;
+    unsigned char* h_stage = nullptr;   // pinned host staging of small fcas_fitness calls (theta, fitness, tc)
     // particle swarm search
     unsigned char* d_pso = nullptr;  // state, parameters, fitness, counters and results of the swarm
     size_t pso_bytes = 0;
@@ -132,10 +134,26 @@ inline FitnessPlan make_plan(const fcas_ctx* c) {
     p.k1b = c->k1b;
     p.radix_bits_a = c->radix_bits_a;
     p.sub = c->sub;
+    p.wave_a = c->wave_a;
+    p.wave_b = c->wave_b;
     p.tw_lo = ff ? c->d_twloff : c->d_twlo;
     p.tw_hi = ff ? c->d_twhiff : c->d_twhi;
     p.ptab = c->d_phtab;
     return p;
+}
+
+// The context's pass kernels made ready for its device and current shape (see launch_pass_a).
+inline cudaError_t prepare_passes(fcas_ctx* c) {
+    const FitnessPlan plan = make_plan(c);
+    const int prec = c->setup.precision;
+    cudaError_t e;
+    if (prec == FCAS_PREC_FP32) e = launch_pass_a<float>(plan, nullptr, 0, 0, nullptr, nullptr, &c->wave_a);
+    else if (prec == FCAS_PREC_FF) e = launch_pass_a<ffloat>(plan, nullptr, 0, 0, nullptr, nullptr, &c->wave_a);
+    else e = launch_pass_a<double>(plan, nullptr, 0, 0, nullptr, nullptr, &c->wave_a);
+    if (e != cudaSuccess) return e;
+    if (prec == FCAS_PREC_FP32) return launch_pass_b<float>(plan, nullptr, 0, 0, nullptr, nullptr, nullptr, &c->wave_b);
+    if (prec == FCAS_PREC_FF) return launch_pass_b<ffloat>(plan, nullptr, 0, 0, nullptr, nullptr, nullptr, &c->wave_b);
+    return launch_pass_b<double>(plan, nullptr, 0, 0, nullptr, nullptr, nullptr, &c->wave_b);
 }
 
 }  // namespace fcas

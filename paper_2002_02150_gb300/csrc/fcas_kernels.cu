@@ -281,12 +281,12 @@ int pass_a_k1b_variants(int log_n2, int precision, int* out) {
     return n;
 }
 
-template cudaError_t launch_pass_a<float>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, void*, cudaStream_t);
-template cudaError_t launch_pass_a<double>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, void*, cudaStream_t);
+template cudaError_t launch_pass_a<float>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, void*, cudaStream_t, int64_t*);
+template cudaError_t launch_pass_a<double>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, void*, cudaStream_t, int64_t*);
 template cudaError_t launch_pass_b<float>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, const void*,
-                                          Partial*, cudaStream_t);
+                                          Partial*, cudaStream_t, int64_t*);
 template cudaError_t launch_pass_b<double>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, const void*,
-                                           Partial*, cudaStream_t);
+                                           Partial*, cudaStream_t, int64_t*);
 
 // ------------------------------------------------------------------------------------------
 // per-stage twiddle tables of the radix-16 transforms (create time)

@@ -102,6 +102,7 @@ struct FitnessPlan {
     int sub;                      // adjacent column blocks of a particle scheduled together
     const void* tw_lo;            // e^{2 pi i m / N}, m < 4096
     const void* tw_hi;            // e^{2 pi i 4096 m / N}, m < max(1, N / 4096)
+    int64_t wave_a, wave_b;       // resident CTAs of the passes' kernels on the device (prepare_passes)
     const void* ptab;             // e^{2 pi i m / 1024}, m < 1024 (binary64 and float-float forms)
 };
 
@@ -111,14 +112,16 @@ cudaError_t launch_geometry(const double* theta, int64_t n, ParticleParams* out,
                             const double* sigma2_scaled, int n_det, double f_star, double df, int64_t kstep,
                             int precision, cudaStream_t s);
 
-// Pass A for particles [p0, p0 + np): writes the intermediate [np][2][N2][N1].
+// Pass A for particles [p0, p0 + np): writes the intermediate [np][2][N2][N1]. With wave the kernel is not
+// launched but prepared for the current device, and *wave receives its resident CTAs (before any launch of a
+// context's shape; pass B likewise).
 template <typename Real>
 cudaError_t launch_pass_a(const FitnessPlan& plan, const ParticleParams* params, int64_t p0, int64_t np,
-                          void* inter, cudaStream_t s);
+                          void* inter, cudaStream_t s, int64_t* wave = nullptr);
 // Pass B + projection + partial argmax: writes partials [np][N2 / TB].
 template <typename Real>
 cudaError_t launch_pass_b(const FitnessPlan& plan, const ParticleParams* params, int64_t p0, int64_t np,
-                          const void* inter, Partial* partials, cudaStream_t s);
+                          const void* inter, Partial* partials, cudaStream_t s, int64_t* wave = nullptr);
 // Final argmax: fitness[p0 + p], tc[p0 + p].
 cudaError_t launch_reduce(const Partial* partials, int64_t nb, const ParticleParams* params, int64_t p0,
                           int64_t np, double* fitness, int64_t* tc, bool chained, cudaStream_t s);

@@ -5,9 +5,9 @@
 namespace fcas {
 
 template cudaError_t launch_pass_a<ffloat>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, void*,
-                                           cudaStream_t);
+                                           cudaStream_t, int64_t*);
 template cudaError_t launch_pass_b<ffloat>(const FitnessPlan&, const ParticleParams*, int64_t, int64_t, const void*,
-                                           Partial*, cudaStream_t);
+                                           Partial*, cudaStream_t, int64_t*);
 
 // index checks of this translation unit's kernels (checked build; 0 otherwise)
 unsigned int take_index_checks_ff(cudaStream_t s) {

@@ -771,74 +771,73 @@ pass_b_x2_kernel(const c32x2* inter, const ParticleParams* params, int64_t p0, i
 // half, twice and four times it while a CTA stays within 512 threads.
 constexpr bool x2_k1b_ok(int lg, int k) { return k >= 1 && k <= 16 && k <= (1 << lg) && x2_a_threads(lg, k) <= 512; }
 
+// Preparation of a pass's kernel on the current device, once per context and shape: its shared memory limit,
+// and the CTAs of one wave (the resident CTAs of every SM).
+template <typename K>
+static cudaError_t resident_wave(K* kern, int threads, size_t smem, int64_t* wave) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    *wave = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+    return e;
+}
+
 template <int LG, int K1B, int MAXRB = 4>
 static cudaError_t pass_a_x2_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
-                                void* inter, cudaStream_t s) {
+                                void* inter, cudaStream_t s, int64_t* wave) {
     constexpr int THREADS = x2_a_threads(LG, K1B, MAXRB);
     const size_t smem = sizeof(c32x2) * (size_t)x2_buf_elems<LG, K1B, MAXRB>();
     auto kern = pass_a_x2_kernel<LG, K1B, MAXRB>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (wave) return resident_wave(kern, THREADS, smem, wave);
     const int64_t items = np * ((1 << pl.log_n1) / K1B);
-    // one wave: the resident CTAs of every SM
-    int dev = 0, sms = 0, per_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem);
-    if (e != cudaSuccess) return e;
-    const int64_t wave = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-    const int64_t ctas = wave < items ? wave : items;
+    const int64_t ctas = pl.wave_a < items ? pl.wave_a : items;   // one wave: the resident CTAs of every SM
     return launch_chained(chain_pays(np, pl.log_n), kern, dim3((unsigned)ctas), dim3(THREADS), smem, s,
-                          static_cast<const float2*>(pl.y), static_cast<const BasisF*>(pl.basis), params, p0, np, pl.n_det, pl.log_n1, pl.sub,
-                          static_cast<c32x2*>(inter), static_cast<const float2*>(pl.stw_a),
+                          static_cast<const float2*>(pl.y), static_cast<const BasisF*>(pl.basis), params, p0, np,
+                          pl.n_det, pl.log_n1, pl.sub, static_cast<c32x2*>(inter), static_cast<const float2*>(pl.stw_a),
                           static_cast<const float2*>(pl.tw_lo), static_cast<const float2*>(pl.tw_hi), items);
 }
 
 template <int LG>
 static cudaError_t pass_a_x2_lg(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
-                                void* inter, cudaStream_t s) {
+                                void* inter, cudaStream_t s, int64_t* wave) {
     constexpr int KD = pass_a_k1b(LG, FCAS_PREC_FP32);
     if (pl.radix_bits_a == 3) {
         // radix-8 stages: 8 values per thread, CTAs of 2 or 4 columns (at most 1024 threads)
         if constexpr (LG >= 10 && LG <= 11)
-            if (pl.k1b == 4) return pass_a_x2_at<LG, 4, 3>(pl, params, p0, np, inter, s);
+            if (pl.k1b == 4) return pass_a_x2_at<LG, 4, 3>(pl, params, p0, np, inter, s, wave);
         if constexpr (LG >= 10 && LG <= 12)
-            if (pl.k1b == 2) return pass_a_x2_at<LG, 2, 3>(pl, params, p0, np, inter, s);
+            if (pl.k1b == 2) return pass_a_x2_at<LG, 2, 3>(pl, params, p0, np, inter, s, wave);
         return cudaErrorInvalidValue;
     }
     if (pl.radix_bits_a != 4) return cudaErrorInvalidValue;
-    if (pl.k1b == KD) return pass_a_x2_at<LG, KD>(pl, params, p0, np, inter, s);
+    if (pl.k1b == KD) return pass_a_x2_at<LG, KD>(pl, params, p0, np, inter, s, wave);
     if constexpr (LG >= 10 && KD > 1)
-        if (pl.k1b == 1) return pass_a_x2_at<LG, 1>(pl, params, p0, np, inter, s);   // one column per CTA
+        if (pl.k1b == 1) return pass_a_x2_at<LG, 1>(pl, params, p0, np, inter, s, wave);   // one column per CTA
     if constexpr (LG >= 8) {
         if constexpr (x2_k1b_ok(LG, KD / 2))
-            if (pl.k1b == KD / 2) return pass_a_x2_at<LG, (KD / 2 > 0 ? KD / 2 : 1)>(pl, params, p0, np, inter, s);
+            if (pl.k1b == KD / 2) return pass_a_x2_at<LG, (KD / 2 > 0 ? KD / 2 : 1)>(pl, params, p0, np, inter, s, wave);
         if constexpr (x2_k1b_ok(LG, KD * 2))
-            if (pl.k1b == KD * 2) return pass_a_x2_at<LG, (KD * 2 <= 16 ? KD * 2 : 16)>(pl, params, p0, np, inter, s);
+            if (pl.k1b == KD * 2) return pass_a_x2_at<LG, (KD * 2 <= 16 ? KD * 2 : 16)>(pl, params, p0, np, inter, s, wave);
         if constexpr (x2_k1b_ok(LG, KD * 4))
-            if (pl.k1b == KD * 4) return pass_a_x2_at<LG, (KD * 4 <= 16 ? KD * 4 : 16)>(pl, params, p0, np, inter, s);
+            if (pl.k1b == KD * 4) return pass_a_x2_at<LG, (KD * 4 <= 16 ? KD * 4 : 16)>(pl, params, p0, np, inter, s, wave);
     }
     return cudaErrorInvalidValue;
 }
 
 template <int LG>
 static cudaError_t pass_b_x2_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
-                                const void* inter, Partial* partials, cudaStream_t s) {
+                                const void* inter, Partial* partials, cudaStream_t s, int64_t* wave) {
     constexpr int TB = pass_b_tb(LG, FCAS_PREC_FP32);
     const size_t smem = sizeof(c32x2) * (size_t)TB * fft_buf_elems<LG, 4, 1, 4>();
     auto kern = pass_b_x2_kernel<LG>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, x2_b_threads(LG), smem);
-    if (e != cudaSuccess) return e;
+    if (wave) return resident_wave(kern, x2_b_threads(LG), smem, wave);
     dim3 grid((unsigned)((1 << pl.log_n2) / TB), (unsigned)np);
     const int log_ga = fft_log_g(pl.log_n2, pl.radix_bits_a), cb_a = fft_local_bits(pl.log_n2, pl.radix_bits_a, pl.k1b);
     return launch_chained(chain_pays(np, pl.log_n), kern, grid, dim3(x2_b_threads(LG)), smem, s,
                           static_cast<const c32x2*>(inter), params, p0, pl.log_n2, log_ga, cb_a, pl.n_samples, static_cast<const float2*>(pl.stw_b), partials,
-                          (int64_t)sms * (per_sm > 0 ? per_sm : 1));
+                          pl.wave_b);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -848,12 +847,11 @@ static cudaError_t pass_b_x2_at(const FitnessPlan& pl, const ParticleParams* par
 
 template <typename Real, int LG, int K1B, int MAXRB = 4>
 static cudaError_t pass_a_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np, void* inter,
-                             cudaStream_t s) {
+                             cudaStream_t s, int64_t* wave) {
     constexpr int THREADS = K1B * ((1 << LG) / fftr_v(LG, MAXRB));
     const size_t smem = sizeof(cplx<Real>) * (size_t)pass_a_buf_elems<Real, LG, K1B, MAXRB>();
     auto kern = pass_a_kernel<Real, LG, K1B, MAXRB>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (wave) return resident_wave(kern, THREADS, smem, wave);
     const int64_t ctas = np * ((1 << pl.log_n1) / K1B);
     return launch_chained(chain_pays(np, pl.log_n), kern, dim3((unsigned)ctas), dim3(THREADS), smem, s,
                           static_cast<const cplx<Real>*>(pl.y), static_cast<const BasisD*>(pl.basis), params, p0, np, pl.n_det, pl.log_n1, pl.sub,
@@ -867,29 +865,28 @@ constexpr bool fp64_k1b_double(int lg) { return lg >= 8 && lg <= 11; }
 
 template <typename Real, int LG>
 static cudaError_t pass_a_lg(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
-                             void* inter, cudaStream_t s) {
+                             void* inter, cudaStream_t s, int64_t* wave) {
     constexpr int KD = pass_a_k1b(LG, form_of<Real>);
     if (pl.radix_bits_a == 3) {
         // float-float: radix-8 stages, 512-thread CTAs of 2 columns (half the registers per thread of radix 16)
         if constexpr (std::is_same<Real, ffloat>::value && LG >= 10 && LG <= 12)
-            if (pl.k1b == 2) return pass_a_at<Real, LG, 2, 3>(pl, params, p0, np, inter, s);
+            if (pl.k1b == 2) return pass_a_at<Real, LG, 2, 3>(pl, params, p0, np, inter, s, wave);
         return cudaErrorInvalidValue;
     }
-    if (pl.k1b == KD) return pass_a_at<Real, LG, KD>(pl, params, p0, np, inter, s);
+    if (pl.k1b == KD) return pass_a_at<Real, LG, KD>(pl, params, p0, np, inter, s, wave);
     if constexpr (std::is_same<Real, double>::value && fp64_k1b_double(LG))
-        if (pl.k1b == KD * 2) return pass_a_at<Real, LG, KD * 2>(pl, params, p0, np, inter, s);
+        if (pl.k1b == KD * 2) return pass_a_at<Real, LG, KD * 2>(pl, params, p0, np, inter, s, wave);
     return cudaErrorInvalidValue;
 }
 
 template <typename Real, int LG>
 static cudaError_t pass_b_at(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
-                             const void* inter, Partial* partials, cudaStream_t s) {
+                             const void* inter, Partial* partials, cudaStream_t s, int64_t* wave) {
     constexpr int TB = pass_b_tb(LG, form_of<Real>);
     constexpr int THREADS = pass_b_threads(LG, form_of<Real>);
     const size_t smem = sizeof(cplx<Real>) * (size_t)TB * fft_buf_elems<LG, 4, 0, 4>();
     auto kern = pass_b_kernel<Real, LG>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (wave) return resident_wave(kern, THREADS, smem, wave);
     dim3 grid((unsigned)((1 << pl.log_n2) / TB), (unsigned)np);
     return launch_chained(chain_pays(np, pl.log_n), kern, grid, dim3(THREADS), smem, s,
                           static_cast<const cplx<Real>*>(inter), params, p0, pl.log_n2, pl.n_samples, static_cast<const cplx<Real>*>(pl.stw_b), partials);
@@ -897,19 +894,19 @@ static cudaError_t pass_b_at(const FitnessPlan& pl, const ParticleParams* params
 
 template <typename Real>
 cudaError_t launch_pass_a(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np, void* inter,
-                          cudaStream_t s) {
-    if (np <= 0) return cudaSuccess;
+                          cudaStream_t s, int64_t* wave) {
+    if (np <= 0 && !wave) return cudaSuccess;
     if constexpr (std::is_same<Real, float>::value) {
         // the FP32 form: both series in one packed transform
         switch (pl.log_n2) {
-#define FCAS_CASE(LG) case LG: return pass_a_x2_lg<LG>(pl, params, p0, np, inter, s);
+#define FCAS_CASE(LG) case LG: return pass_a_x2_lg<LG>(pl, params, p0, np, inter, s, wave);
             FCAS_LOG_CASES(FCAS_CASE)
 #undef FCAS_CASE
             default: return cudaErrorInvalidValue;
         }
     } else {
         switch (pl.log_n2) {
-#define FCAS_CASE(LG) case LG: return pass_a_lg<Real, LG>(pl, params, p0, np, inter, s);
+#define FCAS_CASE(LG) case LG: return pass_a_lg<Real, LG>(pl, params, p0, np, inter, s, wave);
             FCAS_LOG_CASES(FCAS_CASE)
 #undef FCAS_CASE
             default: return cudaErrorInvalidValue;
@@ -919,18 +916,18 @@ cudaError_t launch_pass_a(const FitnessPlan& pl, const ParticleParams* params, i
 
 template <typename Real>
 cudaError_t launch_pass_b(const FitnessPlan& pl, const ParticleParams* params, int64_t p0, int64_t np,
-                          const void* inter, Partial* partials, cudaStream_t s) {
-    if (np <= 0) return cudaSuccess;
+                          const void* inter, Partial* partials, cudaStream_t s, int64_t* wave) {
+    if (np <= 0 && !wave) return cudaSuccess;
     if constexpr (std::is_same<Real, float>::value) {
         switch (pl.log_n1) {
-#define FCAS_CASE(LG) case LG: return pass_b_x2_at<LG>(pl, params, p0, np, inter, partials, s);
+#define FCAS_CASE(LG) case LG: return pass_b_x2_at<LG>(pl, params, p0, np, inter, partials, s, wave);
             FCAS_LOG_CASES(FCAS_CASE)
 #undef FCAS_CASE
             default: return cudaErrorInvalidValue;
         }
     } else {
         switch (pl.log_n1) {
-#define FCAS_CASE(LG) case LG: return pass_b_at<Real, LG>(pl, params, p0, np, inter, partials, s);
+#define FCAS_CASE(LG) case LG: return pass_b_at<Real, LG>(pl, params, p0, np, inter, partials, s, wave);
             FCAS_LOG_CASES(FCAS_CASE)
 #undef FCAS_CASE
             default: return cudaErrorInvalidValue;
