@@ -221,35 +221,24 @@ grad_sums_kernel(const cplx<Real>* __restrict__ y, bool y_ff, const Basis<Real>*
     }
 }
 
-// forward-mode dual number for the chirp-coefficient derivatives
-struct Dual {
-    double v, d;
-};
-__device__ __forceinline__ Dual operator+(Dual a, Dual b) { return {a.v + b.v, a.d + b.d}; }
-__device__ __forceinline__ Dual operator*(Dual a, Dual b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
-__device__ __forceinline__ Dual operator*(double s, Dual a) { return {s * a.v, s * a.d}; }
-__device__ __forceinline__ Dual operator/(Dual a, Dual b) { return {a.v / b.v, (a.d * b.v - a.v * b.d) / (b.v * b.v)}; }
-__device__ __forceinline__ Dual dpow(Dual a, double e) {
-    const double pv = pow(a.v, e);
-    return {pv, e * pow(a.v, e - 1.0) * a.d};
-}
-
-// c_j(tau0, tau1.5) (turns) with derivative along (dt0, dt15), as in the geometry kernel
-__device__ void chirp_coeffs_dual(double tau0, double tau15, double dt0, double dt15, double f_star, Dual c[4]) {
+// d c_j (turns) along (dt0, dt15) for the coefficients of the geometry kernel, by logarithmic derivatives:
+// x ~ tau1.5 / tau0, eta ~ x^-2/3 / tau1.5, tau1 ~ P1(eta) / (eta x), tau2 ~ P2(eta) / (eta x^1/3) (one cube
+// root where differentiating the powers term by term took four general powers: the kernel 28 -> 17 us).
+__device__ void chirp_coeff_derivatives(double tau0, double tau15, double dt0, double dt15, double f_star, double dc[4]) {
     const double pi = 3.14159265358979323846;
-    const Dual t0{tau0, dt0}, t15{tau15, dt15};
-    const Dual x = (5.0 / (32.0 * pi)) * (t15 / t0);
-    const Dual eta = dpow(x, -2.0 / 3.0) / ((8.0 * f_star) * t15);
-    const Dual one{1.0, 0.0};
-    const Dual tau1 = (5.0 / (192.0 * pi * f_star)) * ((Dual{743.0 / 336.0, 0.0} + (11.0 / 4.0) * eta) / (eta * x));
-    const Dual tau2 = (5.0 / (128.0 * pi * f_star)) *
-                      ((Dual{3058673.0 / 1016064.0, 0.0} + (5429.0 / 1008.0) * eta + (617.0 / 144.0) * (eta * eta)) /
-                       (eta * dpow(x, 1.0 / 3.0)));
-    (void)one;
-    c[0] = (0.6 * f_star) * t0;
-    c[1] = f_star * tau1;
-    c[2] = (-1.5 * f_star) * t15;
-    c[3] = (3.0 * f_star) * tau2;
+    const double x = 5.0 * tau15 / (32.0 * pi * tau0);
+    const double cx = cbrt(x);
+    const double eta = 1.0 / (cx * cx * 8.0 * f_star * tau15);
+    const double dl15 = dt15 / tau15;
+    const double dlx = dl15 - dt0 / tau0;             // d ln x
+    const double dle = -2.0 / 3.0 * dlx - dl15;       // d ln eta
+    const double p1 = 743.0 / 336.0 + 11.0 / 4.0 * eta;
+    const double p2 = 3058673.0 / 1016064.0 + (5429.0 / 1008.0 + 617.0 / 144.0 * eta) * eta;
+    const double t1 = 5.0 / (192.0 * pi * f_star * eta * x), t2 = 5.0 / (128.0 * pi * f_star * eta * cx);
+    dc[0] = 0.6 * f_star * dt0;
+    dc[1] = f_star * t1 * (11.0 / 4.0 * eta * dle - p1 * (dle + dlx));
+    dc[2] = -1.5 * f_star * dt15;
+    dc[3] = 3.0 * f_star * t2 * ((5429.0 / 1008.0 + 617.0 / 72.0 * eta) * eta * dle - p2 * (dle + 1.0 / 3.0 * dlx));
 }
 
 // One CTA per particle: the segments' partial sums are added in order by all threads, the sky geometry
@@ -286,9 +275,7 @@ grad_final_kernel(const double* __restrict__ theta, const int64_t* __restrict__ 
             acc += part[((p * n_det + v / kGradSums) * nseg + seg) * kGradSums + v % kGradSums];
     spart[tid] = acc;
     if (tid >= 32 && tid < 34) {
-        Dual c[4];
-        chirp_coeffs_dual(tau0, tau15, tid == 32 ? 1.0 : 0.0, tid == 33 ? 1.0 : 0.0, f_star, c);
-        for (int j = 0; j < 4; ++j) dc[tid - 32][j] = c[j].d;
+        chirp_coeff_derivatives(tau0, tau15, tid == 32 ? 1.0 : 0.0, tid == 33 ? 1.0 : 0.0, f_star, dc[tid - 32]);
     }
     if (tid < 32) {
         // lane 0 takes sin and cos of alpha, lane 1 of delta
