@@ -1008,7 +1008,7 @@ int fcas_group_search_boxes(fcas_group* g, const fcas_pso_config* cfg, const dou
         if (rc) return rc;
         g->params_cap = rows;
     }
-    if (cfg->n_iter * n_ctx >= kGrowIterations)
+    if ((int64_t)cfg->n_iter * n_ctx >= kGrowIterations)
         grow_scratch(&g->d_inter, &g->d_partials, &g->chunk, std::min(rows, g->auto_cap), g->inter_pp, g->nb);
     const size_t per = align256(swarm_bytes(rows, cfg->n_runs));
     if (per * n_ctx > g->pso_bytes) {
