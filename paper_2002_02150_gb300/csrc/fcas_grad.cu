@@ -103,8 +103,9 @@ __device__ __forceinline__ void warp_sums(Acc (&v)[kGradVals], int lane) {
 // column blocks (blks of them) at the rows k2 that hold band bins. The segments do not depend on the
 // number of particles, so neither do the sums' bits. One CTA per (particle, detector) over the whole band
 // left most SMs idle for a few particles and its twelve binary64 sums per bin held the binary64 unit: 8
-// particles of the 60-min workload 42.9 -> 1.36 ms a call, forward and backward of 40 particles on 64 s
-// 799 -> 398 us. Bound now by FP32 issue (about 200 instructions per bin and detector).
+// particles of the 60-min workload 42.9 -> 1.36 ms a call, and 1.32 -> 1.02 ms with each bin's loads one bin
+// ahead; forward and backward of 40 particles on 64 s 799 -> 398 us. Bound now by FP32 issue (about 200
+// instructions per bin and detector).
 template <typename Real>
 __global__ void __launch_bounds__(kGradThreads, 2)
 grad_sums_kernel(const cplx<Real>* __restrict__ y, bool y_ff, const Basis<Real>* __restrict__ basis,
@@ -134,11 +135,31 @@ grad_sums_kernel(const cplx<Real>* __restrict__ y, bool y_ff, const Basis<Real>*
         for (int blk = seg * blks; blk < (seg + 1) * blks; ++blk) {
             const Basis<Real>* bb = basis + blk * per_blk;
             const cplx<Real>* yb = y + ((int64_t)blk * n_det + i0) * per_blk;
-            for (int r = threadIdx.x; r < rows << log_k1b; r += kGradThreads) {
-                const int e = r + (k2_lo << log_k1b);
+            // FP32: the next bin's basis and spectrum are requested before this bin's arithmetic
+            const int count = rows << log_k1b, e0 = k2_lo << log_k1b;
+            Basis<Real> bn{};
+            cplx<Real> yn[kGradDet] = {};
+            auto request = [&](int r) {
+                if (r >= count) return;
+                bn = bb[e0 + r];
+#pragma unroll
+                for (int u = 0; u < kGradDet; ++u)
+                    if (u < nd) yn[u] = yb[u * per_blk + e0 + r];
+            };
+            if constexpr (sizeof(Real) == 4) request(threadIdx.x);
+            for (int r = threadIdx.x; r < count; r += kGradThreads) {
+                const int e = r + e0;
                 const int k = blk * k1b + (e & (k1b - 1)) + ((e >> log_k1b) << log_n1);
+                Basis<Real> b;
+                cplx<Real> yc[kGradDet];
+                if constexpr (sizeof(Real) == 4) {
+                    b = bn;
+#pragma unroll
+                    for (int u = 0; u < kGradDet; ++u) yc[u] = yn[u];
+                    request(r + kGradThreads);
+                }
                 if (k < k_lo || k > k_hi) continue;
-                const Basis<Real> b = bb[e];
+                if constexpr (sizeof(Real) != 4) b = bb[e];
                 const unsigned m = ((unsigned)k * tu) & nmask;   // k t mod N (the low bits of the product)
                 if constexpr (sizeof(Real) == 4) {
                     const float shift = (float)m * __int_as_float((127 - log_n) << 23);   // m / N, exact
@@ -151,7 +172,7 @@ grad_sums_kernel(const cplx<Real>* __restrict__ y, bool y_ff, const Basis<Real>*
 #pragma unroll
                     for (int u = 0; u < kGradDet; ++u) {
                         if (u >= nd) break;
-                        const float2 yv = yb[u * per_blk + e];
+                        const float2 yv = yc[u];
                         float th = s + frac_mul_ff(kk, 0.0f, pp.dh[i0 + u], pp.dl[i0 + u]) + shift;
                         th -= rintf(th);
                         float sn, cs;
