@@ -337,8 +337,9 @@ int apply_layout(fcas_ctx* c, int bias, int k1b, int sub, int radix_bits_a, cuda
     c->radix_bits_a = radix_bits_a;
     c->nb_partials = nb;
     const bool local = c->setup.precision == FCAS_PREC_FP32;   // the form with warp-local exchanges
-    cudaError_t e = launch_stage_tables(l2, radix_bits_a, local ? k1b : 0, c->d_stw_a64, c->d_stw_a32, st);
-    if (e == cudaSuccess) e = launch_stage_tables(l1, 4, local ? 1 : 0, c->d_stw_b64, c->d_stw_b32, st);
+    const bool lf = c->setup.precision == FCAS_PREC_FP64;
+    cudaError_t e = launch_stage_tables(l2, radix_bits_a, local ? k1b : 0, lf, c->d_stw_a64, c->d_stw_a32, st);
+    if (e == cudaSuccess) e = launch_stage_tables(l1, 4, local ? 1 : 0, lf, c->d_stw_b64, c->d_stw_b32, st);
     if (e == cudaSuccess && c->d_stw_aff) e = launch_split_ff(c->d_stw_a64, c->d_stw_aff, (int64_t)1 << l2, st);
     if (e == cudaSuccess && c->d_stw_bff) e = launch_split_ff(c->d_stw_b64, c->d_stw_bff, (int64_t)1 << l1, st);
     if (e == cudaSuccess)

@@ -13,7 +13,8 @@
 // The threads that work on one residue class of the index (modulo 16 after the first radix-16 stage) are
 // consecutive, so that from the second exchange on all data stay within a warp: those exchanges need no
 // barrier of the CTA (see fft_local_bits).
-// Twiddles come from a per-length table laid out stage by stage as
+// Twiddles (of all forms but binary64, whose fused butterflies have their own entries: lf_dft) come from a
+// per-length table laid out stage by stage as
 //   T[(Ns - 1) + (r - 1) Ns + P(jm)] = e^{2 pi i r jm / (Ns R)},   r = 1..R-1, jm = 0..Ns-1,
 // with P the order in which the stage's threads take jm (fft_tw_pos), so that a warp reads consecutive
 // entries; the stages together use L - 1 entries.
@@ -280,6 +281,55 @@ __device__ __forceinline__ void dft_r(C (&a)[R]) {
     }
 }
 
+// Twiddled stage of the binary64 form: sum_r a[r] w^r e^{2 pi i r u / R} as radix-2 levels whose products are
+// fused into the additions (Linzer & Feig 1993): with z = c (1 + i t), z O = c ((O.x - t O.y) + i (O.y + t O.x)),
+// so that E + z O and E - z O take six multiply-adds where a product and two additions take eight operations
+// (192 instead of 220 per radix-16 butterfly with its twiddles; the binary64 unit is what this form waits for:
+// 60-min passes 11.84 -> 10.48 ms per 4 particles, 64-s ones 753 -> 689 us per 40, the same errors).
+// Level l combines the sub-transforms s and s + R/2^l with z = w^(R/2^l) e^{2 pi i u / 2^l}; u in the upper half
+// of its range is the lower half's z times i. The (c, t) of the lower halves are tabulated (fft_lf_entry):
+// entry 0 for l = 1, 2^(l-2) + u for l >= 2, each a run of ns values. Where c is 0 the table holds 2^-60 and
+// t = 2^60, whose product is the sine; rounding errors scale with c t = sin, so a large t costs nothing.
+template <int R>
+__device__ __forceinline__ void lf_dft(double2 (&a)[R], const double2* __restrict__ t, int ns, int room) {
+#pragma unroll
+    for (int l = 1; (1 << l) <= R; ++l) {
+        const int S = R >> l, half = 1 << (l - 1);
+        double2 n[R];
+#pragma unroll
+        for (int u = 0; u < half; ++u) {
+            const bool rot = l >= 2 && u >= half / 2;
+            const int e = l == 1 ? 0 : half / 2 + (rot ? u - half / 2 : u);
+            double2 z = make_double2(1.0, 0.0);
+            if (FCAS_CHECK(e * ns < room, kCheckTwiddle)) z = __ldg(t + e * ns);
+#pragma unroll
+            for (int q = 0; q < S; ++q) {
+                const double2 E = a[q + u * 2 * S], O = a[q + S + u * 2 * S];
+                const double x = fma(-z.y, O.y, O.x), y = fma(z.y, O.x, O.y);
+                if (rot) {
+                    n[q + u * S] = make_double2(fma(-z.x, y, E.x), fma(z.x, x, E.y));
+                    n[q + (u + half) * S] = make_double2(fma(z.x, y, E.x), fma(-z.x, x, E.y));
+                } else {
+                    n[q + u * S] = make_double2(fma(z.x, x, E.x), fma(z.x, y, E.y));
+                    n[q + (u + half) * S] = make_double2(fma(-z.x, x, E.x), fma(-z.x, y, E.y));
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q) a[q] = n[q];
+    }
+}
+// turns of entry e of lf_dft's table at jm, as a numerator over ns R
+__host__ __device__ constexpr long long fft_lf_entry(int e, long long jm, long long ns, int r_) {
+    int l = 1;
+    while (l < 2 || (1 << (l - 1)) <= e) {
+        if (e == 0) break;
+        ++l;
+    }
+    const int u = e == 0 ? 0 : e - (1 << (l - 2));
+    return jm * (r_ >> l) + (long long)u * ((ns * r_) >> l);
+}
+
 // LH (first stage only): the upper half of the input (v[V/2 ..]) is zero. TWL: the stage twiddles
 // w^r (r < 4) and w^{4h} come from the table and the rest as one product each (instead of w and w^4
 // loaded and the other powers formed by products); fewer instructions, a few more registers.
@@ -330,7 +380,11 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
         C a[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) a[r] = v[h + r * T];
-        if constexpr (NS > 1) {
+        if constexpr (NS > 1 && std::is_same<Real, double>::value) {
+            static_assert(S > 0, "the binary64 passes transform with e^{+i}");
+            const int jm = jj & (NS - 1);
+            lf_dft<R>(a, stw + (NS - 1) + jm, NS, L - (NS - 1) - jm);
+        } else if constexpr (NS > 1) {
             // the twiddle's place P(jm) from the thread's own number: j itself where the block holds G entries
             // or more, class-major within the block otherwise
             constexpr int LG = fft_log_g(LOG_L, MAXRB);
@@ -338,7 +392,7 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
                            : NS >= G                ? jr + h * G
                                                     : (jr >> (LG - CB)) * (NS >> CB) + (jr & ((NS >> CB) - 1));
             const W* t = stw + (NS - 1) + jm;
-            constexpr bool kLoadAll = std::is_same<Real, ffloat>::value || std::is_same<Real, double>::value;
+            constexpr bool kLoadAll = std::is_same<Real, ffloat>::value;
             if constexpr (R >= 8 && TWL && !kLoadAll) {
                 W wl[4], wh[R / 4];
                 wl[0] = wh[0] = tw_one(W{});
@@ -365,8 +419,7 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
                 }
             } else if constexpr (R >= 8 && !kLoadAll) {
                 // w^r for r = 1..R-1 from two table entries: w and w^4 (powers by products, <= 3 roundings);
-                // the binary64 and float-float forms load every power instead (a product costs more than
-                // a load there: binary64 60-min pass B 5.82 -> 5.05 ms per 4 particles)
+                // the float-float form loads every power instead (a double-word product costs more than a load)
                 W w1 = tw_one(W{}), w4 = w1;
                 if (FCAS_CHECK((NS - 1) + jm + 3 * NS < L, kCheckTwiddle)) {
                     w1 = ldg_c(t);
@@ -401,7 +454,7 @@ __device__ __forceinline__ void fftr_stage(cplx<Real> (&v)[fftr_v(LOG_L, MAXRB)]
             }
         }
         // with R = V (T = 1) the zero upper half of the first stage is the upper half of a[]
-        dft_r<S, R, LH && FIRST && T == 1 && R >= 8>(a);
+        if constexpr (NS == 1 || !std::is_same<Real, double>::value) dft_r<S, R, LH && FIRST && T == 1 && R >= 8>(a);
 #pragma unroll
         for (int r = 0; r < R; ++r) v[h + r * T] = a[r];
     }

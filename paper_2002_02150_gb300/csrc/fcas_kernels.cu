@@ -292,7 +292,8 @@ template cudaError_t launch_pass_b<double>(const FitnessPlan&, const ParticlePar
 // per-stage twiddle tables of the radix-16 transforms (create time)
 // ------------------------------------------------------------------------------------------
 // entry order: fft_tw_pos of transforms whose exchanges are local from bit cb on
-__global__ void stage_table_kernel(int log_l, int maxrb, int cb, double2* t64, float2* t32) {
+// lf: (c, t) entries of the binary64 form's fused butterflies
+__global__ void stage_table_kernel(int log_l, int maxrb, int cb, bool lf, double2* t64, float2* t32) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     const int l = 1 << log_l;
     if (m >= l) return;
@@ -303,6 +304,15 @@ __global__ void stage_table_kernel(int log_l, int maxrb, int cb, double2* t64, f
         const int r_ = 1 << fftr_radix_bits(log_l, done, maxrb);
         if (ns > 1 && m >= ns - 1 && m < ns * r_ - 1) {
             const int off = m - (ns - 1);
+            if (lf) {
+                const int e = off / ns;
+                if (e >= r_ / 2) continue;
+                double sn, cs;
+                sincospi(2.0 * (double)fft_lf_entry(e, off % ns, ns, r_) / (double)(ns * r_), &sn, &cs);
+                if (cs == 0.0) cs = 8.673617379884035e-19;   // 2^-60
+                val = make_double2(cs, sn / cs);
+                continue;
+            }
             const int r = off / ns + 1;
             // the inverse of fft_tw_pos on 0..ns-1
             const int pos = off % ns;
@@ -332,9 +342,9 @@ unsigned int take_index_checks(cudaStream_t s) {
 #endif
 }
 
-cudaError_t launch_stage_tables(int log_l, int maxrb, int k, double2* t64, float2* t32, cudaStream_t s) {
+cudaError_t launch_stage_tables(int log_l, int maxrb, int k, bool lf, double2* t64, float2* t32, cudaStream_t s) {
     const int l = 1 << log_l;
-    stage_table_kernel<<<(l + 255) / 256, 256, 0, s>>>(log_l, maxrb, fft_local_bits(log_l, maxrb, k), t64, t32);
+    stage_table_kernel<<<(l + 255) / 256, 256, 0, s>>>(log_l, maxrb, fft_local_bits(log_l, maxrb, k), lf, t64, t32);
     return cudaGetLastError();
 }
 

@@ -138,7 +138,8 @@ unsigned int take_index_checks_ff(cudaStream_t s);   // the float-float passes' 
 // compiled pass-A column-block widths (radix-16 stages) for a length: writes up to 5 values, returns the count
 int pass_a_k1b_variants(int log_n2, int precision, int* out);
 // per-stage twiddles of length-2^log_l transforms, in the order of threads shared by k columns (0: jm's own)
-cudaError_t launch_stage_tables(int log_l, int maxrb, int k, double2* t64, float2* t32, cudaStream_t s);
+// lf: the binary64 form's fused-butterfly entries (lf_dft) in t64
+cudaError_t launch_stage_tables(int log_l, int maxrb, int k, bool lf, double2* t64, float2* t32, cudaStream_t s);
 // pass A with radix-8 stages (8 values per thread) is compiled for these shapes
 bool pass_a_radix8_available(int log_n2, int precision, int k1b);
 // pass-A stage radix bits a context starts with (and fcas_set_shape's radix_bits_a = 0)
