@@ -101,6 +101,7 @@ void free_ctx(fcas_ctx* c) {
                     c->d_tw32, c->d_twlo32, c->d_twhi32, c->d_stw_a64, c->d_stw_a32, c->d_stw_b64, c->d_stw_b32,
                     c->d_twloff, c->d_twhiff, c->d_stw_aff, c->d_stw_bff, c->d_phtab,
                     c->d_params, c->d_theta, c->d_fit, c->d_tc, c->d_inter, c->d_partials, c->d_pso,
+                    c->d_search_inter, c->d_search_partials,
                     c->d_gsums, c->d_gstage, c->d_ynat, c->d_polish};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -277,8 +278,30 @@ int64_t auto_chunk(size_t per_particle, size_t scratch) {
     return std::max<int64_t>(1, std::min(want, most));
 }
 
-// A larger intermediate and argmax array for chunks of `want` particles; the present ones stay when the device
-// has no room for more.
+// The search's own intermediate and argmax array, for chunks of up to `want` particles. They are apart from the
+// context's, whose addresses a caller may hold in a captured graph of fcas_fitness and which therefore are never
+// replaced here; nothing outlives a search that points at these. When the device has no room for them the search
+// uses the context's.
+void grow_search_scratch(fcas_ctx* c, int64_t want, size_t inter_pp) {
+    if (want <= c->search_chunk) return;
+    if (c->d_search_inter) cudaFree(c->d_search_inter);
+    if (c->d_search_partials) cudaFree(c->d_search_partials);
+    c->d_search_inter = nullptr;
+    c->d_search_partials = nullptr;
+    c->search_chunk = 0;
+    if (cudaMalloc(&c->d_search_inter, inter_pp * (size_t)want) == cudaSuccess &&
+        cudaMalloc(reinterpret_cast<void**>(&c->d_search_partials), sizeof(Partial) * (size_t)want * c->nb_cap) ==
+            cudaSuccess) {
+        c->search_chunk = want;
+        return;
+    }
+    cudaGetLastError();
+    if (c->d_search_inter) cudaFree(c->d_search_inter);
+    c->d_search_inter = nullptr;
+    c->d_search_partials = nullptr;
+}
+
+// The group's scratch for chunks of `want` particles; the present one stays when the device has no room for more.
 void grow_scratch(void** inter, Partial** partials, int64_t* chunk, int64_t want, size_t inter_pp, int64_t nb) {
     if (want <= *chunk) return;
     void* i = nullptr;
@@ -751,14 +774,22 @@ int fcas_search(fcas_ctx* c, const fcas_pso_config* cfg, fcas_search_result* res
     int rc = pso_validate(cfg, msg, sizeof(msg));
     if (rc) return fail(rc, "fcas_search: %s", msg);
     const int64_t rows = (int64_t)cfg->n_runs * cfg->n_particles;
-    rc = ensure_particles(c, rows);
-    if (!rc) rc = ensure_scratch(c);
-    if (rc) return rc;
+    // the search's arrays are its own: it never replaces one that a captured fcas_fitness points at
     if (c->setup.max_batch == 0 && cfg->n_iter >= kGrowIterations) {
         const size_t pp = inter_bytes_per_particle(c->setup.precision, c->setup.n_fft);
-        grow_scratch(&c->d_inter, &c->d_partials, &c->chunk, std::min(rows, auto_chunk(pp, kSearchScratch)), pp, c->nb_cap);
+        const int64_t want = std::min(rows, auto_chunk(pp, kSearchScratch));
+        if (want > c->chunk) grow_search_scratch(c, want, pp);
     }
-    const size_t need = swarm_bytes(rows, cfg->n_runs);
+    const bool own = c->search_chunk > c->chunk;
+    if (!own) {
+        rc = ensure_scratch(c);
+        if (rc) return rc;
+    }
+    void* inter = own ? c->d_search_inter : c->d_inter;
+    Partial* partials = own ? c->d_search_partials : c->d_partials;
+    const int64_t chunk = own ? c->search_chunk : c->chunk;
+    const size_t swarm = align256(swarm_bytes(rows, cfg->n_runs));
+    const size_t need = swarm + sizeof(ParticleParams) * (size_t)rows;
     if (need > c->pso_bytes) {
         if (c->d_pso) cudaFree(c->d_pso);
         c->d_pso = nullptr;
@@ -768,6 +799,7 @@ int fcas_search(fcas_ctx* c, const fcas_pso_config* cfg, fcas_search_result* res
         c->pso_bytes = need;
     }
     const Swarm w = carve_swarm(c->d_pso, rows, cfg->n_runs);
+    ParticleParams* params = reinterpret_cast<ParticleParams*>(c->d_pso + swarm);
     if (!c->search_stream) FCAS_CUDA(cudaStreamCreateWithFlags(&c->search_stream, cudaStreamNonBlocking));
     cudaStream_t st = c->search_stream;
     cudaEvent_t ev;
@@ -780,8 +812,7 @@ int fcas_search(fcas_ctx* c, const fcas_pso_config* cfg, fcas_search_result* res
     cudaError_t e = launch_pso_init(g, w.s, st);
     if (e == cudaSuccess)
         e = run_iterations(cfg->n_iter, st,
-                           [&]() { return swarm_iteration(c, g, w, c->d_params, c->d_inter, c->d_partials, c->chunk,
-                                                          rows, st); });
+                           [&]() { return swarm_iteration(c, g, w, params, inter, partials, chunk, rows, st); });
     if (e == cudaSuccess) e = launch_pso_result(g, w.s, w.res, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(results, w.res, sizeof(fcas_search_result) * cfg->n_runs, cudaMemcpyDeviceToHost, st);

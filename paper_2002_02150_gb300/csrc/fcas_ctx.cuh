@@ -80,8 +80,11 @@ struct fcas_ctx {
     size_t polish_bytes = 0;
     unsigned char* h_stage = nullptr;   // pinned host staging of small fcas_fitness calls (theta, fitness, tc)
     // particle swarm search
-    unsigned char* d_pso = nullptr;  // state, parameters, fitness, counters and results of the swarm
+    unsigned char* d_pso = nullptr;  // state, parameters, fitness, counters, results and particle records of the swarm
     size_t pso_bytes = 0;
+    void* d_search_inter = nullptr;  // the search's own d_inter and d_partials, for larger chunks than the context's
+    fcas::Partial* d_search_partials = nullptr;
+    int64_t search_chunk = 0;
     cudaStream_t search_stream = nullptr;
     // profiling
     bool prof = false;
