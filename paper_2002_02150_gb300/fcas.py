@@ -311,8 +311,9 @@ def fcas_fitness_noalloc(ctx, theta, fitness, tc, stream=None):
     import torch
     dev = torch.cuda.current_device()
     f64, i64 = torch.float64, torch.int64
-    ok = all(isinstance(a, torch.Tensor) and a.is_cuda and a.dtype is want and a.get_device() == dev and a.is_contiguous()
-             for a, want in ((theta, f64), (fitness, f64), (tc, i64)))
+    # _is_torch as in array_desc and _stream: what passes here is what the long check takes, and gets its stream
+    ok = all(_is_torch(a) and isinstance(a, torch.Tensor) and a.is_cuda and a.dtype is want and a.get_device() == dev
+             and a.is_contiguous() for a, want in ((theta, f64), (fitness, f64), (tc, i64)))
     if ok and theta.dim() == 2 and theta.shape[1] == 4:
         n = theta.shape[0]
         ok = fitness.numel() >= n and tc.numel() >= n
