@@ -230,11 +230,11 @@ cudaError_t launch_passes(fcas_ctx* c, int64_t n, double* d_fit, int64_t* d_tc, 
     return launch_passes_with(c, c->d_params, c->d_inter, c->d_partials, c->chunk, n, d_fit, d_tc, st);
 }
 
-// Buffers of the adjoint: partial band sums of one launch's particles and a staging array for host outputs.
+// Buffers of the adjoint: partial band sums of one launch's particles and a staging array for host outputs. Their
+// sizes depend on n alone, not on the launch shape: a change of shape and back leaves the addresses that a captured
+// fcas_gradient points at.
 int ensure_grad(fcas_ctx* c, int64_t n) {
-    const FitnessPlan plan = make_plan(c);
-    const size_t need = sizeof(double) * 12 * (size_t)c->setup.n_det * grad_segments(plan) *
-                        (size_t)std::min(n, grad_chunk(plan));
+    const size_t need = sizeof(double) * 12 * (size_t)c->setup.n_det * (size_t)grad_launch_segments(c->log_n, n);
     if (need > c->gsums_bytes) {
         if (c->d_gsums) cudaFree(c->d_gsums);
         c->d_gsums = nullptr;

@@ -398,12 +398,18 @@ grad_final_kernel(const double* __restrict__ theta, const int64_t* __restrict__ 
 
 // Segments of the band sums: ~2048 bins per CTA, at most 256 segments and one column block per segment
 // (a power of two, as the number of column blocks is).
-int grad_segments(const FitnessPlan& pl) {
-    const int nblk = (1 << pl.log_n1) / pl.k1b;
-    return imax_c(1, imin_c(imin_c(nblk, 256), pl.log_n > 12 ? 1 << (pl.log_n - 12) : 1));
+static int most_segments(int log_n) { return log_n > 12 ? imin_c(256, 1 << (log_n - 12)) : 1; }
+static int grad_segments(const FitnessPlan& pl) {
+    return imax_c(1, imin_c((1 << pl.log_n1) / pl.k1b, most_segments(pl.log_n)));
 }
 
-int64_t grad_chunk(const FitnessPlan& pl) { return imax_c(1, 32768 / grad_segments(pl)); }
+// (particle, segment) pairs of one launch, which bound the partial sums (12.6 MB with four detectors)
+constexpr int64_t kGradPairs = 32768;
+
+int64_t grad_launch_segments(int log_n, int64_t n) {
+    const int64_t m = most_segments(log_n);
+    return n < kGradPairs / m ? n * m : kGradPairs;
+}
 
 cudaError_t launch_gradient(const FitnessPlan& pl, int precision, int64_t k_lo, int64_t k_hi,
                             const ParticleParams* params, const double* theta, const int64_t* tc, int64_t n,
@@ -413,7 +419,7 @@ cudaError_t launch_gradient(const FitnessPlan& pl, int precision, int64_t k_lo, 
     const int blks = (1 << pl.log_n1) / pl.k1b / nseg;
     int log_k1b = 0;
     while ((1 << log_k1b) < pl.k1b) ++log_k1b;
-    const int64_t chunk = grad_chunk(pl);   // bounds the partial sums (12.6 MB with four detectors)
+    const int64_t chunk = kGradPairs / nseg;
     for (int64_t p0 = 0; p0 < n; p0 += chunk) {
         const int64_t np = n - p0 < chunk ? n - p0 : chunk;
         const unsigned ctas = (unsigned)(np * pairs * nseg);

@@ -147,9 +147,9 @@ int pass_a_default_radix_bits(int log_n2, int precision);
 
 // ---- adjoint (fcas_grad.cu) ----
 // d Gamma^2 / d theta at the lags tc of n particles whose parameters (geometry) are in params. part: scratch
-// of grad_chunk() particles, grad_segments() x n_det x 12 binary64 partial sums each.
-int grad_segments(const FitnessPlan& plan);
-int64_t grad_chunk(const FitnessPlan& plan);
+// of grad_launch_segments() x n_det x 12 binary64 partial sums.
+// grad_launch_segments: the most (particle, segment) pairs that a launch for n particles has in any launch shape
+int64_t grad_launch_segments(int log_n, int64_t n);
 cudaError_t launch_gradient(const FitnessPlan& plan, int precision, int64_t k_lo, int64_t k_hi,
                             const ParticleParams* params, const double* theta, const int64_t* tc, int64_t n,
                             double* part, const double* det9, const double* s2, double f_star, double df, double* grad,

@@ -39,3 +39,33 @@ def test_a_search_leaves_a_captured_fitness_valid(captured):
             np.testing.assert_array_equal(fit.cpu().numpy(), f)
             np.testing.assert_array_equal(tc.cpu().numpy(), t)
         assert fc.fcas_search(ctx, cfg) == first
+
+
+def test_a_change_of_shape_and_back_leaves_a_captured_gradient_valid():
+    # 2^18 points: sixteen columns per CTA split the band into fewer segments than the default width does
+    import dataclasses
+
+    import torch
+    import paper_2002_02150_gb300 as fc
+    w = dataclasses.replace(sd.C1, n_fft=1 << 18, n_samples=200001, f_low=40.0)
+    data = sd.make_dataset(w, 11)
+    sets = [torch.tensor(sd.make_particles(w, 6, seed=s, f_star=w.f_low), device="cuda:0") for s in (1, 2)]
+    with make_ctx(w, data, "fp32") as ctx:
+        fc.fcas_set_shape(ctx, 0, 16, 16, 4)
+        lags = [fc.fcas_fitness(ctx, th)[1] for th in sets]
+        expect = [fc.fcas_gradient(ctx, th, t).cpu().numpy() for th, t in zip(sets, lags)]
+        theta, tc, grad = sets[0].clone(), lags[0].clone(), torch.zeros_like(sets[0])
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            fc.fcas_gradient(ctx, theta, tc, grad=grad)
+        fc.fcas_set_shape(ctx, 0, 0, 16, 0)
+        fc.fcas_gradient(ctx, theta, tc)
+        torch.cuda.synchronize()
+        fc.fcas_set_shape(ctx, 0, 16, 16, 4)
+        for th, t, g in zip(sets, lags, expect):
+            theta.copy_(th)
+            tc.copy_(t)
+            graph.replay()
+            torch.cuda.synchronize()
+            np.testing.assert_array_equal(grad.cpu().numpy(), g)
