@@ -349,6 +349,8 @@ int apply_layout(fcas_ctx* c, int bias, int k1b, int sub, int radix_bits_a, cuda
     if (radix_bits_a != 4 && !(radix_bits_a == 3 && pass_a_radix8_available(l2, c->setup.precision, k1b)))
         return fail(FCAS_ERR_INVALID, "pass-A radix %d not compiled for this shape", 1 << radix_bits_a);
     const int64_t nb = pass_b_blocks_per_particle(l1, l2, c->setup.precision);
+    // (fewer rows than one CTA takes: the short split of 2^6 to 2^9 points)
+    if (nb < 1) return fail(FCAS_ERR_INVALID, "split bias %d leaves a pass-B CTA with too few rows", bias);
     if (c->nb_cap && nb > c->nb_cap) return fail(FCAS_ERR_INVALID, "split bias %d needs more argmax partials", bias);
     c->split_bias = bias;
     c->log_n2 = l2;
@@ -879,12 +881,14 @@ int fcas_autotune(fcas_ctx* c, int64_t n_particles, const char* cache_path, void
     const bool prof = c->prof;
     c->prof = false;
     double best_ms = 1e300;
-    int best_bias = c->split_bias, best_k = c->k1b, best_sub = c->sub, best_rb = c->radix_bits_a;
+    const int was_bias = c->split_bias, was_k = c->k1b, was_sub = c->sub, was_rb = c->radix_bits_a;
+    int best_bias = was_bias, best_k = was_k, best_sub = was_sub, best_rb = was_rb;
     int last_l2 = -1;
     const int subs[4] = {1, 4, 8, 16};
     for (int bias = 0; bias <= 1 && rc == FCAS_OK; ++bias) {
         const int l2 = split_log_n2_with(c->log_n, bias);
         if (l2 == last_l2 || c->log_n - l2 > kMaxLogPass) continue;
+        if (pass_b_blocks_per_particle(c->log_n - l2, l2, c->setup.precision) < 1) continue;   // (apply_layout)
         last_l2 = l2;
         int ks[8], rbs[8];
         int nk = pass_a_k1b_variants(l2, c->setup.precision, ks);   // at most 5, plus 2 radix-8 shapes below
@@ -924,9 +928,14 @@ int fcas_autotune(fcas_ctx* c, int64_t n_particles, const char* cache_path, void
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     c->prof = prof;
-    if (rc) return rc;
-    rc = apply_layout(c, best_bias, best_k, best_sub, best_rb, st);
-    if (rc) return rc;
+    if (!rc) rc = apply_layout(c, best_bias, best_k, best_sub, best_rb, st);
+    if (rc) {
+        // the shape the context had (its arrays hold another one's layout now); the first failure is reported
+        const std::string first = g_last_error;
+        if (apply_layout(c, was_bias, was_k, was_sub, was_rb, st) == FCAS_OK) cudaStreamSynchronize(st);
+        g_last_error = first;
+        return rc;
+    }
     c->tuned_ms = best_ms;
     FCAS_CUDA(cudaStreamSynchronize(st));
     if (cache_path) {
