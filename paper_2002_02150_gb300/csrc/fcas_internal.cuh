@@ -1,6 +1,8 @@
 // Internal declarations shared by the CUDA translation units of libfcas.
 #pragma once
 
+#include <cmath>
+
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -65,14 +67,14 @@ __device__ __forceinline__ float2 operator+(float2 a, float2 b) { return make_fl
 __device__ __forceinline__ float2 operator-(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ double2 operator+(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 operator-(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+__host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+__host__ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
-__device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-__device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
+__host__ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
+__host__ __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
 // multiply by S*i (S = +1 or -1)
@@ -102,9 +104,10 @@ struct ParticleParams {
     float2 dstep[FCAS_MAX_DET];    // e^{2 pi i S Delta^i df}, S = N / V_A: the FP32 pass A's step of the
                                    // delay phasor between a thread's consecutive bins (binary64 phase)
     // binary64 and float-float pass A: delays relative to detector 0's (whose own phase joins the chirp
-    // phase) and the phasor of the same step, e^{2 pi i S rturn}; filled for those forms only
+    // phase) and the phasors of the same step and of four, e^{2 pi i S rturn}; filled for those forms only
     double rturn[FCAS_MAX_DET];
     double2 rstep[FCAS_MAX_DET];
+    double2 rstep4[FCAS_MAX_DET];  // e^{2 pi i 4 S rturn}
     int32_t valid;                 // 0: non-finite / non-positive input -> fitness NaN, tc -1
     int32_t taylor_ok;             // FP32 pass A may step the chirp phase from an anchor bin to the
                                    // next 3 (bit 0) or 7 (bit 1) bins: remainder below 1e-7 turns

@@ -169,11 +169,15 @@ geometry_kernel(const double* __restrict__ theta, int64_t n, ParticleParams* __r
         const double rel = det_lane ? dturn - d0 : 0.0;
         double ur = (double)kstep * rel;
         ur -= rint(ur);
-        double sr, cr;
+        double ur4 = 4.0 * ur;   // (exact, as kstep rel is: powers of two)
+        ur4 -= rint(ur4);
+        double sr, cr, s4, c4;
         sincospi(2.0 * ur, &sr, &cr);
+        sincospi(2.0 * ur4, &s4, &c4);
         if (have) {
             pp->rturn[sub] = rel;
             pp->rstep[sub] = make_double2(cr, sr);
+            pp->rstep4[sub] = make_double2(c4, s4);
         }
     }
     if (!have) return;

@@ -19,6 +19,7 @@
 
 #include "fcas_fft16.cuh"
 #include "fcas_kernels.cuh"
+#include "fcas_phasor.cuh"
 
 namespace fcas {
 
@@ -129,61 +130,11 @@ __device__ __forceinline__ void st_stream(ff2* p, ff2 v) {
     __stcs(reinterpret_cast<float4*>(p), make_float4(v.x.h, v.x.l, v.y.h, v.y.l));
 }
 
-// a x + y and the next value of a three-term recurrence, c2 b - a per component
-__device__ __forceinline__ double axpy(double a, double x, double y) { return fma(a, x, y); }
-__device__ __forceinline__ ffloat axpy(ffloat a, ffloat x, ffloat y) { return ff_fma(a, x, y); }
-template <typename Real>
-__device__ __forceinline__ cplx<Real> three_term(Real c2, cplx<Real> b, cplx<Real> a) {
-    return mkc(axpy(c2, b.x, -a.x), axpy(c2, b.y, -a.y));
-}
-__device__ __forceinline__ double twice(double a) { return 2.0 * a; }
-__device__ __forceinline__ ffloat twice(ffloat a) { return ffloat(2.0f * a.h, 2.0f * a.l); }
-
-// N phasors e^{i (phi + q theta)}, q = 0..N-1, given to use(q, phasor): at_mid = e^{i (phi + (N/2 - 1) theta)}
-// and one product give the two middle ones, the others follow outwards by p(q +- 1) = 2 cos(theta) p(q) -
-// p(q -+ 1), half the arithmetic of a product each. The recurrence loses at most N/2 + 1 units of rounding
-// over its N/2 - 1 steps, as many as N - 1 products in a row.
-template <typename Real, int N, typename F>
-__device__ __forceinline__ void phasor_run(cplx<Real> at_mid, cplx<Real> step, F&& use) {
-    using C = cplx<Real>;
-    if constexpr (N >= 4) {
-        constexpr int M = N / 2;
-        const Real c2 = twice(step.x);
-        const C up = cmul(at_mid, step);
-        use(M - 1, at_mid);
-        use(M, up);
-        C a = at_mid, b = up;
-#pragma unroll
-        for (int q = M + 1; q < N; ++q) {
-            const C n = three_term<Real>(c2, b, a);
-            use(q, n);
-            a = b;
-            b = n;
-        }
-        a = up;
-        b = at_mid;
-#pragma unroll
-        for (int q = M - 2; q >= 0; --q) {
-            const C n = three_term<Real>(c2, b, a);
-            use(q, n);
-            a = b;
-            b = n;
-        }
-    } else {
-        C w = at_mid;   // N / 2 - 1 = 0, or N = 1
-#pragma unroll
-        for (int q = 0; q < N; ++q) {
-            use(q, w);
-            if (q + 1 < N) w = cmul(w, step);
-        }
-    }
-}
-__host__ __device__ constexpr int phasor_mid(int n) { return n >= 4 ? n / 2 - 1 : 0; }
-
 template <typename Real>
 struct DetConst {
     double rturn[FCAS_MAX_DET];          // delay relative to detector 0's [turns per bin]
-    cplx<Real> step[FCAS_MAX_DET];       // its phasor over a thread's bin step
+    cplx<Real> step[FCAS_MAX_DET];       // its phasor over a thread's bin step, and over four
+    cplx<Real> step4[FCAS_MAX_DET];
     Real w1[FCAS_MAX_DET], w2[FCAS_MAX_DET];
 };
 
@@ -232,9 +183,10 @@ pass_a_kernel(const cplx<Real>* __restrict__ y, const BasisD* __restrict__ basis
     // (CTAs of fewer than 8 threads fill the constants in turns)
     for (int i = threadIdx.x; i < FCAS_MAX_DET; i += blockDim.x) {
         const double d = pp->rturn[i];
-        const double2 st = pp->rstep[i];
+        const double2 st = pp->rstep[i], st4 = pp->rstep4[i];
         sc.rturn[i] = d;
         sc.step[i] = mkc(Real(st.x), Real(st.y));
+        sc.step4[i] = mkc(Real(st4.x), Real(st4.y));
         sc.w1[i] = Real(pp->w1[i]);
         sc.w2[i] = Real(pp->w2[i]);
         if constexpr (kFF) {
@@ -296,14 +248,14 @@ pass_a_kernel(const cplx<Real>* __restrict__ y, const BasisD* __restrict__ basis
 #pragma unroll kDetUnroll
     for (int i = 1; i < FCAS_MAX_DET; ++i) {
         if (i >= n_det) break;
-        const int kmid = kbase + phasor_mid(VH) * kstep;
+        const int kmid = kbase + phasor_anchor(VH) * kstep;
         C dph;
         if constexpr (kFF)
             dph = ff_unit_phasor(ff_frac_mul_int(kmid, dsplit[0][i], dsplit[1][i], dsplit[2][i]), ptab);
         else
             dph = unit_phasor((double)kmid * sc.rturn[i], ptab);
         const Real w1 = sc.w1[i], w2 = sc.w2[i];
-        phasor_run<Real, VH>(dph, sc.step[i], [&](int q, C ph) {
+        phasor_run<Real, VH>(dph, sc.step[i], sc.step4[i], [&](int q, C ph) {
             const C t = cmul(spectrum(i, q), ph);
             r1[q] = mkc(axpy(w1, t.x, r1[q].x), axpy(w1, t.y, r1[q].y));
             r2[q] = mkc(axpy(w2, t.x, r2[q].x), axpy(w2, t.y, r2[q].y));
@@ -329,10 +281,13 @@ pass_a_kernel(const cplx<Real>* __restrict__ y, const BasisD* __restrict__ basis
         fftr<Real, +1, LOG_L, MAXRB, 0, 0, true, false, pass_a_pad_shift<Real, MAXRB>(), false>(v, smem + c, K1B, j, stw);
         C* orow = out + ((p * kSeries + a) * L) * (int64_t)n1 + k1;
         // e^{2 pi i k1 ta / N} for ta = j + q G, steps of e^{2 pi i k1 G / N}
-        const int m0 = k1 * (j + phasor_mid(V) * G), ms = k1 * G;   // < N
-        const C w0 = cmul(ldg_c(tw_hi + (m0 >> kTwLoBits)), ldg_c(tw_lo + (m0 & ((1 << kTwLoBits) - 1))));
-        const C step = cmul(ldg_c(tw_hi + (ms >> kTwLoBits)), ldg_c(tw_lo + (ms & ((1 << kTwLoBits) - 1))));
-        phasor_run<Real, V>(w0, step, [&](int q, C w) {
+        const int m0 = k1 * (j + phasor_anchor(V) * G), ms = k1 * G;   // < N
+        auto twiddle = [&](int m) {
+            return cmul(ldg_c(tw_hi + (m >> kTwLoBits)), ldg_c(tw_lo + (m & ((1 << kTwLoBits) - 1))));
+        };
+        const C step = twiddle(ms);
+        const C step4 = V >= 8 ? twiddle((4 * ms) & ((n1 << LOG_L) - 1)) : step;   // (4 ms < 2^26)
+        phasor_run<Real, V>(twiddle(m0), step, step4, [&](int q, C w) {
             const int ta = j + q * G;
             if (FCAS_CHECK((p * kSeries + a) * (int64_t)L * n1 + k1 + (int64_t)ta * n1 < np * kSeries * (int64_t)L * n1,
                            kCheckInterWrite))
