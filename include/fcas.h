@@ -258,8 +258,10 @@ int fcas_search(fcas_ctx* ctx, const fcas_pso_config* cfg, fcas_search_result* r
  *   grad  : [n][4] (d/d alpha, d/d delta, d/d tau0, d/d tau1.5) of Gamma^2 [per rad, per s]
  *           (host or device).
  * The six band sums each detector needs at t_c (Z, sum k Q, and the four chirp-basis moments)
- * are reduced in binary64; the per-particle combination (antenna patterns, delays, G^-1 and
- * the chirp coefficients, differentiated analytically) is binary64. Particles with invalid input,
+ * are reduced in binary64 in the binary64 and float-float forms, and in the FP32 form, whose terms
+ * are FP32 numbers, as pairs of floats within CTAs (some 48 bits) and in binary64 across them; the
+ * per-particle combination (antenna patterns, delays, G^-1 and the chirp coefficients,
+ * differentiated analytically) is binary64. Particles with invalid input,
  * tc < 0, or an ill-conditioned G (the rank-1 rule of fcas_fitness) get NaN.
  */
 int fcas_gradient(fcas_ctx* ctx, int64_t n, const double* theta, const int64_t* tc, double* grad, void* stream);

@@ -12,62 +12,13 @@
 // the sums in binary64.
 #include <cmath>
 
-#include "fcas_ff.cuh"
 #include "fcas_kernels.cuh"
+#include "fcas_sums.cuh"
 
 namespace fcas {
 
 constexpr int kGradSums = 12;   // Z, F (= sum k Q), S_53, S_1, S_23, S_13: complex, as (re, im) doubles
 
-// One running sum of the adjoint. The FP32 form's terms are FP32 values times float-float weights; their
-// sum is kept as a compensated pair on the FP32 units (Ogita, Rump & Oishi 2005: the rounding error of
-// every product and every addition is formed exactly and added to the second word), as accurate as the
-// binary64 sum of the same terms for the at most 2^10 terms a thread adds, at ~11 FP32 instructions per
-// term where a binary64 one holds the SM's binary64 unit for as long as 64 FP32 instructions would take.
-struct SumF {
-    float h, l;
-};
-__device__ __forceinline__ void sum_zero(SumF& a) { a.h = a.l = 0.0f; }
-__device__ __forceinline__ void sum_zero(double& a) { a = 0.0; }
-__device__ __forceinline__ void sum_add(SumF& a, float q) {
-    float e;
-    a.h = ff_two_sum(a.h, q, e);
-    a.l = __fadd_rn(a.l, e);
-}
-// a += w q for an exact float w
-__device__ __forceinline__ void sum_add_w(SumF& a, float w, float q) {
-    const float p = __fmul_rn(w, q);
-    float e;
-    a.h = ff_two_sum(a.h, p, e);
-    a.l = __fadd_rn(a.l, __fadd_rn(e, __fmaf_rn(w, q, -p)));
-}
-// a += (w.x + w.y) q
-__device__ __forceinline__ void sum_add_w(SumF& a, float2 w, float q) {
-    const float p = __fmul_rn(w.x, q);
-    float e;
-    a.h = ff_two_sum(a.h, p, e);
-    a.l = __fadd_rn(a.l, __fadd_rn(e, __fmaf_rn(w.y, q, __fmaf_rn(w.x, q, -p))));
-}
-__device__ __forceinline__ void sum_add(double& a, double q) { a += q; }
-__device__ __forceinline__ void sum_add_w(double& a, double w, double q) { a += w * q; }
-__device__ __forceinline__ SumF sum_of(SumF a, SumF b) {
-    const ffloat r = ff_add(ffloat(a.h, a.l), ffloat(b.h, b.l));
-    return SumF{r.h, r.l};
-}
-__device__ __forceinline__ double sum_of(double a, double b) { return a + b; }
-// the pair as a float-float number (the second word may have outgrown half an ulp of the first)
-__device__ __forceinline__ void sum_normalise(SumF& a) {
-    float e;
-    a.h = ff_two_sum(a.h, a.l, e);
-    a.l = e;
-}
-__device__ __forceinline__ void sum_normalise(double&) {}
-__device__ __forceinline__ SumF sum_xor(SumF a, int off) {
-    return SumF{__shfl_xor_sync(0xffffffffu, a.h, off), __shfl_xor_sync(0xffffffffu, a.l, off)};
-}
-__device__ __forceinline__ double sum_xor(double a, int off) { return __shfl_xor_sync(0xffffffffu, a, off); }
-__device__ __forceinline__ double sum_value(SumF a) { return (double)a.h + (double)a.l; }
-__device__ __forceinline__ double sum_value(double a) { return a; }
 template <typename Real> struct grad_sum { using type = double; };
 template <> struct grad_sum<float> { using type = SumF; };
 
