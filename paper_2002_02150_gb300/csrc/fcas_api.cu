@@ -301,24 +301,6 @@ void grow_search_scratch(fcas_ctx* c, int64_t want, size_t inter_pp) {
     c->d_search_partials = nullptr;
 }
 
-// The group's scratch for chunks of `want` particles; the present one stays when the device has no room for more.
-void grow_scratch(void** inter, Partial** partials, int64_t* chunk, int64_t want, size_t inter_pp, int64_t nb) {
-    if (want <= *chunk) return;
-    void* i = nullptr;
-    Partial* p = nullptr;
-    if (cudaMalloc(&i, inter_pp * (size_t)want) == cudaSuccess &&
-        cudaMalloc(reinterpret_cast<void**>(&p), sizeof(Partial) * (size_t)want * nb) == cudaSuccess) {
-        if (*inter) cudaFree(*inter);
-        if (*partials) cudaFree(*partials);
-        *inter = i;
-        *partials = p;
-        *chunk = want;
-        return;
-    }
-    cudaGetLastError();
-    if (i) cudaFree(i);
-}
-
 // Scratch of the fitness path (allocated at create unless FCAS_SETUP_LAZY_SCRATCH, else on first use).
 int ensure_scratch(fcas_ctx* c) {
     if (c->d_inter) return FCAS_OK;
@@ -967,9 +949,6 @@ int fcas_set_shape(fcas_ctx* c, int32_t split_bias, int32_t k1b, int32_t sub, in
 struct fcas_group {
     std::vector<fcas_ctx*> ctxs;
     int64_t chunk = 0;
-    int64_t auto_cap = 0;           // largest chunk a search may grow the scratch to (0: the caller fixed it)
-    size_t inter_pp = 0;            // scratch per particle: intermediate bytes and argmax partials
-    int64_t nb = 0;
     void* d_inter = nullptr;
     Partial* d_partials = nullptr;
     ParticleParams* d_params = nullptr;
@@ -999,9 +978,6 @@ int fcas_group_create(fcas_group** out, int32_t n_ctx, fcas_ctx* const* ctxs, in
     g->ctxs.assign(ctxs, ctxs + n_ctx);
     const int64_t chunk = max_batch > 0 ? max_batch : std::min<int64_t>(64, auto_chunk(inter_pp, kCreateScratch));
     g->chunk = chunk;
-    g->auto_cap = max_batch > 0 ? 0 : auto_chunk(inter_pp, kSearchScratch);
-    g->inter_pp = inter_pp;
-    g->nb = nb;
     int rc = dev_alloc(&g->d_inter, inter_pp * (size_t)chunk, "group intermediate transform");
     if (!rc) rc = dev_alloc(&g->d_partials, sizeof(Partial) * (size_t)chunk * nb, "group argmax partials");
     if (!rc) {
@@ -1049,8 +1025,6 @@ int fcas_group_search_boxes(fcas_group* g, const fcas_pso_config* cfg, const dou
         if (rc) return rc;
         g->params_cap = rows;
     }
-    if ((int64_t)cfg->n_iter * n_ctx >= kGrowIterations)
-        grow_scratch(&g->d_inter, &g->d_partials, &g->chunk, std::min(rows, g->auto_cap), g->inter_pp, g->nb);
     const size_t per = align256(swarm_bytes(rows, cfg->n_runs));
     if (per * n_ctx > g->pso_bytes) {
         if (g->d_pso) cudaFree(g->d_pso);
