@@ -23,6 +23,10 @@
  *    allocates. A context must not be used from two threads at once.
  *  - A context belongs to the CUDA device that was current when it was created: every call that
  *    takes it must be made with that device current (FCAS_ERR_INVALID otherwise).
+ *  - Calls that are asynchronous on their stream may be captured in a CUDA graph once the same call has
+ *    run on the context with at least as large a batch (it allocated then). Replays stay valid until
+ *    the context is destroyed, tuned or reshaped (fcas_autotune, fcas_set_shape), or given a larger
+ *    batch than any before (fcas_fitness, fcas_gradient, fcas_polish); a search does not affect them.
  *  - All floating-point inputs are IEEE binary64.
  */
 #ifndef FCAS_H
@@ -74,7 +78,10 @@ typedef struct fcas_setup {
     double fs;           /* sampling rate [Hz] */
     double f_low;        /* lower cutoff f_* [Hz] (> 0): the template is zero for f <= f_low (Sec. II.B) */
     double f_high;       /* upper cutoff [Hz]: the template is zero for f > f_high (Sec. II.B) */
-    int32_t max_batch;   /* particles per internal chunk (0 = automatic); bounds scratch memory */
+    int32_t max_batch;   /* particles per internal chunk; bounds scratch memory. 0 = automatic: 64, or what
+                          * 16 GB hold of them; a larger batch makes the context allocate larger chunks
+                          * besides while they fit in 128 MB, and repeated or long searches (fcas_search)
+                          * chunks of their own within 512 MB; all released with the context */
     int32_t flags;       /* 0 or FCAS_SETUP_LAZY_SCRATCH */
 } fcas_setup;
 
@@ -370,7 +377,7 @@ typedef struct fcas_info {
     int64_t n_fft, n1, n2;      /* N = n1 * n2: pass A transforms length n2, pass B length n1 */
     int64_t k_lo, k_hi;         /* first and last template bin */
     int64_t n_band;             /* k_hi - k_lo + 1 */
-    int64_t chunk;              /* particles per internal chunk */
+    int64_t chunk;              /* particles per internal chunk (the largest batch's so far) */
     int32_t n_det, precision;
     double scale;               /* power of two applied to the whitened data (Gamma^2 is invariant) */
     double sigma2[FCAS_MAX_DET];/* unscaled template norms <h_c|h_c>^i */

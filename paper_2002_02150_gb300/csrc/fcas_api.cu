@@ -100,8 +100,8 @@ void free_ctx(fcas_ctx* c) {
     void* ptrs[] = {c->d_det, c->d_sigma2s, c->d_y, c->d_basis, c->d_tw64, c->d_twlo64, c->d_twhi64,
                     c->d_tw32, c->d_twlo32, c->d_twhi32, c->d_stw_a64, c->d_stw_a32, c->d_stw_b64, c->d_stw_b32,
                     c->d_twloff, c->d_twhiff, c->d_stw_aff, c->d_stw_bff, c->d_phtab,
-                    c->d_params, c->d_theta, c->d_fit, c->d_tc, c->d_inter, c->d_partials, c->d_pso,
-                    c->d_search_inter, c->d_search_partials,
+                    c->d_params, c->d_theta, c->d_fit, c->d_tc, c->scratch.inter, c->batch_scratch.inter,
+                    c->search_scratch.inter, c->d_pso,
                     c->d_gsums, c->d_gstage, c->d_ynat, c->d_polish};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -199,10 +199,16 @@ void prof_end(fcas_ctx* c, size_t slot, cudaStream_t s) {
     if (slot != SIZE_MAX) cudaEventRecord(c->events[slot].b, s);
 }
 
+// The scratch of the context's own calls.
+const Scratch& fitness_scratch(const fcas_ctx* c) { return c->batch_scratch.inter ? c->batch_scratch : c->scratch; }
+
 // Passes A, B and the final argmax over chunks of particle parameters, with the given scratch: as many
 // equal chunks as needed (77 particles by 64: 39 + 38 instead of 64 + 13, whose last waves are emptier).
-cudaError_t launch_passes_with(fcas_ctx* c, const ParticleParams* params, void* inter, Partial* partials,
-                               int64_t chunk, int64_t n, double* d_fit, int64_t* d_tc, cudaStream_t st) {
+cudaError_t launch_passes_with(fcas_ctx* c, const ParticleParams* params, const Scratch& scratch, int64_t n,
+                               double* d_fit, int64_t* d_tc, cudaStream_t st) {
+    void* inter = scratch.inter;
+    Partial* partials = scratch.partials;
+    int64_t chunk = scratch.chunk;
     const FitnessPlan plan = make_plan(c);
     const int prec = c->setup.precision;
     size_t slot;
@@ -227,7 +233,7 @@ cudaError_t launch_passes_with(fcas_ctx* c, const ParticleParams* params, void* 
 }
 
 cudaError_t launch_passes(fcas_ctx* c, int64_t n, double* d_fit, int64_t* d_tc, cudaStream_t st) {
-    return launch_passes_with(c, c->d_params, c->d_inter, c->d_partials, c->chunk, n, d_fit, d_tc, st);
+    return launch_passes_with(c, c->d_params, fitness_scratch(c), n, d_fit, d_tc, st);
 }
 
 // Buffers of the adjoint: partial band sums of one launch's particles and a staging array for host outputs. Their
@@ -265,48 +271,93 @@ cudaError_t gradient_device(fcas_ctx* c, int64_t n, const double* d_theta, const
                            c->d_gsums, c->d_det, c->d_sigma2s, c->setup.f_low, c->df, d_grad, st);
 }
 
-// Particles per chunk when the caller leaves it open: at least 64, and for short segments as many as the given
-// scratch holds (a chunk's launches have fixed costs and a last wave: 320 particles on 64 s take 239 us in
-// chunks of 64, 221 in three and 195 in one, on 4096 points 95 and 38 us; from 2^19 points on 64 is enough).
-// Bounded by 16 GB, and by 2048 (the passes' grids have one row of CTAs per particle).
-constexpr size_t kCreateScratch = (size_t)128 << 20;   // allocated with a context: no slower than 64 MB
-constexpr size_t kSearchScratch = (size_t)512 << 20;   // what a search of kGrowIterations or more grows it to
-constexpr int kGrowIterations = 12;                    // the growth takes ~250 us, an iteration saves ~25
-int64_t auto_chunk(size_t per_particle, size_t scratch) {
-    const int64_t most = (int64_t)(((size_t)16 << 30) / per_particle);
-    const int64_t want = std::min<int64_t>(2048, std::max<int64_t>(64, (int64_t)(scratch / per_particle)));
-    return std::max<int64_t>(1, std::min(want, most));
+// Particles per chunk when the caller leaves it open (setup.max_batch = 0): 64, less where 16 GB hold fewer. For
+// short segments larger chunks are faster, since a chunk's launches have fixed costs and a last wave (us per
+// fitness call of 320 particles in chunks of 64 / 128 / 320: 2^12 points 67 / 51 / 30, 2^14 94 / 79 / 58, 2^16 207 /
+// 197 / 195, 2^17 400 / 401 / 364): they are allocated for the batches that ask for them, within kBatchScratch for
+// evaluations (more than 64 particles up to 2^16 points) and kSearchScratch for searches (up to 2^18). 2048 at most
+// (the passes' grids have one row of CTAs per particle).
+constexpr size_t kBatchScratch = (size_t)128 << 20;
+constexpr size_t kSearchScratch = (size_t)512 << 20;
+size_t inter_pp(const fcas_ctx* c) { return inter_bytes_per_particle(c->setup.precision, c->setup.n_fft); }
+int64_t base_chunk(size_t per_particle) {
+    return std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)(((size_t)16 << 30) / per_particle)));
+}
+int64_t larger_chunk(const fcas_ctx* c, int64_t n, size_t scratch) {
+    return std::min<int64_t>(std::min<int64_t>(n, 2048), (int64_t)(scratch / inter_pp(c)));
 }
 
-// The search's own intermediate and argmax array, for chunks of up to `want` particles. They are apart from the
-// context's, whose addresses a caller may hold in a captured graph of fcas_fitness and which therefore are never
-// replaced here; nothing outlives a search that points at these. When the device has no room for them the search
-// uses the context's.
-void grow_search_scratch(fcas_ctx* c, int64_t want, size_t inter_pp) {
-    if (want <= c->search_chunk) return;
-    if (c->d_search_inter) cudaFree(c->d_search_inter);
-    if (c->d_search_partials) cudaFree(c->d_search_partials);
-    c->d_search_inter = nullptr;
-    c->d_search_partials = nullptr;
-    c->search_chunk = 0;
-    if (cudaMalloc(&c->d_search_inter, inter_pp * (size_t)want) == cudaSuccess &&
-        cudaMalloc(reinterpret_cast<void**>(&c->d_search_partials), sizeof(Partial) * (size_t)want * c->nb_cap) ==
-            cudaSuccess) {
-        c->search_chunk = want;
-        return;
+// Scratch for chunks of `chunk` particles in place of what *s holds; on failure *s holds nothing.
+cudaError_t alloc_scratch(const fcas_ctx* c, int64_t chunk, Scratch* s) {
+    if (s->inter) cudaFree(s->inter);
+    *s = Scratch();
+    const size_t inter = inter_pp(c) * (size_t)chunk;   // (a multiple of 256: the partials are aligned)
+    void* p = nullptr;
+    const cudaError_t e = cudaMalloc(&p, inter + sizeof(Partial) * (size_t)chunk * c->nb_cap);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
     }
-    cudaGetLastError();
-    if (c->d_search_inter) cudaFree(c->d_search_inter);
-    c->d_search_inter = nullptr;
-    c->d_search_partials = nullptr;
+    s->inter = p;
+    s->partials = reinterpret_cast<Partial*>(static_cast<unsigned char*>(p) + inter);
+    s->chunk = chunk;
+    return cudaSuccess;
 }
 
 // Scratch of the fitness path (allocated at create unless FCAS_SETUP_LAZY_SCRATCH, else on first use).
 int ensure_scratch(fcas_ctx* c) {
-    if (c->d_inter) return FCAS_OK;
-    const size_t per_particle = inter_bytes_per_particle(c->setup.precision, c->setup.n_fft);
-    int rc = dev_alloc(&c->d_inter, per_particle * (size_t)c->chunk, "intermediate transform");
-    if (!rc) rc = dev_alloc(&c->d_partials, sizeof(Partial) * (size_t)c->chunk * c->nb_cap, "argmax partials");
+    if (fitness_scratch(c).inter) return FCAS_OK;
+    const cudaError_t e = alloc_scratch(c, c->chunk, &c->scratch);
+    if (e == cudaSuccess) return FCAS_OK;
+    return fail(FCAS_ERR_NOMEM, "cudaMalloc for the intermediate transform of %lld particles failed: %s",
+                (long long)c->chunk, cudaGetErrorString(e));
+}
+
+// Everything an evaluation of n particles needs. Its arrays are replaced only in a call that replaces the particle
+// records too, one with a larger batch than any before: until then a captured call of the context stays valid.
+// Larger chunks are tried for once per larger batch, and not while the stream is being captured.
+int ensure_batch(fcas_ctx* c, int64_t n, cudaStream_t st) {
+    const bool larger = n > c->params_cap;
+    const int rc = ensure_particles(c, n);
+    if (rc) return rc;
+    if (c->setup.max_batch == 0 && n > std::max(c->chunk, c->batch_seen)) {
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        const bool idle = cudaStreamIsCapturing(st, &capturing) == cudaSuccess &&
+                          capturing == cudaStreamCaptureStatusNone;
+        const int64_t want = larger_chunk(c, n, kBatchScratch);
+        if (idle && (larger || !c->batch_scratch.inter)) {
+            c->batch_seen = n;
+            if (want > std::max(c->chunk, c->batch_scratch.chunk)) alloc_scratch(c, want, &c->batch_scratch);
+        }
+        cudaGetLastError();
+    }
+    return ensure_scratch(c);
+}
+
+// Scratch of a search of n_iter iterations of `rows` particles: larger chunks than the context's once its searches
+// have lost more by smaller ones (kChunkUs per chunk and iteration: 64 against all of 320 or 640 rows 6 to 13 us a
+// chunk at 2^12 to 2^18 points) than they cost to allocate and to release (200 us, and 0.6 us per MB of them).
+// They are the searches' own: a search replaces no array that a captured call of the context points at, and
+// nothing outlives a search that points at these. Without room for them it uses the context's.
+int ensure_search(fcas_ctx* c, int64_t rows, int n_iter, Scratch* use) {
+    constexpr double kChunkUs = 7.0, kAllocUs = 200.0, kAllocUsPerByte = 0.6 / (1 << 20);
+    const int64_t want = c->setup.max_batch == 0 ? larger_chunk(c, rows, kSearchScratch) : 0;
+    const int64_t have = std::max(std::max(c->chunk, fitness_scratch(c).chunk), c->search_scratch.chunk);
+    if (want > have) {
+        const int64_t fewer = (rows + have - 1) / have - (rows + want - 1) / want;
+        c->search_lost_us += kChunkUs * (double)fewer * n_iter;
+        if (c->search_lost_us > kAllocUs + kAllocUsPerByte * (double)inter_pp(c) * (double)want) {
+            c->search_lost_us = 0.0;
+            alloc_scratch(c, want, &c->search_scratch);
+        }
+    }
+    int rc = FCAS_OK;
+    if (c->search_scratch.chunk <= std::max(c->chunk, fitness_scratch(c).chunk)) {
+        rc = ensure_scratch(c);
+        *use = fitness_scratch(c);
+    } else {
+        *use = c->search_scratch;
+    }
     return rc;
 }
 
@@ -589,9 +640,7 @@ int create_impl(fcas_ctx** out, const fcas_setup* setup, const fcas_detector* de
                           pass_a_default_radix_bits(split_log_n2_with(c->log_n, FCAS_SPLIT_BIAS), s.precision), st));
 
     // scratch for the fitness path (partials sized for every split the tuner may choose)
-    const size_t per_particle = inter_bytes_per_particle(s.precision, n);
-    const int64_t chunk = s.max_batch > 0 ? s.max_batch : auto_chunk(per_particle, kCreateScratch);
-    c->chunk = chunk;
+    c->chunk = s.max_batch > 0 ? s.max_batch : base_chunk(inter_pp(c));
     c->nb_cap = 0;
     for (int bias = 0; bias <= 1; ++bias) {
         const int l2 = split_log_n2_with(log_n, bias);
@@ -630,8 +679,7 @@ int fcas_fitness(fcas_ctx* c, int64_t n, const double* theta, double* fitness, i
                             (long long)p);
         }
     }
-    int rc = ensure_particles(c, n);
-    if (!rc) rc = ensure_scratch(c);
+    int rc = ensure_batch(c, n, st);
     if (rc) return rc;
     const bool host = !th_dev || !f_dev || !t_dev;
     unsigned char* hs = host && n <= kHostStage ? host_stage(c) : nullptr;
@@ -711,12 +759,12 @@ Swarm carve_swarm(unsigned char* b, int64_t rows, int runs) {
 }
 
 // One PSO iteration of one segment: parameters of the particles inside the box, their fitness, update.
-cudaError_t swarm_iteration(fcas_ctx* c, const PsoDev& g, const Swarm& w, ParticleParams* params, void* inter,
-                            Partial* partials, int64_t chunk, int64_t rows, cudaStream_t st) {
+cudaError_t swarm_iteration(fcas_ctx* c, const PsoDev& g, const Swarm& w, ParticleParams* params,
+                            const Scratch& scratch, int64_t rows, cudaStream_t st) {
     // (w.theta holds the positions' parameters: written by the initialisation and by every update)
     cudaError_t x = launch_geometry(w.theta, rows, params, c->d_det, c->d_sigma2s, c->setup.n_det, c->setup.f_low, c->df,
                             pass_a_kstep(c), c->setup.precision, st);
-    if (x == cudaSuccess) x = launch_passes_with(c, params, inter, partials, chunk, rows, w.fit, w.tcs, st);
+    if (x == cudaSuccess) x = launch_passes_with(c, params, scratch, rows, w.fit, w.tcs, st);
     if (x == cudaSuccess) x = launch_pso_update(g, 0, w.fit, w.tcs, w.s, st, chain_pays(rows, c->log_n));
     return x;
 }
@@ -758,20 +806,10 @@ int fcas_search(fcas_ctx* c, const fcas_pso_config* cfg, fcas_search_result* res
     int rc = pso_validate(cfg, msg, sizeof(msg));
     if (rc) return fail(rc, "fcas_search: %s", msg);
     const int64_t rows = (int64_t)cfg->n_runs * cfg->n_particles;
-    // the search's arrays are its own: it never replaces one that a captured fcas_fitness points at
-    if (c->setup.max_batch == 0 && cfg->n_iter >= kGrowIterations) {
-        const size_t pp = inter_bytes_per_particle(c->setup.precision, c->setup.n_fft);
-        const int64_t want = std::min(rows, auto_chunk(pp, kSearchScratch));
-        if (want > c->chunk) grow_search_scratch(c, want, pp);
-    }
-    const bool own = c->search_chunk > c->chunk;
-    if (!own) {
-        rc = ensure_scratch(c);
-        if (rc) return rc;
-    }
-    void* inter = own ? c->d_search_inter : c->d_inter;
-    Partial* partials = own ? c->d_search_partials : c->d_partials;
-    const int64_t chunk = own ? c->search_chunk : c->chunk;
+    // the search's arrays are its own: it replaces none that a captured fcas_fitness points at
+    Scratch scratch;
+    rc = ensure_search(c, rows, cfg->n_iter, &scratch);
+    if (rc) return rc;
     const size_t swarm = align256(swarm_bytes(rows, cfg->n_runs));
     const size_t need = swarm + sizeof(ParticleParams) * (size_t)rows;
     if (need > c->pso_bytes) {
@@ -796,7 +834,7 @@ int fcas_search(fcas_ctx* c, const fcas_pso_config* cfg, fcas_search_result* res
     cudaError_t e = launch_pso_init(g, w.s, st);
     if (e == cudaSuccess)
         e = run_iterations(cfg->n_iter, st,
-                           [&]() { return swarm_iteration(c, g, w, params, inter, partials, chunk, rows, st); });
+                           [&]() { return swarm_iteration(c, g, w, params, scratch, rows, st); });
     if (e == cudaSuccess) e = launch_pso_result(g, w.s, w.res, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(results, w.res, sizeof(fcas_search_result) * cfg->n_runs, cudaMemcpyDeviceToHost, st);
@@ -843,8 +881,7 @@ int fcas_autotune(fcas_ctx* c, int64_t n_particles, const char* cache_path, void
             fclose(f);
         }
     }
-    int rc = ensure_particles(c, n_particles);
-    if (!rc) rc = ensure_scratch(c);
+    int rc = ensure_batch(c, n_particles, st);
     if (!rc) rc = ensure_staging(c, n_particles);
     if (rc) return rc;
     std::vector<double> th(4 * (size_t)n_particles);
@@ -976,7 +1013,7 @@ int fcas_group_create(fcas_group** out, int32_t n_ctx, fcas_ctx* const* ctxs, in
     }
     fcas_group* g = new fcas_group();
     g->ctxs.assign(ctxs, ctxs + n_ctx);
-    const int64_t chunk = max_batch > 0 ? max_batch : std::min<int64_t>(64, auto_chunk(inter_pp, kCreateScratch));
+    const int64_t chunk = max_batch > 0 ? max_batch : base_chunk(inter_pp);
     g->chunk = chunk;
     int rc = dev_alloc(&g->d_inter, inter_pp * (size_t)chunk, "group intermediate transform");
     if (!rc) rc = dev_alloc(&g->d_partials, sizeof(Partial) * (size_t)chunk * nb, "group argmax partials");
@@ -1051,8 +1088,8 @@ int fcas_group_search_boxes(fcas_group* g, const fcas_pso_config* cfg, const dou
         e = run_iterations(cfg->n_iter, st, [&]() {
             cudaError_t x = cudaSuccess;
             for (int i = 0; i < n_ctx && x == cudaSuccess; ++i)
-                x = swarm_iteration(g->ctxs[i], gs[i], ws[i], g->d_params, g->d_inter, g->d_partials, g->chunk, rows,
-                                    st);
+                x = swarm_iteration(g->ctxs[i], gs[i], ws[i], g->d_params,
+                                    Scratch{g->d_inter, g->d_partials, g->chunk}, rows, st);
             return x;
         });
     for (int i = 0; i < n_ctx && e == cudaSuccess; ++i) {
@@ -1162,8 +1199,7 @@ int fcas_polish(fcas_ctx* c, int64_t n, double* theta, double* fitness, int64_t*
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const bool th_dev = is_device_ptr(theta), f_dev = is_device_ptr(fitness), t_dev = is_device_ptr(tc);
     const bool a_dev = accepted && is_device_ptr(accepted);
-    int rc = ensure_particles(c, n);
-    if (!rc) rc = ensure_scratch(c);
+    int rc = ensure_batch(c, n, st);
     if (!rc) rc = ensure_grad(c, n);
     if (rc) return rc;
     // working arrays: theta, trial points, directions, gradients [n][4]; fitness, trial fitness and step
@@ -1274,7 +1310,7 @@ int fcas_get_info(const fcas_ctx* c, fcas_info* info) {
     info->k_lo = c->k_lo;
     info->k_hi = c->k_hi;
     info->n_band = c->k_hi - c->k_lo + 1;
-    info->chunk = c->chunk;
+    info->chunk = std::max(c->chunk, c->batch_scratch.chunk);
     info->n_det = c->setup.n_det;
     info->precision = c->setup.precision;
     info->scale = c->scale;

@@ -21,6 +21,13 @@ inline size_t inter_bytes_per_particle(int precision, int64_t n_fft) {
     return (precision == FCAS_PREC_FP32 ? sizeof(float2) : sizeof(double2)) * (size_t)kSeries * (size_t)n_fft;
 }
 
+// Scratch of the two passes for chunks of up to `chunk` particles, in one allocation.
+struct Scratch {
+    void* inter = nullptr;          // [chunk][2][N2][N1] complex
+    Partial* partials = nullptr;    // [chunk][blocks per particle], after it
+    int64_t chunk = 0;
+};
+
 }  // namespace fcas
 
 struct fcas_ctx {
@@ -67,9 +74,12 @@ struct fcas_ctx {
     double* d_fit = nullptr;        // staging for host outputs
     int64_t* d_tc = nullptr;
     int64_t stage_cap = 0;
-    void* d_inter = nullptr;        // [chunk][2][N2][N1] complex
-    fcas::Partial* d_partials = nullptr;  // [chunk][blocks per particle]
-    int64_t chunk = 0;
+    int64_t chunk = 0;              // particles per chunk of `scratch`
+    fcas::Scratch scratch;          // of every context once it evaluates; never replaced
+    fcas::Scratch batch_scratch;    // larger chunks for larger batches on short segments (ensure_batch)
+    int64_t batch_seen = 0;         // the largest batch that they were tried for
+    fcas::Scratch search_scratch;   // larger chunks for searches (ensure_search)
+    double search_lost_us = 0.0;    // what smaller chunks have cost the context's searches
     int64_t nb_partials = 0;
     // adjoint
     double* d_gsums = nullptr;       // [n][D][segments][12] partial per-detector sums at t*
@@ -82,9 +92,6 @@ struct fcas_ctx {
     // particle swarm search
     unsigned char* d_pso = nullptr;  // state, parameters, fitness, counters, results and particle records of the swarm
     size_t pso_bytes = 0;
-    void* d_search_inter = nullptr;  // the search's own d_inter and d_partials, for larger chunks than the context's
-    fcas::Partial* d_search_partials = nullptr;
-    int64_t search_chunk = 0;
     cudaStream_t search_stream = nullptr;
     // profiling
     bool prof = false;

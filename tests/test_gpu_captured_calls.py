@@ -69,3 +69,32 @@ def test_a_change_of_shape_and_back_leaves_a_captured_gradient_valid():
             graph.replay()
             torch.cuda.synchronize()
             np.testing.assert_array_equal(grad.cpu().numpy(), g)
+
+
+def test_larger_chunks_leave_a_captured_fitness_valid():
+    # the gradient call has made the particle records large enough: the larger evaluation replaces nothing
+    import torch
+    import paper_2002_02150_gb300 as fc
+    w = sd.SMALL
+    data = sd.make_dataset(w, 12)
+    many = torch.tensor(sd.make_particles(w, 320, seed=1), device="cuda:0")
+    sets = [many[:40].clone(), many[40:80].clone()]
+    with make_ctx(w, data, "fp32") as ctx:
+        fc.fcas_gradient(ctx, many, torch.zeros(320, dtype=torch.int64, device="cuda:0"))
+        expect = [[x.cpu().numpy() for x in fc.fcas_fitness(ctx, th)] for th in sets]
+        theta = sets[0].clone()
+        fit = torch.zeros(40, dtype=torch.float64, device="cuda:0")
+        tc = torch.zeros(40, dtype=torch.int64, device="cuda:0")
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            fc.fcas_fitness(ctx, theta, fitness=fit, tc=tc)
+        chunk = fc.fcas_get_info(ctx)["chunk"]
+        fc.fcas_fitness(ctx, many)
+        assert fc.fcas_get_info(ctx)["chunk"] > chunk
+        for th, (f, t) in zip(sets, expect):
+            theta.copy_(th)
+            graph.replay()
+            torch.cuda.synchronize()
+            np.testing.assert_array_equal(fit.cpu().numpy(), f)
+            np.testing.assert_array_equal(tc.cpu().numpy(), t)
