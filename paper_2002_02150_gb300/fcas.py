@@ -551,7 +551,8 @@ def fcas_autotune(ctx, n_particles=64, cache_path=None, stream=None):
     return fcas_get_info(ctx)
 
 
-def fcas_set_shape(ctx, split_bias=0, k1b=0, sub=8, radix_bits_a=4, stream=None):
+def fcas_set_shape(ctx, split_bias=0, k1b=0, sub=16, radix_bits_a=4, stream=None):
+    """Pin the launch shape; by default the FP32 and binary64 forms' own at creation."""
     s = ctypes.c_void_p(int(stream)) if stream is not None else ctypes.c_void_p(0)
     _check(load_library().fcas_set_shape(ctx.handle, int(split_bias), int(k1b), int(sub), int(radix_bits_a), s))
     return fcas_get_info(ctx)

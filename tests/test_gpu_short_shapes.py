@@ -42,3 +42,14 @@ def test_every_accepted_shape_and_the_tuned_one_evaluate(precision, n_fft, n_sam
         info = fc.fcas_autotune(ctx, 8)
         assert info["tuned_ms_per_particle"] > 0
         check(ctx, f"N={n_fft} tuned {shape(info)}")
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("w", [sd.SMALL, sd.C1], ids=["small", "64s"])
+def test_the_binding_s_default_shape_is_the_one_at_creation(w, precision):
+    import paper_2002_02150_gb300 as fc
+    with make_ctx(w, sd.make_dataset(w, 3), precision) as ctx:
+        created = fc.fcas_get_info(ctx)
+        fc.fcas_set_shape(ctx, sub=1)
+        again = fc.fcas_set_shape(ctx)
+    assert again == created
