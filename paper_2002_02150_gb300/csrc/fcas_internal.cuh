@@ -18,17 +18,20 @@ constexpr int kTwLoBits = 12;          // two-level table for e^{2 pi i m / N}: 
 // ------------------------------------------------------------------------------------------
 // Overlapped launches. The kernels of one evaluation follow each other directly on the stream; each is
 // launched so that its CTAs may be scheduled (and read what the call does not write) while the last CTAs of
-// its predecessor drain, and waits for the predecessor's completion before anything else (chain_wait; the
-// memory of all earlier kernels is visible then, since each of them waited for its own predecessor).
-// What a predecessor writes is read through plain pointers: a const __restrict__ pointer or a read-only load
-// would let the compiler move the read ahead of the wait.
-// chain_go lets the successor be scheduled once every CTA of this grid has started; it stands after chain_wait,
-// so that a grid starts with all grids but its predecessor complete (an SM's first-level cache then holds no
-// line that one of them changed later). Both do nothing in a kernel launched without the attribute or without
-// a successor that has it. The first kernel of a call is
-// launched the ordinary way. Used where a chunk covers at most 2^23 points of transform (chain_pays), where the
-// gaps between kernels count: one particle on 64 s 59.1 -> 50.8 us a call, 40 particles 51.4 -> 45, one on 60
-// min 149.0 -> 147.2; 320 particles on 64 s lose 1 % by it.
+// its predecessor drain, and waits for the predecessor's completion before anything else (chain_wait).
+//  - A wait covers the predecessor alone. chain_go therefore stands after chain_wait: it lets the successor be
+//    scheduled once every CTA of this grid has started and waited, so that a grid starts with all grids but its
+//    predecessor complete. Letting it go before the wait gave wrong results (a group of mixed forms); which read
+//    was too early was not established, and nothing here relies on it.
+//  - What a kernel of the call writes is read through plain pointers: a const __restrict__ pointer or a read-only
+//    load would let the compiler move the read ahead of the wait. The adjoint's kernels read theta and tc through
+//    such pointers: these are complete before the call's first kernel, which is launched the ordinary way.
+//  - Both do nothing in a kernel launched without the attribute or without a successor that has it.
+// Used where a chunk covers at most 2^23 points of transform (chain_pays). us per call without / with, FP32:
+// 512 particles of 2^12 points 43.1 / 39.1; 2^14: 128 42.6 / 34.9, 512 92.4 / 87.4; 2^16: 32 42.1 / 33.1, 128 90.6 /
+// 84.0; 2^21: 1 47.3 / 39.2, 4 115 / 109; one of 2^23 141.7 / 135.2. The gaps between kernels count for less the
+// more points there are; beyond the line they still do (512 particles of 2^16 331 / 304, 16 of 2^21 346 / 339, four
+// of 2^23 410 / 403), so a line further up would gain there too.
 // ------------------------------------------------------------------------------------------
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -131,7 +134,10 @@ __host__ __device__ constexpr int shape_v(int log_l) { return log_l >= 4 ? 16 : 
 // of 64 bytes; 2 columns write 32-byte pieces and lose 12 % at 2^11 points) while a CTA stays within 512
 // threads. Several small CTAs per SM are in different phases (loads, arithmetic, exchanges) at any time, one
 // large one is in the same phase throughout: us per 64 particles with 4 / 8 / 16 columns, 2^8 points 28.2 /
-// 27.4 / 29.6, 2^9 points 101 / 110 / 121, 2^10 points 778 / 827 / -. Binary64: 128 threads for the same reason
+// 27.4 / 29.6, 2^9 points 101 / 110 / 121, 2^10 points 778 / 827 / -. Sixteen columns form every bin's chirp phase,
+// two to eight step it from shared anchor bins where the particle's bound allows: the errors against 64 bits are the
+// same to within their scatter (rms of Gamma^2 over 256 to 512 particles, 4 columns against every bin's phase: 2^17
+// to 2^22 points 0.996, 0.998, 1.008, 1.007, 1.016, 1.007; 8 columns 1.000, 1.000, 1.000, 0.998, 0.998, -). Binary64: 128 threads for the same reason
 // (2^8 points, 40 particles: 8 / 16 columns 463 / 520 us; 2^11 points, 4 particles: 1 / 2 columns 6.78 / 6.92
 // ms). Float-float: 256 threads, whose warps share the instruction fetches of its long unrolled code.
 __host__ __device__ constexpr int pass_a_k1b(int log_l, int form) {
