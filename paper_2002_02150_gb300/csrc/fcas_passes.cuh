@@ -141,10 +141,10 @@ struct DetConst {
 // Pass A of the binary64 and float-float forms. The binary64 form waits for the binary64 unit alone (two
 // lanes per SM and clock), the float-float form for FP32 issue and instruction fetch: both follow the number
 // of real operations. Detector 0 needs no phasor (its delay joins the chirp phase), phasors along a thread's
-// bins and outputs come from three-term recurrences, accurate phasors from a table, the step phasors from
-// the geometry kernel: binary64 60-min pass A 9.15 -> 6.78 ms per 4 particles (with 128-thread CTAs), 64-s
-// 704 -> 463 us per 40; float-float 4.00 -> 3.63 ms per 8 particles of the 60-min workload, 15-min 2.69 ->
-// 1.86 ms per 16; errors against the oracle unchanged.
+// bins and outputs come from phasor_run, accurate phasors from a table, the step phasors from the geometry
+// kernel: binary64 60-min pass A 9.15 -> 6.30 ms per 4 particles (with 128-thread CTAs and lf_dft's butterflies),
+// 64-s 704 -> 447 us per 40; float-float 4.00 -> 3.59 ms per 8 particles of the 60-min workload, 15-min 2.69 ->
+// 2.04 ms per 16; errors against 64 bits no larger.
 template <typename Real, int LOG_L, int K1B, int MAXRB>
 __global__ void __launch_bounds__(K1B * ((1 << LOG_L) / fftr_v(LOG_L, MAXRB)), 1)
 pass_a_kernel(const cplx<Real>* __restrict__ y, const BasisD* __restrict__ basis,
