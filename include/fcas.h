@@ -327,7 +327,8 @@ typedef struct fcas_group fcas_group;
  */
 int fcas_set_shape(fcas_ctx* ctx, int32_t split_bias, int32_t k1b, int32_t sub, int32_t radix_bits_a, void* stream);
 
-/* max_batch: particles per chunk of the shared scratch (0 = automatic, <= 64). */
+/* max_batch: particles per chunk of the shared scratch (0 = automatic, <= 64; a search that larger chunks
+ * repay by themselves also holds scratch for these, within 512 MB, until it returns). */
 int fcas_group_create(fcas_group** out, int32_t n_ctx, fcas_ctx* const* ctxs, int32_t max_batch);
 
 /*

@@ -283,17 +283,17 @@ size_t inter_pp(const fcas_ctx* c) { return inter_bytes_per_particle(c->setup.pr
 int64_t base_chunk(size_t per_particle) {
     return std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)(((size_t)16 << 30) / per_particle)));
 }
-int64_t larger_chunk(const fcas_ctx* c, int64_t n, size_t scratch) {
-    return std::min<int64_t>(std::min<int64_t>(n, 2048), (int64_t)(scratch / inter_pp(c)));
+int64_t larger_chunk(size_t per_particle, int64_t n, size_t scratch) {
+    return std::min<int64_t>(std::min<int64_t>(n, 2048), (int64_t)(scratch / per_particle));
 }
 
-// Scratch for chunks of `chunk` particles in place of what *s holds; on failure *s holds nothing.
-cudaError_t alloc_scratch(const fcas_ctx* c, int64_t chunk, Scratch* s) {
+// Scratch for chunks of `chunk` particles, nb partials each, in place of what *s holds; on failure *s holds nothing.
+cudaError_t alloc_scratch(size_t per_particle, int64_t nb, int64_t chunk, Scratch* s) {
     if (s->inter) cudaFree(s->inter);
     *s = Scratch();
-    const size_t inter = inter_pp(c) * (size_t)chunk;   // (a multiple of 256: the partials are aligned)
+    const size_t inter = per_particle * (size_t)chunk;   // (a multiple of 256: the partials are aligned)
     void* p = nullptr;
-    const cudaError_t e = cudaMalloc(&p, inter + sizeof(Partial) * (size_t)chunk * c->nb_cap);
+    const cudaError_t e = cudaMalloc(&p, inter + sizeof(Partial) * (size_t)chunk * nb);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e;
@@ -307,7 +307,7 @@ cudaError_t alloc_scratch(const fcas_ctx* c, int64_t chunk, Scratch* s) {
 // Scratch of the fitness path (allocated at create unless FCAS_SETUP_LAZY_SCRATCH, else on first use).
 int ensure_scratch(fcas_ctx* c) {
     if (fitness_scratch(c).inter) return FCAS_OK;
-    const cudaError_t e = alloc_scratch(c, c->chunk, &c->scratch);
+    const cudaError_t e = alloc_scratch(inter_pp(c), c->nb_cap, c->chunk, &c->scratch);
     if (e == cudaSuccess) return FCAS_OK;
     return fail(FCAS_ERR_NOMEM, "cudaMalloc for the intermediate transform of %lld particles failed: %s",
                 (long long)c->chunk, cudaGetErrorString(e));
@@ -324,31 +324,40 @@ int ensure_batch(fcas_ctx* c, int64_t n, cudaStream_t st) {
         cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
         const bool idle = cudaStreamIsCapturing(st, &capturing) == cudaSuccess &&
                           capturing == cudaStreamCaptureStatusNone;
-        const int64_t want = larger_chunk(c, n, kBatchScratch);
+        const int64_t want = larger_chunk(inter_pp(c), n, kBatchScratch);
         if (idle && (larger || !c->batch_scratch.inter)) {
             c->batch_seen = n;
-            if (want > std::max(c->chunk, c->batch_scratch.chunk)) alloc_scratch(c, want, &c->batch_scratch);
+            if (want > std::max(c->chunk, c->batch_scratch.chunk))
+                alloc_scratch(inter_pp(c), c->nb_cap, want, &c->batch_scratch);
         }
         cudaGetLastError();
     }
     return ensure_scratch(c);
 }
 
+// What n iterations of `rows` particles lose by chunks of `have` particles instead of `want` (7 us per chunk and
+// iteration: 64 against all of 320 or 640 rows 6 to 13 us at 2^12 to 2^18 points), and what scratch for `want`
+// costs to allocate and to release (200 us, and 0.6 us per MB).
+double chunk_loss_us(int64_t rows, int64_t have, int64_t want, int64_t n) {
+    return 7.0 * (double)((rows + have - 1) / have - (rows + want - 1) / want) * (double)n;
+}
+double scratch_cost_us(size_t per_particle, int64_t want) {
+    return 200.0 + 0.6 / (1 << 20) * (double)per_particle * (double)want;
+}
+
 // Scratch of a search of n_iter iterations of `rows` particles: larger chunks than the context's once its searches
-// have lost more by smaller ones (kChunkUs per chunk and iteration: 64 against all of 320 or 640 rows 6 to 13 us a
-// chunk at 2^12 to 2^18 points) than they cost to allocate and to release (200 us, and 0.6 us per MB of them).
-// They are the searches' own: a search replaces no array that a captured call of the context points at, and
-// nothing outlives a search that points at these. Without room for them it uses the context's.
+// have lost more by smaller ones than they cost. They are the searches' own: a search replaces no array that a
+// captured call of the context points at, and nothing outlives a search that points at these. Without room for
+// them it uses the context's.
 int ensure_search(fcas_ctx* c, int64_t rows, int n_iter, Scratch* use) {
-    constexpr double kChunkUs = 7.0, kAllocUs = 200.0, kAllocUsPerByte = 0.6 / (1 << 20);
-    const int64_t want = c->setup.max_batch == 0 ? larger_chunk(c, rows, kSearchScratch) : 0;
+    const size_t pp = inter_pp(c);
+    const int64_t want = c->setup.max_batch == 0 ? larger_chunk(pp, rows, kSearchScratch) : 0;
     const int64_t have = std::max(std::max(c->chunk, fitness_scratch(c).chunk), c->search_scratch.chunk);
     if (want > have) {
-        const int64_t fewer = (rows + have - 1) / have - (rows + want - 1) / want;
-        c->search_lost_us += kChunkUs * (double)fewer * n_iter;
-        if (c->search_lost_us > kAllocUs + kAllocUsPerByte * (double)inter_pp(c) * (double)want) {
+        c->search_lost_us += chunk_loss_us(rows, have, want, n_iter);
+        if (c->search_lost_us > scratch_cost_us(pp, want)) {
             c->search_lost_us = 0.0;
-            alloc_scratch(c, want, &c->search_scratch);
+            alloc_scratch(pp, c->nb_cap, want, &c->search_scratch);
         }
     }
     int rc = FCAS_OK;
@@ -986,6 +995,9 @@ int fcas_set_shape(fcas_ctx* c, int32_t split_bias, int32_t k1b, int32_t sub, in
 struct fcas_group {
     std::vector<fcas_ctx*> ctxs;
     int64_t chunk = 0;
+    bool automatic = false;         // the caller left the chunk open
+    size_t inter_pp = 0;            // scratch per particle: intermediate bytes and argmax partials
+    int64_t nb = 0;
     void* d_inter = nullptr;
     Partial* d_partials = nullptr;
     ParticleParams* d_params = nullptr;
@@ -1015,6 +1027,9 @@ int fcas_group_create(fcas_group** out, int32_t n_ctx, fcas_ctx* const* ctxs, in
     g->ctxs.assign(ctxs, ctxs + n_ctx);
     const int64_t chunk = max_batch > 0 ? max_batch : base_chunk(inter_pp);
     g->chunk = chunk;
+    g->automatic = max_batch == 0;
+    g->inter_pp = inter_pp;
+    g->nb = nb;
     int rc = dev_alloc(&g->d_inter, inter_pp * (size_t)chunk, "group intermediate transform");
     if (!rc) rc = dev_alloc(&g->d_partials, sizeof(Partial) * (size_t)chunk * nb, "group argmax partials");
     if (!rc) {
@@ -1077,6 +1092,15 @@ int fcas_group_search_boxes(fcas_group* g, const fcas_pso_config* cfg, const dou
         ws[i] = carve_swarm(g->d_pso + per * i, rows, cfg->n_runs);
         gs[i] = pso_dev(&cfgs[i]);
     }
+    // larger chunks for this search alone, where they pay for themselves in it (without room: the group's)
+    struct Release {
+        Scratch s;
+        ~Release() { if (s.inter) cudaFree(s.inter); }
+    } larger;
+    const int64_t want = g->automatic ? larger_chunk(g->inter_pp, rows, kSearchScratch) : 0;
+    if (want > g->chunk && chunk_loss_us(rows, g->chunk, want, (int64_t)cfg->n_iter * n_ctx) > scratch_cost_us(g->inter_pp, want))
+        alloc_scratch(g->inter_pp, g->nb, want, &larger.s);
+    const Scratch scratch = larger.s.inter ? larger.s : Scratch{g->d_inter, g->d_partials, g->chunk};
     cudaStream_t st = g->st;
     cudaEvent_t ev;
     FCAS_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
@@ -1088,8 +1112,7 @@ int fcas_group_search_boxes(fcas_group* g, const fcas_pso_config* cfg, const dou
         e = run_iterations(cfg->n_iter, st, [&]() {
             cudaError_t x = cudaSuccess;
             for (int i = 0; i < n_ctx && x == cudaSuccess; ++i)
-                x = swarm_iteration(g->ctxs[i], gs[i], ws[i], g->d_params,
-                                    Scratch{g->d_inter, g->d_partials, g->chunk}, rows, st);
+                x = swarm_iteration(g->ctxs[i], gs[i], ws[i], g->d_params, scratch, rows, st);
             return x;
         });
     for (int i = 0; i < n_ctx && e == cudaSuccess; ++i) {
