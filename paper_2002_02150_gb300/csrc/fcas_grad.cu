@@ -55,8 +55,8 @@ __device__ __forceinline__ void warp_sums(Acc (&v)[kGradVals], int lane) {
 // number of particles, so neither do the sums' bits. One CTA per (particle, detector) over the whole band
 // left most SMs idle for a few particles and its twelve binary64 sums per bin held the binary64 unit: 8
 // particles of the 60-min workload 42.9 -> 1.36 ms a call, and 1.32 -> 1.02 ms with each bin's loads one bin
-// ahead; forward and backward of 40 particles on 64 s 799 -> 398 us. Bound now by FP32 issue (about 200
-// instructions per bin and detector).
+// ahead; forward and backward of 40 particles on 64 s 799 -> 398 us. Bound now by FP32 issue (248
+// instructions per bin and detector; 77 % of cycles issue).
 template <typename Real>
 __global__ void __launch_bounds__(kGradThreads, 2)
 grad_sums_kernel(const cplx<Real>* __restrict__ y, bool y_ff, const Basis<Real>* __restrict__ basis,

@@ -136,8 +136,8 @@ __host__ __device__ constexpr int shape_v(int log_l) { return log_l >= 4 ? 16 : 
 // large one is in the same phase throughout: us per 64 particles with 4 / 8 / 16 columns, 2^8 points 28.2 /
 // 27.4 / 29.6, 2^9 points 101 / 110 / 121, 2^10 points 778 / 827 / -. Sixteen columns form every bin's chirp phase,
 // two to eight step it from shared anchor bins where the particle's bound allows: the errors against 64 bits are the
-// same to within their scatter (rms of Gamma^2 over 256 to 512 particles, 4 columns against every bin's phase: 2^17
-// to 2^22 points 0.996, 0.998, 1.008, 1.007, 1.016, 1.007; 8 columns 1.000, 1.000, 1.000, 0.998, 0.998, -). Binary64: 128 threads for the same reason
+// same to within their scatter (rms of Gamma^2 over 924 to 1232 particles against every bin's phase, 2^18 / 2^19 / 2^20 /
+// 2^21 points: 4 columns 1.009 / 1.004 / 0.985 / 0.989, 8 columns 1.000 / 1.000 / 0.995 / 0.998, each +- 0.008). Binary64: 128 threads for the same reason
 // (2^8 points, 40 particles: 8 / 16 columns 463 / 520 us; 2^11 points, 4 particles: 1 / 2 columns 6.78 / 6.92
 // ms). Float-float: 256 threads, whose warps share the instruction fetches of its long unrolled code.
 __host__ __device__ constexpr int pass_a_k1b(int log_l, int form) {
