@@ -96,15 +96,21 @@ int check_device_array(const void* p, const char* fn, const char* what) {
 
 namespace {
 
+void free_scratch(Scratch* s) {
+    if (s->inter) cudaFree(s->inter);
+    if (s->partials) cudaFree(s->partials);
+    *s = Scratch();
+}
+
 void free_ctx(fcas_ctx* c) {
     void* ptrs[] = {c->d_det, c->d_sigma2s, c->d_y, c->d_basis, c->d_tw64, c->d_twlo64, c->d_twhi64,
                     c->d_tw32, c->d_twlo32, c->d_twhi32, c->d_stw_a64, c->d_stw_a32, c->d_stw_b64, c->d_stw_b32,
                     c->d_twloff, c->d_twhiff, c->d_stw_aff, c->d_stw_bff, c->d_phtab,
-                    c->d_params, c->d_theta, c->d_fit, c->d_tc, c->scratch.inter, c->batch_scratch.inter,
-                    c->search_scratch.inter, c->d_pso,
+                    c->d_params, c->d_theta, c->d_fit, c->d_tc, c->d_pso,
                     c->d_gsums, c->d_gstage, c->d_ynat, c->d_polish};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    for (Scratch* s : {&c->scratch, &c->batch_scratch, &c->search_scratch}) free_scratch(s);
     if (c->h_stage) cudaFreeHost(c->h_stage);
     if (c->search_stream) cudaStreamDestroy(c->search_stream);
     for (auto& e : c->events) {
@@ -289,17 +295,15 @@ int64_t larger_chunk(size_t per_particle, int64_t n, size_t scratch) {
 
 // Scratch for chunks of `chunk` particles, nb partials each, in place of what *s holds; on failure *s holds nothing.
 cudaError_t alloc_scratch(size_t per_particle, int64_t nb, int64_t chunk, Scratch* s) {
-    if (s->inter) cudaFree(s->inter);
-    *s = Scratch();
-    const size_t inter = per_particle * (size_t)chunk;   // (a multiple of 256: the partials are aligned)
-    void* p = nullptr;
-    const cudaError_t e = cudaMalloc(&p, inter + sizeof(Partial) * (size_t)chunk * nb);
+    free_scratch(s);
+    cudaError_t e = cudaMalloc(&s->inter, per_particle * (size_t)chunk);
+    if (e == cudaSuccess)
+        e = cudaMalloc(reinterpret_cast<void**>(&s->partials), sizeof(Partial) * (size_t)chunk * nb);
     if (e != cudaSuccess) {
         cudaGetLastError();
+        free_scratch(s);
         return e;
     }
-    s->inter = p;
-    s->partials = reinterpret_cast<Partial*>(static_cast<unsigned char*>(p) + inter);
     s->chunk = chunk;
     return cudaSuccess;
 }
@@ -1095,7 +1099,7 @@ int fcas_group_search_boxes(fcas_group* g, const fcas_pso_config* cfg, const dou
     // larger chunks for this search alone, where they pay for themselves in it (without room: the group's)
     struct Release {
         Scratch s;
-        ~Release() { if (s.inter) cudaFree(s.inter); }
+        ~Release() { free_scratch(&s); }
     } larger;
     const int64_t want = g->automatic ? larger_chunk(g->inter_pp, rows, kSearchScratch) : 0;
     if (want > g->chunk && chunk_loss_us(rows, g->chunk, want, (int64_t)cfg->n_iter * n_ctx) > scratch_cost_us(g->inter_pp, want))

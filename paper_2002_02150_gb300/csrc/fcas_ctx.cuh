@@ -21,10 +21,10 @@ inline size_t inter_bytes_per_particle(int precision, int64_t n_fft) {
     return (precision == FCAS_PREC_FP32 ? sizeof(float2) : sizeof(double2)) * (size_t)kSeries * (size_t)n_fft;
 }
 
-// Scratch of the two passes for chunks of up to `chunk` particles, in one allocation.
+// Scratch of the two passes for chunks of up to `chunk` particles.
 struct Scratch {
     void* inter = nullptr;          // [chunk][2][N2][N1] complex
-    Partial* partials = nullptr;    // [chunk][blocks per particle], after it
+    Partial* partials = nullptr;    // [chunk][blocks per particle]
     int64_t chunk = 0;
 };
 
